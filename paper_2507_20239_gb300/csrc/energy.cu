@@ -7,12 +7,11 @@
 // with weights max(0, 1 - |k - c| / s) over the input columns k inside the image,
 // normalised to sum 1; rows likewise.
 //
-// ||E(I)||_1: a 2D DFT of each channel as two 1D DFT passes -- rows (real input,
-// every row in one block, twiddles from a shared table indexed by n k mod W, the
-// index advanced incrementally) and columns (complex input, the magnitude of each
-// coefficient summed in FP64 per block and added once per block). Images are a
-// few megapixels and the schedule is computed once per scene, so direct O(N^2) DFTs
-// per row and column suffice; no FFT library is used.
+// ||E(I)||_1: a 2D DFT of each channel as two 1D DFT passes -- rows (real input) and
+// columns (complex input, the magnitudes summed in FP64 per block and added once per
+// block), each a direct sum with twiddles from a shared table indexed by n k mod N, the
+// index advanced incrementally; no FFT library is used. The direct sum keeps every
+// coefficient's FP32 rounding sequence independent of how N factors.
 #include <algorithm>
 
 #include "gs_common.cuh"
@@ -20,7 +19,6 @@
 namespace gs {
 
 constexpr int kEnergyMaxDim = 4096;
-constexpr int kEnergyThreads = 256;
 
 __device__ __forceinline__ void aa_taps(int j, int n_in, int n_out, float &c, float &s, int &k0, int &k1,
                                         float &norm) {
@@ -33,6 +31,7 @@ __device__ __forceinline__ void aa_taps(int j, int n_in, int n_out, float &c, fl
   norm = 1.f / sum;
 }
 
+// Any factor: every weight evaluated where it is used.
 __global__ void downscale_kernel(const float *__restrict__ img, int C, int H, int W, float *__restrict__ out,
                                  int Hr, int Wr) {
   const int64_t total = (int64_t)Hr * Wr;
@@ -56,74 +55,232 @@ __global__ void downscale_kernel(const float *__restrict__ img, int C, int H, in
   }
 }
 
-// tw[q] = exp(-2 pi i q / N), q in [0, N)
-__device__ __forceinline__ void fill_twiddles(float2 *tw, int N) {
-  for (int q = threadIdx.x; q < N; q += blockDim.x) {
-    double sn, cs;
-    sincospi(2.0 * (double)q / (double)N, &sn, &cs);
-    tw[q] = make_float2((float)cs, (float)-sn);
+// Factors whose filters have at most kMaxTaps taps (r <= 16: the schedule's are up to 8):
+// a block's 32 x 8 output pixels share 32 column and 8 row filters, evaluated once into
+// shared memory (one division per weight instead of one per tap, pixel and channel, which
+// is what the general kernel spends its time on). blockIdx.z is the channel. Same sums in
+// the same order, so the same bits: scales 2, 3, 4 of a 3 x 826 x 1246
+// image 73 -> 38 us.
+constexpr int kMaxTaps = 36, kDsX = 32, kDsY = 8;
+
+__global__ void __launch_bounds__(kDsX *kDsY) downscale_taps_kernel(const float *__restrict__ img, int H, int W,
+                                                                    float *__restrict__ out, int Hr, int Wr) {
+  __shared__ float s_wx[kMaxTaps][kDsX], s_wy[kMaxTaps][kDsY];
+  __shared__ float s_nx[kDsX], s_ny[kDsY];
+  __shared__ int s_x0[kDsX], s_x1[kDsX], s_y0[kDsY], s_y1[kDsY];
+  const int t = threadIdx.y * kDsX + threadIdx.x;
+  if (t < kDsX + kDsY) {
+    const bool col = t < kDsX;
+    const int i = col ? t : t - kDsX;
+    const int j = (col ? blockIdx.x * kDsX : blockIdx.y * kDsY) + i;
+    float c = 0.f, sc = 1.f, norm = 0.f;
+    int k0 = 0, k1 = -1;
+    if (j < (col ? Wr : Hr)) aa_taps(j, col ? W : H, col ? Wr : Hr, c, sc, k0, k1, norm);
+    for (int k = k0; k <= k1; ++k) {
+      const float w = fmaxf(0.f, 1.f - fabsf((float)k - c) / sc);
+      if (col) s_wx[k - k0][i] = w; else s_wy[k - k0][i] = w;
+    }
+    if (col) {
+      s_x0[i] = k0; s_x1[i] = k1; s_nx[i] = norm;
+    } else {
+      s_y0[i] = k0; s_y1[i] = k1; s_ny[i] = norm;
+    }
   }
+  __syncthreads();
+  const int x = blockIdx.x * kDsX + threadIdx.x, y = blockIdx.y * kDsY + threadIdx.y;
+  if (x >= Wr || y >= Hr) return;
+  const int x0 = s_x0[threadIdx.x], x1 = s_x1[threadIdx.x], y0 = s_y0[threadIdx.y], y1 = s_y1[threadIdx.y];
+  const float *src = img + (int64_t)blockIdx.z * H * W;
+  float acc = 0.f;
+  for (int ky = y0; ky <= y1; ++ky) {
+    const float *line = src + (int64_t)ky * W + x0;
+    float row = 0.f;
+    for (int k = 0; k <= x1 - x0; ++k) row = fmaf(s_wx[k][threadIdx.x], line[k], row);
+    acc = fmaf(s_wy[ky - y0][threadIdx.y], row, acc);
+  }
+  out[(int64_t)blockIdx.z * Hr * Wr + (int64_t)y * Wr + x] = acc * s_nx[threadIdx.x] * s_ny[threadIdx.y];
 }
 
-// One block per (channel, row): X[ch][h][k] = sum_n I[ch][h][n] exp(-2 pi i n k / W).
-__global__ void __launch_bounds__(kEnergyThreads) dft_rows_kernel(const float *__restrict__ img, int W,
-                                                                  float2 *__restrict__ X) {
-  extern __shared__ float4 s_raw[];
-  float2 *tw = reinterpret_cast<float2 *>(s_raw);
-  float *row = reinterpret_cast<float *>(tw + W);
-  const int64_t base = (int64_t)blockIdx.x * W;
-  fill_twiddles(tw, W);
-  for (int n = threadIdx.x; n < W; n += blockDim.x) row[n] = img[base + n];
-  __syncthreads();
-  for (int k = threadIdx.x; k < W; k += blockDim.x) {
-    float re = 0.f, im = 0.f;
-    int q = 0;
-    for (int n = 0; n < W; ++n) {
-      const float2 t = tw[q];
-      re = fmaf(row[n], t.x, re);
-      im = fmaf(row[n], t.y, im);
-      q += k;
-      if (q >= W) q -= W;
-    }
-    X[base + k] = make_float2(re, im);
-  }
+// tw[q] = exp(-2 pi i q / N), q in [0, N), of the rows (N = W) and of the columns (N = H),
+// computed once per call: the double-precision sines, done by every block of a DFT pass,
+// cost more than the pass (FP64 runs at 1/64 of the FP32 rate here).
+__global__ void twiddles_kernel(float2 *__restrict__ tw_w, int W, float2 *__restrict__ tw_h, int H) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= W + H) return;
+  const int N = i < W ? W : H, q = i < W ? i : i - W;
+  double sn, cs;
+  sincospi(2.0 * (double)q / (double)N, &sn, &cs);
+  (i < W ? tw_w : tw_h)[q] = make_float2((float)cs, (float)-sn);
 }
 
-// One block per (channel, column k): Y[m] = sum_h X[h][k] exp(-2 pi i h m / H);
-// the block adds sum_m |Y[m]| to *sum.
-__global__ void __launch_bounds__(kEnergyThreads) dft_cols_l1_kernel(const float2 *__restrict__ X, int H, int W,
-                                                                     double *sum) {
+// Twiddle q sits at slot q + q / 16 of the shared table: lanes of consecutive k read
+// q = n k mod N at stride n, which without the padding puts 2 to 16 lanes on one bank
+// for every even n.
+__device__ __forceinline__ int tw_slot(int q) { return q + (q >> 4); }
+static int tw_slots(int N) { return N + (N >> 4) + 1; }
+
+__device__ __forceinline__ void load_twiddles(float2 *s_tw, const float2 *__restrict__ tw, int N) {
+  for (int q = threadIdx.x; q < N; q += blockDim.x) s_tw[tw_slot(q)] = tw[q];
+}
+
+// Both passes are a direct O(N^2) sum per coefficient, in the order n = 0, 1, ..., on the
+// FP32 pipes. A thread keeps kDftRows lines (rows, or columns) of kDftK frequencies in
+// registers, so a twiddle serves kDftRows lines and a line's value kDftK frequencies.
+// With one line and one frequency per thread the passes ran at the rate of their
+// shared-memory loads (a conflicted twiddle per two FMAs).
+// The input is real, so X[h][W - k] = conj X[h][k] and column W - k has the magnitudes of
+// column k: only k = 0 .. W / 2 are computed, the others counted with weight 2.
+// 3 x 826 x 1246: row pass ~1770 -> 234 us, column pass ~1390 -> 251 us (82% of issue
+// slots; 229 us of FMAs in the two at the FP32 peak); same bits up to the FP64 sum's order.
+constexpr int kDftThreads = 64;
+constexpr int kDftK = 2;                        // frequencies per thread
+constexpr int kDftRows = 16;                    // rows per thread (row pass)
+constexpr int kDftCols = 8;                     // columns per thread (column pass)
+constexpr int kDftChunk = 64;                   // line positions staged at a time
+constexpr int kDftPad = kDftRows + 4;           // staged row position: 16-byte aligned, 4-way at most when filled
+
+// X[line][k] = sum_n I[line][n] exp(-2 pi i n k / W), line = channel * H + row.
+__global__ void __launch_bounds__(kDftThreads, 8) dft_rows_kernel(const float *__restrict__ img, int64_t lines, int W,
+                                                               int K, const float2 *__restrict__ tw,
+                                                               float2 *__restrict__ X) {
   extern __shared__ float4 s_raw[];
-  float2 *tw = reinterpret_cast<float2 *>(s_raw);
-  float2 *col = tw + H;
-  __shared__ double s_part[kEnergyThreads / 32];
-  const int ch = blockIdx.x / W, k = blockIdx.x - ch * W;
-  const float2 *src = X + (int64_t)ch * H * W + k;
-  fill_twiddles(tw, H);
-  for (int h = threadIdx.x; h < H; h += blockDim.x) col[h] = src[(int64_t)h * W];
-  __syncthreads();
-  double part = 0.0;
-  for (int m = threadIdx.x; m < H; m += blockDim.x) {
-    float re = 0.f, im = 0.f;
-    int q = 0;
-    for (int h = 0; h < H; ++h) {
-      const float2 t = tw[q], x = col[h];
-      re = fmaf(x.x, t.x, fmaf(-x.y, t.y, re));
-      im = fmaf(x.x, t.y, fmaf(x.y, t.x, im));
-      q += m;
-      if (q >= H) q -= H;
+  float *s_x = reinterpret_cast<float *>(s_raw);                               // [kDftChunk][kDftPad]
+  float2 *s_tw = reinterpret_cast<float2 *>(s_x + kDftChunk * kDftPad);
+  const int64_t l0 = (int64_t)blockIdx.x * kDftRows;
+  load_twiddles(s_tw, tw, W);
+  int k[kDftK], q[kDftK];
+  float re[kDftK][kDftRows], im[kDftK][kDftRows];
+#pragma unroll
+  for (int j = 0; j < kDftK; ++j) {
+    const int kk = (blockIdx.y * kDftK + j) * kDftThreads + threadIdx.x;
+    k[j] = kk < K ? kk : 0;
+    q[j] = 0;
+#pragma unroll
+    for (int r = 0; r < kDftRows; ++r) re[j][r] = im[j][r] = 0.f;
+  }
+  for (int n0 = 0; n0 < W; n0 += kDftChunk) {
+    const int cnt = min(kDftChunk, W - n0);
+    __syncthreads();
+    for (int i = threadIdx.x; i < kDftChunk * kDftRows; i += kDftThreads) {
+      const int r = i / kDftChunk, n = i - r * kDftChunk;
+      s_x[n * kDftPad + r] = n < cnt && l0 + r < lines ? img[(l0 + r) * W + n0 + n] : 0.f;
     }
-    part += sqrt((double)re * re + (double)im * im);
+    __syncthreads();
+#pragma unroll 2
+    for (int n = 0; n < cnt; ++n) {
+      float x[kDftRows];
+#pragma unroll
+      for (int r = 0; r < kDftRows; r += 4) {
+        const float4 v = *reinterpret_cast<const float4 *>(s_x + n * kDftPad + r);
+        x[r] = v.x; x[r + 1] = v.y; x[r + 2] = v.z; x[r + 3] = v.w;
+      }
+#pragma unroll
+      for (int j = 0; j < kDftK; ++j) {
+        const float2 t = s_tw[tw_slot(q[j])];
+#pragma unroll
+        for (int r = 0; r < kDftRows; ++r) {
+          re[j][r] = fmaf(x[r], t.x, re[j][r]);
+          im[j][r] = fmaf(x[r], t.y, im[j][r]);
+        }
+        q[j] += k[j];
+        q[j] = (int)min((uint32_t)q[j], (uint32_t)(q[j] - W));   // q mod W (q < 2 W)
+      }
+    }
   }
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
-  if ((threadIdx.x & 31) == 0) s_part[threadIdx.x >> 5] = part;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double b = 0.0;
-    for (int w = 0; w < kEnergyThreads / 32; ++w) b += s_part[w];
-    atomicAdd(sum, b);
+  for (int j = 0; j < kDftK; ++j) {
+    const int kk = (blockIdx.y * kDftK + j) * kDftThreads + threadIdx.x;
+    if (kk >= K) continue;
+#pragma unroll
+    for (int r = 0; r < kDftRows; ++r)
+      if (l0 + r < lines) X[(l0 + r) * K + kk] = make_float2(re[j][r], im[j][r]);
   }
+}
+
+// (s, c) += weight |z|, |z| to about 2^-46 in FP32 pairs (the FP64 square root ran for
+// longer than the DFT): z's squares as hi + lo exactly but for lo's last bits, m ~ sqrt(hi)
+// and its correction (hi + lo - m^2) / (2 m). Outside the range where no term of that under-
+// or overflows, the FP64 root, into `wide`. weight: 1 or 2.
+__device__ __forceinline__ void add_magnitude(float re, float im, float weight, float &s, float &c, double &wide) {
+  const float a = fmaxf(fabsf(re), fabsf(im)), b = fminf(fabsf(re), fabsf(im));
+  if (!(a >= 1e-12f && fabsf(re) <= 1e15f && fabsf(im) <= 1e15f)) {
+    if (re != 0.f || im != 0.f) wide += (double)weight * sqrt((double)re * re + (double)im * im);
+    return;
+  }
+  const float a2 = a * a, b2 = b * b;
+  const float hi = a2 + b2;
+  const float lo = (b2 - (hi - a2)) + (fmaf(a, a, -a2) + fmaf(b, b, -b2));
+  const float m = sqrtf(hi);
+  const float e = (fmaf(-m, m, hi) + lo) * (0.5f / m);
+  pair_add(s, c, weight * m);
+  c += weight * e;
+}
+
+// Y[m] = sum_h X[h][k] exp(-2 pi i h m / H) of kDftCols adjacent columns k (of the K kept)
+// of one channel; adds sum |Y[m]| to *sum, columns that stand for W - k too twice.
+__global__ void __launch_bounds__(kDftThreads, 10) dft_cols_l1_kernel(const float2 *__restrict__ X, int H, int W, int K,
+                                                                  const float2 *__restrict__ tw, double *sum) {
+  extern __shared__ float4 s_raw[];
+  float2 *s_x = reinterpret_cast<float2 *>(s_raw);                            // [kDftChunk][kDftCols]
+  float2 *s_tw = s_x + kDftChunk * kDftCols;
+  const int col_blocks = (K + kDftCols - 1) / kDftCols;
+  const int ch = blockIdx.x / col_blocks, c0 = (blockIdx.x - ch * col_blocks) * kDftCols;
+  const float2 *src = X + (int64_t)ch * H * K;
+  load_twiddles(s_tw, tw, H);
+  int m[kDftK], q[kDftK];
+  float re[kDftK][kDftCols], im[kDftK][kDftCols];
+#pragma unroll
+  for (int j = 0; j < kDftK; ++j) {
+    const int mm = (blockIdx.y * kDftK + j) * kDftThreads + threadIdx.x;
+    m[j] = mm < H ? mm : 0;
+    q[j] = 0;
+#pragma unroll
+    for (int c = 0; c < kDftCols; ++c) re[j][c] = im[j][c] = 0.f;
+  }
+  for (int h0 = 0; h0 < H; h0 += kDftChunk) {
+    const int cnt = min(kDftChunk, H - h0);
+    __syncthreads();
+    for (int i = threadIdx.x; i < kDftChunk * kDftCols; i += kDftThreads) {
+      const int h = i / kDftCols, c = i - h * kDftCols;
+      s_x[i] = h < cnt && c0 + c < K ? src[(int64_t)(h0 + h) * K + c0 + c] : make_float2(0.f, 0.f);
+    }
+    __syncthreads();
+#pragma unroll 2
+    for (int h = 0; h < cnt; ++h) {
+      float2 x[kDftCols];
+#pragma unroll
+      for (int c = 0; c < kDftCols; c += 2) {
+        const float4 v = *reinterpret_cast<const float4 *>(s_x + h * kDftCols + c);
+        x[c] = make_float2(v.x, v.y);
+        x[c + 1] = make_float2(v.z, v.w);
+      }
+#pragma unroll
+      for (int j = 0; j < kDftK; ++j) {
+        const float2 t = s_tw[tw_slot(q[j])];
+#pragma unroll
+        for (int c = 0; c < kDftCols; ++c) {
+          re[j][c] = fmaf(x[c].x, t.x, fmaf(-x[c].y, t.y, re[j][c]));
+          im[j][c] = fmaf(x[c].x, t.y, fmaf(x[c].y, t.x, im[j][c]));
+        }
+        q[j] += m[j];
+        q[j] = (int)min((uint32_t)q[j], (uint32_t)(q[j] - H));
+      }
+    }
+  }
+  float part = 0.f, part_c = 0.f;
+  double wide = 0.0;
+#pragma unroll
+  for (int j = 0; j < kDftK; ++j) {
+    if ((blockIdx.y * kDftK + j) * kDftThreads + threadIdx.x >= H) continue;
+#pragma unroll
+    for (int c = 0; c < kDftCols; ++c) {
+      const int k = c0 + c;
+      if (k < K) add_magnitude(re[j][c], im[j][c], k == 0 || 2 * k == W ? 1.f : 2.f, part, part_c, wide);
+    }
+  }
+  if (wide != 0.0) atomicAdd(sum, wide);
+  warp_pair_sum(part, part_c);
+  if ((threadIdx.x & 31) == 0) atomicAdd(sum, (double)part + (double)part_c);
 }
 
 static bool dims_ok(int C, int H, int W) {
@@ -144,16 +301,24 @@ extern "C" gs_status_t gs_downscale(const float *image, int32_t C, int32_t H, in
                                     gs_stream_t stream) {
   if (!image || !out || C <= 0 || H <= 0 || W <= 0 || r < 1) return GS_ERR_INVALID_ARG;
   const int Hr = gs_downscaled_size(H, r), Wr = gs_downscaled_size(W, r);
-  const int64_t total = (int64_t)Hr * Wr;
-  const int grid = (int)std::min<int64_t>((total + 255) / 256, (int64_t)num_sms() * 16);
-  downscale_kernel<<<grid, 256, 0, as_stream(stream)>>>(image, C, H, W, out, Hr, Wr);
+  // taps per axis: at most 2 s + 1 with s = W / Wr <= 1.5 r (Wr rounds W / r down to half)
+  const int64_t taps = 2 * (int64_t)std::max((W + Wr - 1) / Wr, (H + Hr - 1) / Hr) + 1;
+  const dim3 blocks((Wr + kDsX - 1) / kDsX, (Hr + kDsY - 1) / kDsY, C);
+  if (taps <= kMaxTaps && blocks.y <= 65535 && blocks.z <= 65535) {
+    downscale_taps_kernel<<<blocks, dim3(kDsX, kDsY), 0, as_stream(stream)>>>(image, H, W, out, Hr, Wr);
+  } else {
+    const int64_t total = (int64_t)Hr * Wr;
+    const int grid = (int)std::min<int64_t>((total + 255) / 256, (int64_t)num_sms() * 16);
+    downscale_kernel<<<grid, 256, 0, as_stream(stream)>>>(image, C, H, W, out, Hr, Wr);
+  }
   GS_LAUNCH_CHECK();
   return GS_OK;
 }
 
 extern "C" size_t gs_spectrum_workspace_size(int32_t C, int32_t H, int32_t W) {
   if (!dims_ok(C, H, W)) return 0;
-  return sizeof(float2) * (size_t)C * H * W;
+  // the kept coefficients of the row pass, then both passes' twiddles
+  return sizeof(float2) * ((size_t)C * H * (W / 2 + 1) + W + H);
 }
 
 extern "C" gs_status_t gs_spectrum_l1(const float *image, int32_t C, int32_t H, int32_t W, double *d_sum, void *ws,
@@ -162,15 +327,26 @@ extern "C" gs_status_t gs_spectrum_l1(const float *image, int32_t C, int32_t H, 
   if (ws_bytes < gs_spectrum_workspace_size(C, H, W) || (reinterpret_cast<uintptr_t>(ws) & 15u) != 0)
     return GS_ERR_INVALID_ARG;
   cudaStream_t s = as_stream(stream);
+  const int K = W / 2 + 1;
+  const int64_t lines = (int64_t)C * H;
+  const int64_t row_blocks = (lines + kDftRows - 1) / kDftRows;
+  const int64_t col_blocks = (int64_t)C * ((K + kDftCols - 1) / kDftCols);
+  if (row_blocks > 0x7fffffffll || col_blocks > 0x7fffffffll) return GS_ERR_INVALID_ARG;
   float2 *X = static_cast<float2 *>(ws);
-  const size_t smem_rows = (size_t)W * (sizeof(float2) + sizeof(float));
-  const size_t smem_cols = (size_t)H * 2 * sizeof(float2);
-  GS_CUDA_TRY(cudaFuncSetAttribute(dft_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_rows));
-  GS_CUDA_TRY(cudaFuncSetAttribute(dft_cols_l1_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_cols));
+  float2 *tw_w = X + lines * K, *tw_h = tw_w + W;
+  const size_t smem_rows = sizeof(float) * kDftChunk * kDftPad + sizeof(float2) * tw_slots(W);
+  const size_t smem_cols = sizeof(float2) * kDftChunk * kDftCols + sizeof(float2) * tw_slots(H);
+  static_assert(sizeof(float2) * (kDftChunk * kDftCols + kEnergyMaxDim + kEnergyMaxDim / 16 + 1) <= 48 * 1024,
+                "fits the default shared-memory limit");
   GS_CUDA_TRY(cudaMemsetAsync(d_sum, 0, sizeof(double), s));
-  dft_rows_kernel<<<C * H, kEnergyThreads, smem_rows, s>>>(image, W, X);
+  twiddles_kernel<<<(W + H + 127) / 128, 128, 0, s>>>(tw_w, W, tw_h, H);
   GS_LAUNCH_CHECK();
-  dft_cols_l1_kernel<<<C * W, kEnergyThreads, smem_cols, s>>>(X, H, W, d_sum);
+  constexpr int kPer = kDftThreads * kDftK;
+  dft_rows_kernel<<<dim3((unsigned)row_blocks, (K + kPer - 1) / kPer), kDftThreads, smem_rows, s>>>(image, lines, W, K,
+                                                                                                tw_w, X);
+  GS_LAUNCH_CHECK();
+  dft_cols_l1_kernel<<<dim3((unsigned)col_blocks, (H + kPer - 1) / kPer), kDftThreads, smem_cols, s>>>(
+      X, H, W, K, tw_h, d_sum);
   GS_LAUNCH_CHECK();
   return GS_OK;
 }

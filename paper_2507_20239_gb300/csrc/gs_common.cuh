@@ -172,6 +172,23 @@ __device__ __forceinline__ Falloff2 falloff2(float u, float v, float a2, float b
   return f;
 }
 
+// FP32 pair sums, for reductions whose result is wanted in more than FP32: s + c carries
+// about 48 bits. The FP64 pipe runs at 1/64 of the FP32 rate on this chip, so that a block's
+// reductions in FP64 shuffles can take longer than its work.
+__device__ __forceinline__ void pair_add(float &s, float &c, float x) {
+  const float t = __fadd_rn(s, x), bb = __fsub_rn(t, s);
+  c = __fadd_rn(c, __fadd_rn(__fsub_rn(s, __fsub_rn(t, bb)), __fsub_rn(x, bb)));
+  s = t;
+}
+// The sum of the pairs of 2 * first lanes (a power of two), in every one of them.
+__device__ __forceinline__ void warp_pair_sum(float &s, float &c, int first = 16) {
+  for (int o = first; o > 0; o >>= 1) {
+    const float so = __shfl_xor_sync(0xffffffffu, s, o), co = __shfl_xor_sync(0xffffffffu, c, o);
+    c = __fadd_rn(c, co);
+    pair_add(s, c, so);
+  }
+}
+
 // The binning's ellipse-box test, in two steps with one IEEE FP32 rounding per
 // operation (no contraction), so that the decision is reproducible op for op:
 // band_consts_rn once per record, band_span_rn once per row of tiles (the x-extent of

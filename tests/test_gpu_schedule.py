@@ -34,6 +34,29 @@ def test_spectrum_l1_matches_oracle(shape):
     assert abs(got - want) <= 1e-5 * want
 
 
+@pytest.mark.parametrize("shape", [(1, 2, 2), (5, 3, 3), (1, 63, 64), (1, 65, 127), (2, 128, 130), (3, 129, 14),
+                                   (17, 16, 257)])
+def test_spectrum_l1_at_tile_edges(shape):
+    """Line, frequency and column counts around the DFT passes' tiles (16 rows, 8 columns,
+    64-position chunks, 128 frequencies), odd and even widths (the folded half spectrum).
+    A coefficient's FP32 error (at most N roundings of partial sums below 0.8 N) has no
+    preferred sign, so the sum of the magnitudes holds 1e-5."""
+    img = _image(3, *shape)
+    got = S.spectrum_l1(torch.as_tensor(img).cuda())
+    want = osch.spectrum_l1(img)
+    assert abs(got - want) <= 1e-5 * want
+
+
+@pytest.mark.parametrize("shape,r", [((3, 207, 311), 16), ((2, 207, 311), 17), ((1, 207, 311), 40), ((2, 5, 33), 2),
+                                     ((1, 9, 64), 2), ((1, 40, 3), 8)])
+def test_downscale_filter_widths(shape, r):
+    """The tabulated filters up to 36 taps and the general kernel beyond, ragged output tiles."""
+    img = _image(4, *shape)
+    got = S.downscale(torch.as_tensor(img).cuda(), r).cpu().numpy()
+    want = osch.downscale(img, r)
+    assert got.shape == want.shape and np.abs(got - want).max() < 1e-5
+
+
 def test_energy_schedule_matches_oracle():
     imgs = [_image(s, 3, 413, 623) for s in (2, 3)]
     E, T, st = S.energy_schedule(imgs, K=8, T_densify=25000)
