@@ -9,8 +9,9 @@
 // ((mu_x^2 + mu_y^2 + C1)(Sxx - mu_x^2 + Syy - mu_y^2 + C2)). Its gradient w.r.t. the
 // rendered image x is the window's adjoint (the same symmetric window, zero
 // padded) applied to d map / d mu_x, d map / d Sxx and d map / d Sxy, combined as
-// W*(d/dmu) + 2 x W*(d/dSxx) + y W*(d/dSxy). Four separable passes per view, every
-// view of the frame in one launch each; the sums for the loss are FP64.
+// W*(d/dmu) + 2 x W*(d/dSxx) + y W*(d/dSxy). Two kernels, every view of the frame in
+// one launch each: the window sums and the map's derivatives, then their adjoint and the
+// gradient; the sums for the loss are carried in FP32 pairs per thread and FP64 across.
 #include <cmath>
 
 #include "gs_common.cuh"
@@ -19,178 +20,345 @@ namespace gs {
 
 constexpr int kWin = 11, kHalf = 5;
 constexpr float kSsimC1 = 0.01f * 0.01f, kSsimC2 = 0.03f * 0.03f;
-constexpr int kPlanes = 8;   // scratch planes per pixel value
+constexpr int kPlanes = 3;   // scratch planes per pixel value: the map's derivatives
 
 struct float5_t {
   float v[5];
 };
 
-__device__ __forceinline__ void window(float *w) {
-  if (threadIdx.x < kWin && threadIdx.y == 0) {
+// Both kernels take tiles of 64 x 22 output values. The inputs with their halo of 5 go to
+// shared memory once; a thread then forms four adjacent horizontal window sums (14
+// values read for 44 taps) into shared memory, and up to six vertical ones of a column
+// (16 values for 66 taps) from there. Bound by FP32 issue: about 170 instructions a value
+// in the first kernel, 100 in the second, pairs of moments packed (f32x2: the same
+// operations and roundings at half the issue slots). One thread per value with every tap
+// read from global memory, in four passes over eight planes, was bound by those
+// loads: 3 x 826 x 1246 84 + 46 + 44 + 40 us and a finishing launch -> 37 + 27 us, the
+// same bits. Walking down a strip with the last 11 rows' sums in registers came to 44 + 31
+// us (128 registers: too few warps to cover the loads).
+// 22 rows: 32 rows with the halo x 16 groups of four = two rounds of 256 threads.
+constexpr int kTx = 64, kTy = 22, kSsimThreads = 256;
+constexpr int kTileRows = kTy + 2 * kHalf, kTileCols = kTx + 2 * kHalf + 2;   // whole 16-byte pairs
+constexpr int kColRows = (kTy + kSsimThreads / kTx - 1) / (kSsimThreads / kTx);   // output rows per thread
+static_assert((kTileRows * kTx / 4) % kSsimThreads == 0, "whole rounds of horizontal tasks");
+
+// Interleaved pairs are read and written four at a time, 32 bytes apart from thread to
+// thread; swapping neighbouring 16-byte chunks in every other run of eight keeps those
+// accesses off each other's banks. pair_at: the slot of column c of a row.
+__device__ __forceinline__ int chunk_at(int chunk) { return chunk ^ ((chunk >> 3) & 1); }
+__device__ __forceinline__ int pair_at(int c) { return chunk_at(c >> 1) * 2 + (c & 1); }
+
+struct SsimTile {
+  float2 in2[kTileRows][kTileCols + 4];   // two input planes, interleaved (rows of whole 16-chunk swaps)
+  float2 h1[kTileRows][kTx];              // horizontal sums
+  float2 h2[kTileRows][kTx];
+  float h3[kTileRows][kTx];
+};
+struct GradTile {
+  float2 in2[kTileRows][kTileCols + 4];
+  float in1[kTileRows][kTileCols];    // the third plane
+  float2 h1[kTileRows][kTx];
+  float h3[kTileRows][kTx];
+};
+static_assert(kTileCols % 4 == 0, "16-byte aligned rows");
+
+// The window's weights exp(-d^2 / (2 1.5^2)), d = -5 .. 5, for the block (a barrier follows).
+__device__ __forceinline__ void put_window(float *w) {
+  if (threadIdx.x < kWin) {
     const float d = (float)((int)threadIdx.x - kHalf);
     w[threadIdx.x] = expf(-d * d / (2.f * 1.5f * 1.5f));
   }
-  __syncthreads();
-  if (threadIdx.x == 0 && threadIdx.y == 0) {
-    float s = 0.f;
-    for (int i = 0; i < kWin; ++i) s += w[i];
-    w[kWin] = 1.f / s;
-  }
-  __syncthreads();
+}
+// The first six as pairs (the window is symmetric), and the inverse of the sum of all.
+__device__ __forceinline__ float get_window(const float *w, float2 wr[kHalf + 1]) {
+  float s = 0.f;
+#pragma unroll
+  for (int k = 0; k < kWin; ++k) s += w[k];
+#pragma unroll
+  for (int k = 0; k <= kHalf; ++k) wr[k] = f2(w[k]);
+  return 1.f / s;
 }
 
-struct ViewPlane {
-  int W, H;
-  int64_t base;   // offset of this (view, channel) plane in the planar batch layout
-  bool ok;
+struct Tile {
+  int W, H, x0, y0;   // the view's size, the tile's first column and row
+  int64_t base;       // offset of this (view, channel) plane in the planar batch layout
+  bool on;
 };
 
-__device__ __forceinline__ ViewPlane view_plane(const gs_camera_t *cams) {
-  ViewPlane p;
+__device__ __forceinline__ Tile tile_of(const gs_camera_t *cams) {
+  Tile p;
   const int v = blockIdx.z / 3, c = blockIdx.z - 3 * v;
   const gs_camera_t &cam = cams[v];
   p.W = cam.width;
   p.H = cam.height;
   p.base = 3 * cam.pixel_offset + (int64_t)c * p.W * p.H;
-  const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y * blockDim.y + threadIdx.y;
-  p.ok = x < p.W && y < p.H;
+  p.x0 = blockIdx.x * kTx;
+  p.y0 = blockIdx.y * kTy;
+  p.on = p.x0 < p.W && p.y0 < p.H;
   return p;
 }
 
-// pass 1: horizontal window sums of x, y, x^2, y^2, x y (planes 0..4); L1 sum.
-__global__ void ssim_h1_kernel(const gs_camera_t *__restrict__ cams, const float *__restrict__ img,
-                               const float *__restrict__ tgt, float *__restrict__ ws, int64_t stride,
-                               double *__restrict__ l1) {
-  __shared__ float w[kWin + 1];
-  __shared__ float s_red[8];
-  window(w);
-  const ViewPlane p = view_plane(cams);
-  const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y * blockDim.y + threadIdx.y;
-  float ad = 0.f;
-  if (p.ok) {
-    float a[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
-    const int64_t row = p.base + (int64_t)y * p.W;
-    for (int k = -kHalf; k <= kHalf; ++k) {
-      const int xx = x + k;
-      if (xx < 0 || xx >= p.W) continue;
-      const float wk = w[k + kHalf], xi = img[row + xx], yi = tgt[row + xx];
-      a[0] = fmaf(wk, xi, a[0]);
-      a[1] = fmaf(wk, yi, a[1]);
-      a[2] = fmaf(wk, xi * xi, a[2]);
-      a[3] = fmaf(wk, yi * yi, a[3]);
-      a[4] = fmaf(wk, xi * yi, a[4]);
-    }
-    const float n = w[kWin];
-    for (int q = 0; q < 5; ++q) ws[q * stride + row + x] = a[q] * n;
-    ad = fabsf(img[row + x] - tgt[row + x]);
-  }
-  // block sum of |x - y| (16 x 16 threads)
-  const int t = threadIdx.y * blockDim.x + threadIdx.x;
+// The tile's inputs and their halo, zero outside the view: planes a and b interleaved and,
+// with C, plane c.
+template <bool C, typename T>
+__device__ __forceinline__ void load_tile(const Tile &p, T &s, const float *__restrict__ a, const float *__restrict__ b,
+                                          const float *__restrict__ c, float *s_c) {
+  // a warp takes every eighth row, its lanes the columns lane, lane + 32, lane + 64
+  constexpr int kWarps = kSsimThreads / 32, kCols = (kTileCols + 31) / 32;
+  const int lane = threadIdx.x & 31;
+  const int x = p.x0 - kHalf + lane;
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) ad += __shfl_xor_sync(0xffffffffu, ad, o);
-  if ((t & 31) == 0) s_red[t >> 5] = ad;
-  __syncthreads();
-  if (t == 0) {
-    double s = 0.0;
-    for (int i = 0; i < (int)(blockDim.x * blockDim.y) / 32; ++i) s += s_red[i];
-    atomicAdd(l1 + blockIdx.z / 3, s);
-  }
-}
-
-// pass 2: vertical window sums -> SSIM map (summed) and its partial derivatives
-// w.r.t. mu_x, Sxx, Sxy (planes 5..7).
-__global__ void ssim_v1_kernel(const gs_camera_t *__restrict__ cams, float *__restrict__ ws, int64_t stride,
-                               double *__restrict__ ssim_sum) {
-  __shared__ float w[kWin + 1];
-  __shared__ double s_dred[8];
-  window(w);
-  const ViewPlane p = view_plane(cams);
-  const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y * blockDim.y + threadIdx.y;
-  float mapv = 0.f;
-  if (p.ok) {
-    float a[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
-    for (int k = -kHalf; k <= kHalf; ++k) {
-      const int yy = y + k;
-      if (yy < 0 || yy >= p.H) continue;
-      const float wk = w[k + kHalf];
-      const int64_t i = p.base + (int64_t)yy * p.W + x;
-      for (int q = 0; q < 5; ++q) a[q] = fmaf(wk, ws[q * stride + i], a[q]);
-    }
-    const float n = w[kWin];
-    const float mx = a[0] * n, my = a[1] * n, sxx = a[2] * n, syy = a[3] * n, sxy = a[4] * n;
-    const float A1 = 2.f * mx * my + kSsimC1, A2 = 2.f * (sxy - mx * my) + kSsimC2;
-    const float B1 = mx * mx + my * my + kSsimC1, B2 = (sxx - mx * mx) + (syy - my * my) + kSsimC2;
-    const float inv = 1.f / (B1 * B2);
-    mapv = A1 * A2 * inv;
-    const int64_t i = p.base + (int64_t)y * p.W + x;
-    ws[5 * stride + i] = (2.f * my * (A2 - A1)) * inv - mapv * (2.f * mx * (B2 - B1)) * inv;   // d map / d mu_x
-    ws[6 * stride + i] = -mapv / B2;                                                         // d map / d Sxx
-    ws[7 * stride + i] = 2.f * A1 * inv;                                                     // d map / d Sxy
-  }
-  const int t = threadIdx.y * blockDim.x + threadIdx.x;
-  double m = mapv;
+  for (int r = threadIdx.x >> 5; r < kTileRows; r += kWarps) {
+    const int y = p.y0 - kHalf + r;
+    const bool row = (unsigned)y < (unsigned)p.H;
+    const int64_t o = p.base + (int64_t)y * p.W + x;
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) m += __shfl_xor_sync(0xffffffffu, m, o);
-  if ((t & 31) == 0) s_dred[t >> 5] = m;
+    for (int q = 0; q < kCols; ++q) {
+      const int col = lane + 32 * q;
+      if (col >= kTileCols) break;
+      float2 v = make_float2(0.f, 0.f);
+      float u = 0.f;
+      if (row && (unsigned)(x + 32 * q) < (unsigned)p.W) {
+        v = make_float2(a[o + 32 * q], b[o + 32 * q]);
+        if (C) u = c[o + 32 * q];
+      }
+      s.in2[r][pair_at(col)] = v;
+      if (C) s_c[r * kTileCols + col] = u;
+    }
+  }
+}
+
+// The 14 interleaved values from column 4 g of row r.
+__device__ __forceinline__ void read14(const float2 *row, int g, float2 v[14]) {
+#pragma unroll
+  for (int q = 0; q < 7; ++q) {
+    const float4 f = *reinterpret_cast<const float4 *>(row + chunk_at(2 * g + q) * 2);
+    v[2 * q] = make_float2(f.x, f.y);
+    v[2 * q + 1] = make_float2(f.z, f.w);
+  }
+}
+
+__device__ __forceinline__ void write4(float2 *row, int g, const float2 v[4]) {
+  *reinterpret_cast<float4 *>(row + chunk_at(2 * g) * 2) = make_float4(v[0].x, v[0].y, v[1].x, v[1].y);
+  *reinterpret_cast<float4 *>(row + chunk_at(2 * g + 1) * 2) = make_float4(v[2].x, v[2].y, v[3].x, v[3].y);
+}
+
+// Window sums of x, y, x^2, y^2, x y -> SSIM map (summed per view) and its partial
+// derivatives w.r.t. mu_x, Sxx, Sxy (planes 0..2); L1 sum.
+__global__ void __launch_bounds__(kSsimThreads, 3) ssim_map_kernel(
+    const gs_camera_t *__restrict__ cams, const float *__restrict__ img, const float *__restrict__ tgt,
+    float *__restrict__ ws, int64_t stride, double *l1, double *ssim_sum) {
+  extern __shared__ float4 s_raw[];
+  SsimTile &s = *reinterpret_cast<SsimTile *>(s_raw);
+  __shared__ float w[kWin];
+  __shared__ float4 s_red[kSsimThreads / 32];
+  const Tile p = tile_of(cams);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  float ad = 0.f, ad_c = 0.f, ms = 0.f, ms_c = 0.f;
+  if (p.on) {
+    put_window(w);
+    load_tile<false>(p, s, img, tgt, nullptr, nullptr);
+    __syncthreads();
+    float2 wr[kHalf + 1];
+    const float n = get_window(w, wr);
+    for (int t = threadIdx.x; t < kTileRows * kTx / 4; t += kSsimThreads) {
+      const int r = t / (kTx / 4), g = t - r * (kTx / 4);
+      float2 v[14];
+      read14(s.in2[r], g, v);
+      float2 a1[4], a2[4];
+      float a3[4];
+#pragma unroll
+      for (int o = 0; o < 4; ++o) {
+        a1[o] = a2[o] = f2(0.f);
+        a3[o] = 0.f;
+      }
+#pragma unroll
+      for (int c = 0; c < 14; ++c) {   // taps in ascending column order
+        const float2 vv = f2_mul(v[c], v[c]);
+        const float xy = __fmul_rn(v[c].x, v[c].y);
+#pragma unroll
+        for (int o = 0; o < 4; ++o) {
+          const int k = c - o;
+          if (k < 0 || k >= kWin) continue;
+          const float2 wk = wr[k <= kHalf ? k : kWin - 1 - k];
+          a1[o] = f2_fma(wk, v[c], a1[o]);
+          a2[o] = f2_fma(wk, vv, a2[o]);
+          a3[o] = fmaf(wk.x, xy, a3[o]);
+        }
+      }
+#pragma unroll
+      for (int o = 0; o < 4; ++o) {
+        a1[o] = f2_mul(a1[o], f2(n));
+        a2[o] = f2_mul(a2[o], f2(n));
+        a3[o] *= n;
+      }
+      write4(s.h1[r], g, a1);
+      write4(s.h2[r], g, a2);
+      *reinterpret_cast<float4 *>(&s.h3[r][4 * g]) = make_float4(a3[0], a3[1], a3[2], a3[3]);
+    }
+    __syncthreads();
+    const int c = threadIdx.x % kTx, r0 = (threadIdx.x / kTx) * kColRows;
+    const int rows = min(kColRows, min(kTy, p.H - p.y0) - r0);
+    if (p.x0 + c < p.W && rows > 0) {
+      float2 b1[kColRows], b2[kColRows];
+      float b3[kColRows];
+#pragma unroll
+      for (int o = 0; o < kColRows; ++o) {
+        b1[o] = b2[o] = f2(0.f);
+        b3[o] = 0.f;
+      }
+#pragma unroll
+      for (int i = 0; i < kColRows + 2 * kHalf; ++i) {   // taps in ascending row order
+        if (r0 + i >= kTileRows) break;                  // past the tile: rows not kept
+        const float2 h1 = s.h1[r0 + i][pair_at(c)], h2 = s.h2[r0 + i][pair_at(c)];
+        const float h3 = s.h3[r0 + i][c];
+#pragma unroll
+        for (int o = 0; o < kColRows; ++o) {
+          const int k = i - o;
+          if (k < 0 || k >= kWin) continue;
+          const float2 wk = wr[k <= kHalf ? k : kWin - 1 - k];
+          b1[o] = f2_fma(wk, h1, b1[o]);
+          b2[o] = f2_fma(wk, h2, b2[o]);
+          b3[o] = fmaf(wk.x, h3, b3[o]);
+        }
+      }
+#pragma unroll
+      for (int o = 0; o < kColRows; ++o) {
+        if (o >= rows) break;
+        const float mx = b1[o].x * n, my = b1[o].y * n, sxx = b2[o].x * n, syy = b2[o].y * n, sxy = b3[o] * n;
+        const float A1 = 2.f * mx * my + kSsimC1, A2 = 2.f * (sxy - mx * my) + kSsimC2;
+        const float B1 = mx * mx + my * my + kSsimC1, B2 = (sxx - mx * mx) + (syy - my * my) + kSsimC2;
+        const float inv = 1.f / (B1 * B2);
+        const float mapv = A1 * A2 * inv;
+        const int64_t i = p.base + (int64_t)(p.y0 + r0 + o) * p.W + p.x0 + c;
+        ws[i] = (2.f * my * (A2 - A1)) * inv - mapv * (2.f * mx * (B2 - B1)) * inv;   // d map / d mu_x
+        ws[stride + i] = -mapv / B2;                                                  // d map / d Sxx
+        ws[2 * stride + i] = 2.f * A1 * inv;                                          // d map / d Sxy
+        pair_add(ms, ms_c, mapv);
+        const float2 v = s.in2[r0 + o + kHalf][pair_at(c + kHalf)];
+        pair_add(ad, ad_c, fabsf(v.x - v.y));
+      }
+    }
+  }
+  warp_pair_sum(ad, ad_c);
+  warp_pair_sum(ms, ms_c);
+  if (lane == 0) s_red[warp] = make_float4(ad, ad_c, ms, ms_c);
   __syncthreads();
-  if (t == 0) {
-    double s = 0.0;
-    for (int i = 0; i < (int)(blockDim.x * blockDim.y) / 32; ++i) s += s_dred[i];
-    atomicAdd(ssim_sum + blockIdx.z / 3, s);
+  if (warp == 0) {
+    const float4 q = s_red[lane % (kSsimThreads / 32)];
+    ad = q.x; ad_c = q.y; ms = q.z; ms_c = q.w;
+    warp_pair_sum(ad, ad_c, kSsimThreads / 64);
+    warp_pair_sum(ms, ms_c, kSsimThreads / 64);
+  }
+  if (threadIdx.x == 0) {
+    const double da = (double)ad + (double)ad_c, dm = (double)ms + (double)ms_c;
+    atomicAdd(l1 + blockIdx.z / 3, da);
+    atomicAdd(ssim_sum + blockIdx.z / 3, dm);
   }
 }
 
-// pass 3: horizontal adjoint window over planes 5..7 -> planes 0..2.
-__global__ void ssim_h2_kernel(const gs_camera_t *__restrict__ cams, float *__restrict__ ws, int64_t stride) {
-  __shared__ float w[kWin + 1];
-  window(w);
-  const ViewPlane p = view_plane(cams);
-  if (!p.ok) return;
-  const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y * blockDim.y + threadIdx.y;
-  const int64_t row = p.base + (int64_t)y * p.W;
-  float a[3] = {0.f, 0.f, 0.f};
-  for (int k = -kHalf; k <= kHalf; ++k) {
-    const int xx = x + k;
-    if (xx < 0 || xx >= p.W) continue;
-    const float wk = w[k + kHalf];
-    for (int q = 0; q < 3; ++q) a[q] = fmaf(wk, ws[(5 + q) * stride + row + xx], a[q]);
+// Adjoint window sums of the derivative planes -> d loss / d image; the views' losses from
+// the sums.
+__global__ void __launch_bounds__(kSsimThreads, 3) ssim_grad_kernel(const gs_camera_t *__restrict__ cams,
+                                                                    const float *__restrict__ img,
+                                                                    const float *__restrict__ tgt,
+                                                                    const float *__restrict__ ws, int64_t stride,
+                                                                    float lambda, const double *__restrict__ l1,
+                                                                    const double *__restrict__ ssim_sum,
+                                                                    float *__restrict__ loss,
+                                                                    float *__restrict__ d_image) {
+  extern __shared__ float4 s_raw[];
+  GradTile &s = *reinterpret_cast<GradTile *>(s_raw);
+  __shared__ float w[kWin];
+  const Tile p = tile_of(cams);
+  if (!p.on) return;
+  if (blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z % 3 == 0 && threadIdx.x == 0) {
+    const int v = blockIdx.z / 3;
+    const double cnt = 3.0 * p.W * (double)p.H;
+    loss[v] = (float)((1.0 - lambda) * l1[v] / cnt + lambda * (1.0 - ssim_sum[v] / cnt));
   }
-  for (int q = 0; q < 3; ++q) ws[q * stride + row + x] = a[q] * w[kWin];
-}
-
-// pass 4: vertical adjoint window -> d loss / d image.
-__global__ void ssim_v2_kernel(const gs_camera_t *__restrict__ cams, const float *__restrict__ img,
-                               const float *__restrict__ tgt, const float *__restrict__ ws, int64_t stride,
-                               float lambda, float *__restrict__ d_image) {
-  __shared__ float w[kWin + 1];
-  window(w);
-  const ViewPlane p = view_plane(cams);
-  if (!p.ok) return;
-  const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y * blockDim.y + threadIdx.y;
-  float a[3] = {0.f, 0.f, 0.f};
-  for (int k = -kHalf; k <= kHalf; ++k) {
-    const int yy = y + k;
-    if (yy < 0 || yy >= p.H) continue;
-    const float wk = w[k + kHalf];
-    const int64_t i = p.base + (int64_t)yy * p.W + x;
-    for (int q = 0; q < 3; ++q) a[q] = fmaf(wk, ws[q * stride + i], a[q]);
+  put_window(w);
+  load_tile<true>(p, s, ws, ws + stride, ws + 2 * stride, &s.in1[0][0]);
+  __syncthreads();
+  float2 wr[kHalf + 1];
+  const float n = get_window(w, wr);
+  for (int t = threadIdx.x; t < kTileRows * kTx / 4; t += kSsimThreads) {
+    const int r = t / (kTx / 4), g = t - r * (kTx / 4);
+    float2 v[14];
+    read14(s.in2[r], g, v);
+    float u[16];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const float4 f = *reinterpret_cast<const float4 *>(&s.in1[r][4 * (g + q)]);
+      u[4 * q] = f.x; u[4 * q + 1] = f.y; u[4 * q + 2] = f.z; u[4 * q + 3] = f.w;
+    }
+    float2 a1[4];
+    float a3[4];
+#pragma unroll
+    for (int o = 0; o < 4; ++o) {
+      a1[o] = f2(0.f);
+      a3[o] = 0.f;
+    }
+#pragma unroll
+    for (int c = 0; c < 14; ++c)
+#pragma unroll
+      for (int o = 0; o < 4; ++o) {
+        const int k = c - o;
+        if (k < 0 || k >= kWin) continue;
+        const float2 wk = wr[k <= kHalf ? k : kWin - 1 - k];
+        a1[o] = f2_fma(wk, v[c], a1[o]);
+        a3[o] = fmaf(wk.x, u[c], a3[o]);
+      }
+#pragma unroll
+    for (int o = 0; o < 4; ++o) {
+      a1[o] = f2_mul(a1[o], f2(n));
+      a3[o] *= n;
+    }
+    write4(s.h1[r], g, a1);
+    *reinterpret_cast<float4 *>(&s.h3[r][4 * g]) = make_float4(a3[0], a3[1], a3[2], a3[3]);
   }
-  const float n = w[kWin];
-  const int64_t i = p.base + (int64_t)y * p.W + x;
-  const float xi = img[i], yi = tgt[i], d = xi - yi;
+  __syncthreads();
+  const int c = threadIdx.x % kTx, r0 = (threadIdx.x / kTx) * kColRows;
+  const int rows = min(kColRows, min(kTy, p.H - p.y0) - r0);
+  if (p.x0 + c >= p.W || rows <= 0) return;
+  const int64_t i0 = p.base + (int64_t)(p.y0 + r0) * p.W + p.x0 + c;
+  float xs[kColRows], ys[kColRows];
+#pragma unroll
+  for (int o = 0; o < kColRows; ++o)
+    if (o < rows) {
+      xs[o] = img[i0 + (int64_t)o * p.W];
+      ys[o] = tgt[i0 + (int64_t)o * p.W];
+    }
+  float2 b1[kColRows];
+  float b3[kColRows];
+#pragma unroll
+  for (int o = 0; o < kColRows; ++o) {
+    b1[o] = f2(0.f);
+    b3[o] = 0.f;
+  }
+#pragma unroll
+  for (int i = 0; i < kColRows + 2 * kHalf; ++i) {
+    if (r0 + i >= kTileRows) break;
+    const float2 h1 = s.h1[r0 + i][pair_at(c)];
+    const float h3 = s.h3[r0 + i][c];
+#pragma unroll
+    for (int o = 0; o < kColRows; ++o) {
+      const int k = i - o;
+      if (k < 0 || k >= kWin) continue;
+      const float2 wk = wr[k <= kHalf ? k : kWin - 1 - k];
+      b1[o] = f2_fma(wk, h1, b1[o]);
+      b3[o] = fmaf(wk.x, h3, b3[o]);
+    }
+  }
   const float inv_n = 1.f / (3.f * (float)p.W * (float)p.H);
-  const float g_ssim = (a[0] * n + 2.f * xi * (a[1] * n) + yi * (a[2] * n)) * inv_n;
-  const float g_l1 = d > 0.f ? inv_n : (d < 0.f ? -inv_n : 0.f);
-  d_image[i] = (1.f - lambda) * g_l1 - lambda * g_ssim;
-}
-
-__global__ void photometric_finalize_kernel(const gs_camera_t *__restrict__ cams, int n_views, float lambda,
-                                            const double *__restrict__ l1, const double *__restrict__ ssim,
-                                            float *__restrict__ loss) {
-  const int v = blockIdx.x * blockDim.x + threadIdx.x;
-  if (v >= n_views) return;
-  const double n = 3.0 * cams[v].width * (double)cams[v].height;
-  loss[v] = (float)((1.0 - lambda) * l1[v] / n + lambda * (1.0 - ssim[v] / n));
+#pragma unroll
+  for (int o = 0; o < kColRows; ++o) {
+    if (o >= rows) break;
+    const float xi = xs[o], yi = ys[o], d = xi - yi;
+    const float g_ssim = (b1[o].x * n + 2.f * xi * (b1[o].y * n) + yi * (b3[o] * n)) * inv_n;
+    const float g_l1 = d > 0.f ? inv_n : (d < 0.f ? -inv_n : 0.f);
+    d_image[i0 + (int64_t)o * p.W] = (1.f - lambda) * g_l1 - lambda * g_ssim;
+  }
 }
 
 // ------------------------------------------------------------------ optimiser
@@ -284,22 +452,18 @@ extern "C" gs_status_t gs_photometric_loss_grad(const gs_frame_t *frame, const f
     return GS_ERR_INVALID_ARG;
   cudaStream_t s = as_stream(stream);
   const int64_t stride = 3 * frame->n_pixels;
-  float *planes = static_cast<float *>(ws);
-  double *l1 = reinterpret_cast<double *>(planes + kPlanes * stride);
-  double *ssim = l1 + frame->n_views;
+  // the FP64 sums first: the planes may hold an odd number of floats
+  double *l1 = static_cast<double *>(ws), *ssim = l1 + frame->n_views;
+  float *planes = reinterpret_cast<float *>(ssim + frame->n_views);
   GS_CUDA_TRY(cudaMemsetAsync(l1, 0, 2 * sizeof(double) * frame->n_views, s));
-  const dim3 block(16, 16);
-  const dim3 grid((frame->max_width + 15) / 16, (frame->max_height + 15) / 16, 3 * frame->n_views);
-  ssim_h1_kernel<<<grid, block, 0, s>>>(frame->cams_dev, image, target, planes, stride, l1);
+  const dim3 grid((frame->max_width + kTx - 1) / kTx, (frame->max_height + kTy - 1) / kTy, 3 * frame->n_views);
+  GS_CUDA_TRY(cudaFuncSetAttribute(ssim_map_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SsimTile)));
+  GS_CUDA_TRY(cudaFuncSetAttribute(ssim_grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(GradTile)));
+  ssim_map_kernel<<<grid, kSsimThreads, sizeof(SsimTile), s>>>(frame->cams_dev, image, target, planes, stride, l1,
+                                                               ssim);
   GS_LAUNCH_CHECK();
-  ssim_v1_kernel<<<grid, block, 0, s>>>(frame->cams_dev, planes, stride, ssim);
-  GS_LAUNCH_CHECK();
-  ssim_h2_kernel<<<grid, block, 0, s>>>(frame->cams_dev, planes, stride);
-  GS_LAUNCH_CHECK();
-  ssim_v2_kernel<<<grid, block, 0, s>>>(frame->cams_dev, image, target, planes, stride, lambda, d_image);
-  GS_LAUNCH_CHECK();
-  photometric_finalize_kernel<<<(frame->n_views + 127) / 128, 128, 0, s>>>(frame->cams_dev, frame->n_views, lambda,
-                                                                           l1, ssim, loss_dev);
+  ssim_grad_kernel<<<grid, kSsimThreads, sizeof(GradTile), s>>>(frame->cams_dev, image, target, planes, stride, lambda,
+                                                                l1, ssim, loss_dev, d_image);
   GS_LAUNCH_CHECK();
   return GS_OK;
 }
