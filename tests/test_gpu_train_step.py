@@ -38,6 +38,13 @@ def test_photometric_loss_and_gradient_match_oracle(sizes):
         assert rel_l2(got, want_g) < 1e-4
 
 
+@pytest.mark.parametrize("sizes", [[(64, 22)], [(65, 23), (63, 21)], [(128, 44), (1, 1), (11, 200)], [(129, 16), (5, 45)]])
+def test_photometric_loss_at_tile_edges(sizes):
+    """Views around the 64 x 22 tiles' edges, smaller than the window, of different sizes in
+    one frame; tolerances as above."""
+    test_photometric_loss_and_gradient_match_oracle(sizes)
+
+
 def test_photometric_loss_of_identical_images_is_zero():
     frame = R.Frame([_cam(40, 30)])
     img = frame.pack_images([np.random.default_rng(3).uniform(size=(3, 30, 40)).astype(np.float32)])
