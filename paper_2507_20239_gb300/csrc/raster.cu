@@ -167,9 +167,9 @@ __device__ __forceinline__ int warp_select(const float4 *s_rgb, int cnt, int war
 
 // Forward without CTA-wide steps: each warp walks its tile's list on its own, 32
 // entries at a time. Lane l gathers entry base + l, tests it against the warp's
-// 8x8 block (the ellipse's x-extent over the block's rows against its columns) and
-// stages it in the warp's shared slots if it passes; the warp then composites the
-// passing entries in list order. A warp leaves as soon as its 64 pixels have
+// 8x8 block (the ellipse's x-extent over the block's rows against its columns); the
+// passing entries are closed up in the warp's shared slots and composited in list
+// order, two per turn of the loop. A warp leaves as soon as its 64 pixels have
 // stopped, so neither barriers nor finished neighbours hold it (one-warp CTAs,
 // which also free a finished warp's slot, measured no faster).
 struct FwdArgs {
@@ -188,6 +188,8 @@ struct FwdArgs {
   uint64_t n_records, list_cap;   // bounds of the record ids and list positions (debug checks)
 };
 
+constexpr int kFwdSlots = 32;   // a full step of 32 is even: no filler needed beyond it
+
 // One warp's 8 x 8 block `warp` of `tile`, with the warp's staging slots.
 template <int TW, int TH, bool CKPT>
 __device__ __forceinline__ void fwd_warp_block(const FwdArgs &a, int tile, int warp, int lane, float2 *sxy,
@@ -199,6 +201,7 @@ __device__ __forceinline__ void fwd_warp_block(const FwdArgs &a, int tile, int w
   const uint32_t *__restrict__ vals = a.vals;
   const CkptLayout &ckpt = a.ckpt;
   const TileCoord tc = tile_coord(a.cams, a.n_views, tile);
+  const uint32_t lt = (1u << lane) - 1u;
   int lx, ly;
   pixel_of<TW>(warp * 32 + lane, lx, ly);
   const int py = tc.ty * TH + ly;
@@ -270,23 +273,26 @@ __device__ __forceinline__ void fwd_warp_block(const FwdArgs &a, int tile, int w
       const EllipseRows e = ellipse_rows(xy.x, xy.y, co.x, co.y, co.z, c.w * kBinMargin);
       float xl, xr;
       sel = row_span(e, Y0, Y1, xl, xr) && X1 >= xl && X0 <= xr;
-      if (sel) {
-        sxy[lane] = xy;
-        sco[lane] = make_float4(__fmul_rn(co.x, kNegHalfLog2e), co.y, __fmul_rn(co.z, kNegHalfLog2e), co.w);
-        srgb[lane] = c;
-      }
     }
-    uint32_t b = __ballot_sync(0xffffffffu, sel);
+    // the passing entries, closed up in order; the colour's fourth word carries the list
+    // position. An odd count is filled with an entry of opacity 0.
+    const uint32_t b = __ballot_sync(0xffffffffu, sel);
+    const int cnt = __popc(b);
+    if (sel) {
+      const int at = __popc(b & lt);
+      sxy[at] = xy;
+      sco[at] = make_float4(__fmul_rn(co.x, kNegHalfLog2e), co.y, __fmul_rn(co.z, kNegHalfLog2e), co.w);
+      srgb[at] = make_float4(c.x, c.y, c.z, __uint_as_float((uint32_t)j + 1u));
+    }
+    if ((cnt & 1) && lane == 0) {
+      sxy[cnt] = make_float2(0.f, 0.f);
+      sco[cnt] = srgb[cnt] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
     __syncwarp();
-    // both pixels in packed pairs, without branches: an entry a pixel skips (done,
-    // below the floor, or the one that would cross the cut-off) gets weight 0 and
-    // leaves T, the colour and the stop index as they are
-    while (b) {
-      const int i = __ffs(b) - 1;
-      b &= b - 1u;
+    // one entry's sigma at both pixels
+    auto alpha = [&](int i) -> float2 {
       const float2 xy = sxy[i];
       const float4 co = sco[i];
-      float2 al;
       if (CKPT) {
         // the falloff in scalar form (its operands are the entry's, broadcast to both
         // pixels, so packing them costs register moves); the two pixels share dy and
@@ -297,10 +303,14 @@ __device__ __forceinline__ void fwd_warp_block(const FwdArgs &a, int tile, int w
         const float gdd = __fmul_rn(co.z, __fmul_rn(dy, dy));
         const float t0 = __fmaf_rn(co.y, dy, dx0), t1 = __fmaf_rn(co.y, dy, dx1);
         const float e0 = __fmaf_rn(__fmul_rn(co.x, t0), t0, gdd), e1 = __fmaf_rn(__fmul_rn(co.x, t1), t1, gdd);
-        al = f2(fminf(kAlphaMax, __fmul_rn(co.w, ex2_approx(e0))), fminf(kAlphaMax, __fmul_rn(co.w, ex2_approx(e1))));
-      } else {
-        al = falloff2(xy.x, xy.y, co.x, co.y, co.z, co.w, fx, fy).alpha;
+        return f2(fminf(kAlphaMax, __fmul_rn(co.w, ex2_approx(e0))), fminf(kAlphaMax, __fmul_rn(co.w, ex2_approx(e1))));
       }
+      return falloff2(xy.x, xy.y, co.x, co.y, co.z, co.w, fx, fy).alpha;
+    };
+    // both pixels in packed pairs, without branches: an entry a pixel skips (done,
+    // below the floor, or the one that would cross the cut-off) gets weight 0 and
+    // leaves T, the colour and the stop index as they are
+    auto composite = [&](const float2 al, const float4 c) {
       const bool a0 = !done0 && al.x >= kAlphaMin, a1 = !done1 && al.y >= kAlphaMin;
       // transmittance and weight: genuinely per-pixel pairs, packed
       const float2 Tn = f2_mul(T, f2_sub(ONE, al));
@@ -308,7 +318,6 @@ __device__ __forceinline__ void fwd_warp_block(const FwdArgs &a, int tile, int w
       done0 = done0 || (a0 && !c0);
       done1 = done1 || (a1 && !c1);
       const float2 w = f2_mul(f2(c0 ? al.x : 0.f, c1 ? al.y : 0.f), T);
-      const float4 c = srgb[i];
       if (CKPT) {
         cr = f2(fmaf(c.x, w.x, cr.x), fmaf(c.x, w.y, cr.y));
         cg = f2(fmaf(c.y, w.x, cg.x), fmaf(c.y, w.y, cg.y));
@@ -319,8 +328,18 @@ __device__ __forceinline__ void fwd_warp_block(const FwdArgs &a, int tile, int w
         cb = f2_fma(f2(c.z), w, cb);
       }
       T = f2(c0 ? Tn.x : T.x, c1 ? Tn.y : T.y);
-      st0 = c0 ? base + i + 1 : st0;
-      st1 = c1 ? base + i + 1 : st1;
+      const uint32_t pos = __float_as_uint(c.w);
+      st0 = c0 ? pos : st0;
+      st1 = c1 ? pos : st1;
+    };
+    // two entries at a time: their sigmas do not depend on each other, and a warp that
+    // waits for one entry's sigma after another (about 120 cycles each) is what a frame
+    // of few tiles takes its time from: 38 -> 26 us at 16 tiles, 82 -> 53 at 260, 76 -> 60
+    // at 1014, 155 -> 121 at 2542, and 313 -> 292 with checkpoints at 4056
+    for (int i = 0; i < cnt; i += 2) {
+      const float2 al_a = alpha(i), al_b = alpha(i + 1);
+      composite(al_a, srgb[i]);
+      composite(al_b, srgb[i + 1]);
     }
     __syncwarp();
   }
@@ -349,9 +368,9 @@ __device__ __forceinline__ void fwd_warp_block(const FwdArgs &a, int tile, int w
 template <int TW, int TH, bool CKPT>
 __global__ void __launch_bounds__(TW *TH / 2) raster_fwd_warp_kernel(const FwdArgs a) {
   constexpr int NW = TW * TH / 64;
-  __shared__ float2 s_xy[NW][32];
-  __shared__ float4 s_co[NW][32];
-  __shared__ float4 s_rgb[NW][32];
+  __shared__ float2 s_xy[NW][kFwdSlots];
+  __shared__ float4 s_co[NW][kFwdSlots];
+  __shared__ float4 s_rgb[NW][kFwdSlots];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   fwd_warp_block<TW, TH, CKPT>(a, blockIdx.x, warp, lane, s_xy[warp], s_co[warp], s_rgb[warp]);
 }
@@ -366,9 +385,9 @@ template <int TW, int TH, bool CKPT>
 __global__ void __launch_bounds__(32 * kQueueWarps) raster_fwd_queue_kernel(const FwdArgs a, int n_tiles,
                                                                            uint32_t *queue) {
   constexpr int NW = TW * TH / 64;
-  __shared__ float2 s_xy[kQueueWarps][32];
-  __shared__ float4 s_co[kQueueWarps][32];
-  __shared__ float4 s_rgb[kQueueWarps][32];
+  __shared__ float2 s_xy[kQueueWarps][kFwdSlots];
+  __shared__ float4 s_co[kQueueWarps][kFwdSlots];
+  __shared__ float4 s_rgb[kQueueWarps][kFwdSlots];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t units = (uint32_t)n_tiles * NW;
   for (;;) {
