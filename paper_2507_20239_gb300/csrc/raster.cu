@@ -8,7 +8,7 @@
 // have stopped. Optionally it stores each pixel's stop index and, for the per-splat
 // backward, a checkpoint (T, composited colour) every 64 list entries.
 //
-// Both backward kernels re-walk the lists front to back with exactly the forward's
+// The backward kernels re-walk the lists front to back with exactly the forward's
 // FP32 decisions and need, per pixel, only <dL/dout, out>:
 //   dL/dsigma_i = T_i <c_i, g> - (<out, g> - sum_{j<=i} <c_j, g> sigma_j T_j) / (1 - sigma_i).
 // Per (pixel, Gaussian) they accumulate six moments of the falloff gradient and
@@ -16,9 +16,10 @@
 // raster_bwd_kernel is parallel over pixels: the terms are summed over a thread's
 // two pixels in registers, across the warp with a transposing shuffle reduction and
 // across the CTA's warps in shared memory, then added with vector reductions.
-// raster_bwd_splat_kernel is parallel over list entries (one lane per entry, the
+// raster_bwd_splat_kernel is parallel over list entries (two per lane, the
 // pixels flowing through the warp from the forward's checkpoints), so each lane
-// sums its own entry's terms and no reduction is needed.
+// sums its own entries' terms and no reduction is needed. raster_bwd_tile_kernel does the same
+// from checkpoints that it makes itself in shared memory, window by window of the list.
 #include "gs_common.cuh"
 
 namespace gs {
@@ -709,7 +710,7 @@ __global__ void __launch_bounds__(TW *TH / PX) raster_bwd_kernel(
 
 // Per-splat backward (the per-splat parallel back-propagation of the Taming-3DGS
 // lineage that the paper's base trainer uses): the same gradient as
-// raster_bwd_kernel, parallel over list entries instead of pixels. The warps of a
+// raster_bwd_tile_kernel, parallel over list entries instead of pixels. The warps of a
 // tile's CTAs claim its 64-entry buckets (up to the tile's largest stop index) one
 // at a time, two consecutive entries per lane. A bucket's live pixels (stop index
 // beyond its first position) start from the forward's checkpoint (T and the colour
@@ -736,6 +737,129 @@ __device__ __forceinline__ float rcp_approx(float x) {
   float y;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
+}
+
+// One warp's walk of a 64-entry bucket: lane l holds entries 64 b + 2 l and + 1, and the
+// bucket's live pixels flow through the warp diagonally, pixel s - l at lane l in step s.
+struct SplatEntries {
+  float2 U, V, A2, BE, G2, O, NCX, NCY, NCZ;   // .x entry a, .y entry b
+  uint32_t ja, jb;                             // list positions
+  // xy, (k A, beta, k gamma, o) and colour of the two entries
+  __device__ __forceinline__ void set(int j, float2 xya, float2 xyb, float4 coa, float4 cob, float4 ca, float4 cb) {
+    U = f2(xya.x, xyb.x);
+    V = f2(xya.y, xyb.y);
+    A2 = f2(coa.x, cob.x);
+    BE = f2(coa.y, cob.y);
+    G2 = f2(coa.z, cob.z);
+    O = f2(coa.w, cob.w);
+    NCX = f2(-ca.x, -cb.x);
+    NCY = f2(-ca.y, -cb.y);
+    NCZ = f2(-ca.z, -cb.z);
+    ja = (uint32_t)j;
+    jb = (uint32_t)j + 1u;
+  }
+};
+
+// The two entries' sums: six moments of the falloff gradient, accumulated negated, and
+// the colour terms as they are.
+struct SplatMoments {
+  float2 v[9];
+  // Entry h's sums once into its record's gradients.
+  __device__ __forceinline__ void flush(int h, uint32_t r, const float4 *__restrict__ conic_o, float *g_mean2d,
+                                        float *g_co, float *g_rgb) const {
+    float m[9];
+    bool any = false;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+      const float x = h == 0 ? v[k].x : v[k].y;
+      m[k] = k < 6 ? -x : x;
+      any = any || x != 0.f;
+    }
+    if (!any) return;
+    const float4 cu = conic_o[r];
+    const float oA = cu.w * cu.x, ho = -0.5f * cu.w;
+    red_add_v2(g_mean2d + 2 * (size_t)r, -oA * m[0], -(oA * cu.y * m[0] + cu.w * cu.z * m[1]));
+    red_add_v4(g_co + 4 * (size_t)r, ho * m[2], -oA * m[3], ho * m[4], m[5]);
+    red_add_v4(g_rgb + 4 * (size_t)r, m[6], m[7], m[8], 0.f);
+  }
+};
+
+// nl live pixels; ring: this warp's 2 x kSplatRing slots; fill(s0, A, B) gives live pixel
+// s0 + lane: A = (dL/dout, stop bits), B = (x, y, T, R) before the bucket, or (0, 0, 0, 0) and
+// (0, 0, 1, 0) past the list.
+template <typename Fill>
+__device__ __forceinline__ void splat_walk(const SplatEntries &e, int nl, float4 *ring, int lane, SplatMoments &out,
+                                           Fill &&fill) {
+  float4 *ra = ring, *rb = ring + kSplatRing;
+  // slots 32..63 read as stopped until the second chunk replaces them
+  ra[32 + lane] = make_float4(0.f, 0.f, 0.f, 0.f);
+  rb[32 + lane] = make_float4(0.f, 0.f, 1.f, 0.f);
+  float2 v0 = f2(0.f), v1 = f2(0.f), v2 = f2(0.f), v3 = f2(0.f), v4 = f2(0.f), v5 = f2(0.f);
+  float2 v6 = f2(0.f), v7 = f2(0.f), v8 = f2(0.f);
+  float T = 1.f, Rr = 0.f;
+  for (int s0 = 0; s0 < nl + 31; s0 += 32) {
+    {
+      float4 A, B;
+      fill(s0, A, B);
+      ra[(s0 + lane) & (kSplatRing - 1)] = A;
+      rb[(s0 + lane) & (kSplatRing - 1)] = B;
+      __syncwarp();
+    }
+    const int s1 = min(s0 + 32, nl + 31);
+#pragma unroll 8
+    for (int s = s0; s < s1; ++s) {
+      const float4 *q = ra + ((s - lane) & (kSplatRing - 1));
+      const float Tin = __shfl_up_sync(0xffffffffu, T, 1);
+      const float Rin = __shfl_up_sync(0xffffffffu, Rr, 1);
+      const float4 g = q[0], p = q[kSplatRing];
+      T = lane == 0 ? p.z : Tin;
+      Rr = lane == 0 ? p.w : Rin;
+      // falloff of both entries at this pixel: the forward's operations and roundings
+      // (the pixel's coordinates are a broadcast operand: two scalar subtractions
+      // cost less than a packed one and the moves that would build its pair)
+      const float2 dx = f2(__fsub_rn(e.U.x, p.x), __fsub_rn(e.U.y, p.x));
+      const float2 dy = f2(__fsub_rn(e.V.x, p.y), __fsub_rn(e.V.y, p.y));
+      const float2 tt = f2_fma(e.BE, dy, dx);
+      const float2 ex = f2_fma(f2_mul(e.A2, tt), tt, f2_mul(e.G2, f2_mul(dy, dy)));
+      const float2 G = f2(ex2_approx(ex.x), ex2_approx(ex.y));
+      const float2 raw = f2_mul(e.O, G);
+      const float2 al = f2(fminf(kAlphaMax, raw.x), fminf(kAlphaMax, raw.y));
+      // a position before the pixel's stop (false on stopped pixels and for lanes
+      // without an entry) where sigma reaches the floor; elsewhere sigma 0 leaves T,
+      // R and every sum as they are
+      const uint32_t stop = __float_as_uint(g.w);
+      const bool oka = e.ja < stop && al.x >= kAlphaMin, okb = e.jb < stop && al.y >= kAlphaMin;
+      const float2 ncd = f2_fma(e.NCZ, f2(g.z), f2_fma(e.NCY, f2(g.y), f2_mul(e.NCX, f2(g.x))));   // -<c, g>
+      // entry a, then entry b, in list order: -dL/dsigma = -T <c, g> + R / (1 - sigma)
+      const float sa = oka ? al.x : 0.f;
+      const float oma = __fsub_rn(1.f, sa);
+      const float wa = sa * T;
+      Rr = fmaf(ncd.x, wa, Rr);
+      const float nda = fmaf(T, ncd.x, Rr * rcp_approx(oma));
+      T = __fmul_rn(T, oma);
+      const float sb = okb ? al.y : 0.f;
+      const float omb = __fsub_rn(1.f, sb);
+      const float wb = sb * T;
+      Rr = fmaf(ncd.y, wb, Rr);
+      const float ndb = fmaf(T, ncd.y, Rr * rcp_approx(omb));
+      T = __fmul_rn(T, omb);
+      const float2 w = f2(wa, wb);
+      v6 = f2_fma(f2(g.x), w, v6);
+      v7 = f2_fma(f2(g.y), w, v7);
+      v8 = f2_fma(f2(g.z), w, v8);
+      const float2 m = f2(oka && raw.x <= kAlphaMax ? nda * G.x : 0.f, okb && raw.y <= kAlphaMax ? ndb * G.y : 0.f);
+      const float2 mt = f2_mul(m, tt), mdy = f2_mul(m, dy);
+      v0 = f2_add(v0, mt);
+      v1 = f2_add(v1, mdy);
+      v2 = f2_fma(mt, tt, v2);
+      v3 = f2_fma(mt, dy, v3);
+      v4 = f2_fma(mdy, dy, v4);
+      v5 = f2_add(v5, m);
+    }
+    __syncwarp();   // this chunk's reads before the next chunk's ring writes
+  }
+  out.v[0] = v0; out.v[1] = v1; out.v[2] = v2; out.v[3] = v3; out.v[4] = v4; out.v[5] = v5;
+  out.v[6] = v6; out.v[7] = v7; out.v[8] = v8;
 }
 
 template <int TW, int TH>
@@ -792,8 +916,6 @@ __global__ void __launch_bounds__(kSplatThreads, kSplatBlocks) raster_bwd_splat_
   const int nb = (n + 63) >> 6;                     // buckets of 64 list entries
   const uint64_t bk0 = ckpt_bucket(rg.x, tile);
   uint16_t *live = s_live[warp];
-  float4 *ra = s_ring[warp][0], *rb = s_ring[warp][1];
-  const float4 *rw = s_ring[warp][0];
   for (int b = part + kSplatSplit * warp; b < nb;) {
     // this lane's two consecutive list entries (a, b) = (64 b + 2 lane, 64 b + 2 lane + 1)
     const int ja = 64 * b + 2 * lane, jb = ja + 1;
@@ -844,111 +966,276 @@ __global__ void __launch_bounds__(kSplatThreads, kSplatBlocks) raster_bwd_splat_
         kn = ckpt.slots[(uint64_t)sl * 64 + (py & 7) * 8 + (px & 7)];
     };
     fetch(lane);
-    // ring slots 32..63 read as stopped until the second chunk replaces them
-    ra[32 + lane] = make_float4(0.f, 0.f, 0.f, 0.f);
-    rb[32 + lane] = make_float4(0.f, 0.f, 1.f, 0.f);
-    // moments accumulated negated (see nd below), colour terms as they are; .x the
-    // sums of entry a, .y of entry b
-    float2 v0 = f2(0.f), v1 = f2(0.f), v2 = f2(0.f), v3 = f2(0.f), v4 = f2(0.f), v5 = f2(0.f);
-    float2 v6 = f2(0.f), v7 = f2(0.f), v8 = f2(0.f);
-    float T = 1.f, Rr = 0.f;
-    const uint32_t jja = (uint32_t)ja, jjb = (uint32_t)jb;
-    const float2 U = f2(xya.x, xyb.x), V = f2(xya.y, xyb.y);
-    const float2 A2 = f2(__fmul_rn(cua.x, kNegHalfLog2e), __fmul_rn(cub.x, kNegHalfLog2e));
-    const float2 BE = f2(cua.y, cub.y);
-    const float2 G2 = f2(__fmul_rn(cua.z, kNegHalfLog2e), __fmul_rn(cub.z, kNegHalfLog2e));
-    const float2 O = f2(cua.w, cub.w);
-    const float2 NCX = f2(-ca.x, -cb.x), NCY = f2(-ca.y, -cb.y), NCZ = f2(-ca.z, -cb.z);
-    for (int s0 = 0; s0 < nl + 31; s0 += 32) {
-      {
-        // ring slots s0 .. s0 + 31; past the list a slot reads as stopped (stop 0)
-        float4 A = make_float4(0.f, 0.f, 0.f, 0.f), B = make_float4(0.f, 0.f, 1.f, 0.f);
-        if (pn >= 0) {
-          const float4 g = s_g[pn];
-          A = make_float4(g.x, g.y, g.z, __uint_as_float(s_stop[pn]));
-          B = make_float4((float)(tc.tx * TW + pn % TW) + 0.5f, (float)(tc.ty * TH + pn / TW) + 0.5f, kn.x,
-                          g.w - (kn.y * g.x + kn.z * g.y + kn.w * g.z));
-        }
-        ra[(s0 + lane) & (kSplatRing - 1)] = A;
-        rb[(s0 + lane) & (kSplatRing - 1)] = B;
-        fetch(s0 + 32 + lane);
-        __syncwarp();
+    SplatEntries e;
+    e.set(ja, xya, xyb, make_float4(__fmul_rn(cua.x, kNegHalfLog2e), cua.y, __fmul_rn(cua.z, kNegHalfLog2e), cua.w),
+          make_float4(__fmul_rn(cub.x, kNegHalfLog2e), cub.y, __fmul_rn(cub.z, kNegHalfLog2e), cub.w), ca, cb);
+    SplatMoments v;
+    splat_walk(e, nl, s_ring[warp][0], lane, v, [&](int s0, float4 &A, float4 &B) {
+      // live pixel s0 + lane of the walk; past the list a slot reads as stopped (stop 0)
+      A = make_float4(0.f, 0.f, 0.f, 0.f);
+      B = make_float4(0.f, 0.f, 1.f, 0.f);
+      if (pn >= 0) {
+        const float4 g = s_g[pn];
+        A = make_float4(g.x, g.y, g.z, __uint_as_float(s_stop[pn]));
+        B = make_float4((float)(tc.tx * TW + pn % TW) + 0.5f, (float)(tc.ty * TH + pn / TW) + 0.5f, kn.x,
+                        g.w - (kn.y * g.x + kn.z * g.y + kn.w * g.z));
       }
-      const int s1 = min(s0 + 32, nl + 31);
-#pragma unroll 8
-      for (int s = s0; s < s1; ++s) {
-        const float4 *q = rw + ((s - lane) & (kSplatRing - 1));
-        const float Tin = __shfl_up_sync(0xffffffffu, T, 1);
-        const float Rin = __shfl_up_sync(0xffffffffu, Rr, 1);
-        const float4 g = q[0], p = q[kSplatRing];
-        T = lane == 0 ? p.z : Tin;
-        Rr = lane == 0 ? p.w : Rin;
-        // falloff of both entries at this pixel: the forward's operations and roundings
-        // (the pixel's coordinates are a broadcast operand: two scalar subtractions
-        // cost less than a packed one and the moves that would build its pair)
-        const float2 dx = f2(__fsub_rn(U.x, p.x), __fsub_rn(U.y, p.x));
-        const float2 dy = f2(__fsub_rn(V.x, p.y), __fsub_rn(V.y, p.y));
-        const float2 tt = f2_fma(BE, dy, dx);
-        const float2 e = f2_fma(f2_mul(A2, tt), tt, f2_mul(G2, f2_mul(dy, dy)));
-        const float2 G = f2(ex2_approx(e.x), ex2_approx(e.y));
-        const float2 raw = f2_mul(O, G);
-        const float2 al = f2(fminf(kAlphaMax, raw.x), fminf(kAlphaMax, raw.y));
-        // a position before the pixel's stop (false on stopped pixels and for lanes
-        // without an entry) where sigma reaches the floor; elsewhere sigma 0 leaves T,
-        // R and every sum as they are
-        const uint32_t stop = __float_as_uint(g.w);
-        const bool oka = jja < stop && al.x >= kAlphaMin, okb = jjb < stop && al.y >= kAlphaMin;
-        const float2 ncd = f2_fma(NCZ, f2(g.z), f2_fma(NCY, f2(g.y), f2_mul(NCX, f2(g.x))));   // -<c, g>
-        // entry a, then entry b, in list order: -dL/dsigma = -T <c, g> + R / (1 - sigma)
-        const float sa = oka ? al.x : 0.f;
-        const float oma = __fsub_rn(1.f, sa);
-        const float wa = sa * T;
-        Rr = fmaf(ncd.x, wa, Rr);
-        const float nda = fmaf(T, ncd.x, Rr * rcp_approx(oma));
-        T = __fmul_rn(T, oma);
-        const float sb = okb ? al.y : 0.f;
-        const float omb = __fsub_rn(1.f, sb);
-        const float wb = sb * T;
-        Rr = fmaf(ncd.y, wb, Rr);
-        const float ndb = fmaf(T, ncd.y, Rr * rcp_approx(omb));
-        T = __fmul_rn(T, omb);
-        const float2 w = f2(wa, wb);
-        v6 = f2_fma(f2(g.x), w, v6);
-        v7 = f2_fma(f2(g.y), w, v7);
-        v8 = f2_fma(f2(g.z), w, v8);
-        const float2 m = f2(oka && raw.x <= kAlphaMax ? nda * G.x : 0.f, okb && raw.y <= kAlphaMax ? ndb * G.y : 0.f);
-        const float2 mt = f2_mul(m, tt), mdy = f2_mul(m, dy);
-        v0 = f2_add(v0, mt);
-        v1 = f2_add(v1, mdy);
-        v2 = f2_fma(mt, tt, v2);
-        v3 = f2_fma(mt, dy, v3);
-        v4 = f2_fma(mdy, dy, v4);
-        v5 = f2_add(v5, m);
-      }
-      __syncwarp();   // this chunk's reads before the next chunk's ring writes
-    }
+      fetch(s0 + 32 + lane);
+    });
     // each entry's sums once into its record's gradients (record and conic read again)
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int jh = h == 0 ? ja : jb;
-      const float v[9] = {-(h == 0 ? v0.x : v0.y), -(h == 0 ? v1.x : v1.y), -(h == 0 ? v2.x : v2.y),
-                          -(h == 0 ? v3.x : v3.y), -(h == 0 ? v4.x : v4.y), -(h == 0 ? v5.x : v5.y),
-                          h == 0 ? v6.x : v6.y, h == 0 ? v7.x : v7.y, h == 0 ? v8.x : v8.y};
-      if (jh < n && (v[0] != 0.f || v[1] != 0.f || v[2] != 0.f || v[3] != 0.f || v[4] != 0.f ||
-                     v[5] != 0.f || v[6] != 0.f || v[7] != 0.f || v[8] != 0.f)) {
-        const uint32_t r = vals[rg.x + jh];
-        if (!GS_CHECK(r < n_records, 1, r)) continue;
-        const float4 cu = conic_o[r];
-        const float oA = cu.w * cu.x, ho = -0.5f * cu.w;
-        red_add_v2(g_mean2d + 2 * (size_t)r, -oA * v[0], -(oA * cu.y * v[0] + cu.w * cu.z * v[1]));
-        red_add_v4(g_co + 4 * (size_t)r, ho * v[2], -oA * v[3], ho * v[4], v[5]);
-        red_add_v4(g_rgb + 4 * (size_t)r, v[6], v[7], v[8], 0.f);
+    for (int h = 0; h < 2; ++h)
+      if (ja + h < n) {
+        const uint32_t r = vals[rg.x + ja + h];
+        if (GS_CHECK(r < n_records, 1, r)) v.flush(h, r, conic_o, g_mean2d, g_co, g_rgb);
       }
-    }
     __syncwarp();   // the next bucket rewrites this warp's live list
     uint32_t nxt = 0;
     if (lane == 0) nxt = atomicAdd(&s_next, 1u);
     b = part + kSplatSplit * (int)__shfl_sync(0xffffffffu, nxt, 0);
+  }
+}
+
+// Backward without checkpoints from the forward (gs_raster_bwd). One CTA per tile takes the
+// list in windows of WB buckets (64 entries each), every window in two steps:
+//   1. forward: warp w walks the window on 8 x 8 block w (two pixels per lane, the
+//      forward's recurrence and decisions) and leaves (T, R) of its pixels at each
+//      bucket's start in shared memory, and each pixel's last composited position;
+//   2. backward: warp b takes bucket b and lets the pixels still live at its start flow
+//      through its lanes (splat_walk), each lane summing its own two entries.
+// raster_bwd_kernel reduces every entry's nine sums over the warp and the CTA, about 500
+// cycles per entry, one entry after another; on a frame of few tiles the longest tile's list
+// makes that the launch's time. Here the second step has a warp's worth of independent work
+// per bucket however few tiles there are, and no reduction, at the price of a second forward
+// walk (the kernels alone, 16 x 16 tiles, raster_bwd_kernel -> this one): 206 -> 58 us at
+// 2k Gaussians on 64 x 64 (16 tiles), 404 -> 175 at 100k on 312 x 207 (260), 467 -> 290 at
+// 300k on 623 x 413 (1014), 546 -> 446 at 500k on 900 x 600 (2166), 923 -> 905 at 1.5M on
+// 1246 x 826 (4056); 16224 tiles 1981 -> 2214; 8 x 8 tiles 470 -> 437 at 900 x 600 and
+// 906 -> 994 at 1246 x 826; 16 x 32 tiles 632 -> 605 and 1086 -> 1279. Hence the line at
+// kTilePixels padded pixels. Lists of a few entries leave its buckets empty: 44 -> 58 us at
+// 5k Gaussians on 623 x 413, 132 -> 110 at 20k, 62 -> 45 at 5k on 312 x 207; hence
+// kTileRecords records a tile.
+constexpr int64_t kTilePixels = 600000;   // padded pixels of the frame (tiles x tile size), below
+constexpr int64_t kTileRecords = 12;      // records per tile, at least
+
+template <int TW, int TH, int WB>
+struct BwdTile {
+  // two CTAs of eight warps an SM (128 registers a thread), or five of four (102)
+  static constexpr int NP = TW * TH, NB = NP / 64, NW = NB > 4 ? NB : (WB > 4 ? WB : 4), WE = WB * 64;
+  float4 co[WE + 1], rgb[WE + 1];         // (k A, beta, k gamma, o); colour, block mask; last: opacity 0
+  float4 g[NP];                           // (dL/dout, stop bound)
+  float2 ck[WB][NP];                      // (T, R) before the bucket
+  float2 state[NP];                       // (T, R) at the window's start
+  float4 ring[NW][2 * kSplatRing];
+  float2 xy[WE + 1];
+  uint32_t rec[WE];
+  uint32_t stop[NP];                      // one past the last composited position so far
+  uint16_t live[NW][NP];
+};
+
+template <int TW, int TH, bool STOP, int WB>
+__global__ void __launch_bounds__(BwdTile<TW, TH, WB>::NW * 32, BwdTile<TW, TH, WB>::NW > 4 ? 2 : 5) raster_bwd_tile_kernel(
+    const float2 *__restrict__ mean2d, const float4 *__restrict__ conic_o, const float4 *__restrict__ rgb,
+    const uint32_t *__restrict__ vals, const uint2 *__restrict__ ranges, const gs_camera_t *__restrict__ cams,
+    int n_views, const float *__restrict__ image, const float *__restrict__ d_image,
+    const uint32_t *__restrict__ stop_in, float *__restrict__ g_mean2d, float *__restrict__ g_co,
+    float *__restrict__ g_rgb, uint64_t n_records, uint64_t list_cap, int split) {
+  using S = BwdTile<TW, TH, WB>;
+  constexpr int NP = S::NP, NB = S::NB, NT = S::NW * 32, WE = S::WE;
+  extern __shared__ float4 s_raw[];
+  S &s = *reinterpret_cast<S *>(s_raw);
+  __shared__ uint32_t s_max;
+  const int tile = blockIdx.x / split, part = blockIdx.x - tile * split;
+  const TileCoord tc = tile_coord(cams, n_views, tile);
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const uint32_t lt = (1u << lane) - 1u;
+  if (t == 0) {
+    s.xy[WE] = make_float2(0.f, 0.f);
+    s.co[WE] = s.rgb[WE] = make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+  if (STOP) {
+    if (t == 0) s_max = 0;
+    __syncthreads();
+  }
+  {
+    const int64_t plane = (int64_t)tc.W * tc.H;
+    const float *img = image + 3 * tc.pix_off;
+    const float *dim = d_image + 3 * tc.pix_off;
+    uint32_t mx = 0;
+    for (int p = t; p < NP; p += NT) {
+      const int px = tc.tx * TW + p % TW, py = tc.ty * TH + p / TW;
+      float4 g = make_float4(0.f, 0.f, 0.f, 0.f);
+      float R = 0.f;
+      if (px < tc.W && py < tc.H) {
+        const int64_t q = (int64_t)py * tc.W + px;
+        g.x = dim[q]; g.y = dim[plane + q]; g.z = dim[2 * plane + q];
+        R = g.x * img[q] + g.y * img[plane + q] + g.z * img[2 * plane + q];
+        const uint32_t st = STOP ? stop_in[tc.pix_off + q] : 0xffffffffu;
+        g.w = __uint_as_float(st);
+        mx = max(mx, st);
+      }
+      s.g[p] = g;
+      s.state[p] = make_float2(1.f, R);
+      s.stop[p] = 0u;
+    }
+    if (STOP) {
+      mx = __reduce_max_sync(0xffffffffu, mx);
+      if (lane == 0) atomicMax(&s_max, mx);
+    }
+  }
+  __syncthreads();
+  uint2 rg = ranges[tile];
+  if (!GS_CHECK(rg.x <= rg.y && (uint64_t)rg.y <= list_cap, 2, tile)) rg = make_uint2(0u, 0u);
+  int n = (int)(rg.y - rg.x);
+  if (STOP) n = min(n, (int)min(s_max, 0x7fffffffu));
+  // this CTA's blocks are part, part + split, ...; warp w walks the w-th of them forward, two
+  // pixels per lane
+  const int blocks = NB / split, block = part + split * (warp < blocks ? warp : 0);
+  int lx, ly;
+  pixel_of<TW>(block * 32 + lane, lx, ly);
+  const int p0 = ly * TW + lx;
+  const float fy = (float)(tc.ty * TH + ly) + 0.5f;
+  const float fx0 = (float)(tc.tx * TW + lx) + 0.5f, fx1 = fx0 + 1.f;
+  for (int w0 = 0; w0 < n; w0 += WE) {
+    const int cnt = min(WE, n - w0), nb = (cnt + 63) >> 6;
+    for (int j = t; j < 64 * nb; j += NT) {
+      if (j < cnt) {
+        uint32_t r = vals[rg.x + w0 + j];
+        if (!GS_CHECK(r < n_records, 1, r)) r = 0;
+        float4 raw;
+        s.rec[j] = r;
+        stage<TW, TH, 8, 8>(mean2d, conic_o, rgb, r, tc.tx * TW, tc.ty * TH, tc.W, tc.H, s.xy[j], s.co[j], s.rgb[j],
+                            raw);
+      } else {   // the rest of the last bucket: no block, and past every stop
+        s.xy[j] = make_float2(0.f, 0.f);
+        s.co[j] = s.rgb[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+    }
+    __syncthreads();
+    bool going = false;
+    if (warp < blocks) {
+      float4 tr = *reinterpret_cast<const float4 *>(&s.state[p0]);   // (T, R) of both pixels
+      const float4 g0 = s.g[p0], g1 = s.g[p0 + 1];
+      uint32_t st0 = s.stop[p0], st1 = s.stop[p0 + 1];
+      const uint32_t end0 = __float_as_uint(g0.w), end1 = __float_as_uint(g1.w);
+      // past the image, or past the walk's end (without a stop index the transmittance
+      // of a stopped pixel is kept below zero)
+      bool done0 = STOP ? end0 <= (uint32_t)w0 : (end0 == 0u || tr.x < 0.f);
+      bool done1 = STOP ? end1 <= (uint32_t)w0 : (end1 == 0u || tr.z < 0.f);
+      for (int kb = 0; kb < nb; ++kb) {
+        if (__all_sync(0xffffffffu, done0 && done1)) break;
+        *reinterpret_cast<float4 *>(&s.ck[kb][p0]) = tr;
+        // the bucket's entries that meet the block, closed up, an odd count filled with the
+        // entry of opacity 0 that ends the window
+        uint16_t *list = s.live[warp];
+        int ns = 0;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int j = 64 * kb + 32 * h + lane;
+          const bool on = (__float_as_uint(s.rgb[j].w) >> block) & 1u;
+          const uint32_t bal = __ballot_sync(0xffffffffu, on);
+          if (on) list[ns + __popc(bal & lt)] = (uint16_t)j;
+          ns += __popc(bal);
+        }
+        if ((ns & 1) && lane == 0) list[ns] = (uint16_t)WE;
+        __syncwarp();
+        auto alpha = [&](int j, float &al0, float &al1) {
+          const float2 xy = s.xy[j];
+          const float4 co = s.co[j];
+          // the checkpointing forward's falloff, operation for operation
+          const float dx0 = __fsub_rn(xy.x, fx0), dx1 = __fsub_rn(xy.x, fx1), dy = __fsub_rn(xy.y, fy);
+          const float gdd = __fmul_rn(co.z, __fmul_rn(dy, dy));
+          const float t0 = __fmaf_rn(co.y, dy, dx0), t1 = __fmaf_rn(co.y, dy, dx1);
+          const float e0 = __fmaf_rn(__fmul_rn(co.x, t0), t0, gdd), e1 = __fmaf_rn(__fmul_rn(co.x, t1), t1, gdd);
+          al0 = fminf(kAlphaMax, __fmul_rn(co.w, ex2_approx(e0)));
+          al1 = fminf(kAlphaMax, __fmul_rn(co.w, ex2_approx(e1)));
+        };
+        auto composite = [&](int j, float al0, float al1) {
+          const float4 c = s.rgb[j];
+          const uint32_t pos = (uint32_t)(w0 + j);
+          const bool a0 = !done0 && al0 >= kAlphaMin && (!STOP || pos < end0);
+          const bool a1 = !done1 && al1 >= kAlphaMin && (!STOP || pos < end1);
+          const float Tn0 = __fmul_rn(tr.x, __fsub_rn(1.f, al0)), Tn1 = __fmul_rn(tr.z, __fsub_rn(1.f, al1));
+          const bool c0 = a0 && (STOP || !(Tn0 < kTMin)), c1 = a1 && (STOP || !(Tn1 < kTMin));
+          if (!STOP) {
+            done0 = done0 || (a0 && !c0);
+            done1 = done1 || (a1 && !c1);
+          }
+          const float wt0 = (c0 ? al0 : 0.f) * tr.x, wt1 = (c1 ? al1 : 0.f) * tr.z;
+          const float cd0 = fmaf(c.z, g0.z, fmaf(c.y, g0.y, c.x * g0.x));
+          const float cd1 = fmaf(c.z, g1.z, fmaf(c.y, g1.y, c.x * g1.x));
+          tr.y = fmaf(-cd0, wt0, tr.y);
+          tr.w = fmaf(-cd1, wt1, tr.w);
+          tr.x = c0 ? Tn0 : tr.x;
+          tr.z = c1 ? Tn1 : tr.z;
+          st0 = c0 ? pos + 1u : st0;
+          st1 = c1 ? pos + 1u : st1;
+        };
+        for (int i = 0; i < ns; i += 2) {   // two entries' sigmas at a time, as in the forward
+          const int j = list[i], k = list[i + 1];
+          float aj0, aj1, ak0, ak1;
+          alpha(j, aj0, aj1);
+          alpha(k, ak0, ak1);
+          composite(j, aj0, aj1);
+          composite(k, ak0, ak1);
+        }
+        __syncwarp();
+        if (STOP) {
+          done0 = end0 <= (uint32_t)(w0 + 64 * kb + 64);
+          done1 = end1 <= (uint32_t)(w0 + 64 * kb + 64);
+        }
+      }
+      going = !(done0 && done1);
+      if (!STOP) {
+        if (done0) tr.x = -1.f;
+        if (done1) tr.z = -1.f;
+      }
+      *reinterpret_cast<float4 *>(&s.state[p0]) = tr;
+      s.stop[p0] = st0;
+      s.stop[p0 + 1] = st1;
+    }
+    const bool more = __syncthreads_or(going);
+    // warp -> bucket; in a short window the warps left over share the buckets' pixels, by
+    // 8 x 8 blocks
+    const int nbp = nb > 4 ? 8 : (nb > 2 ? 4 : nb);
+    const int parts = min(S::NW / nbp, blocks), bucket = warp & (nbp - 1), pp = warp / nbp;
+    if (bucket < nb && pp < parts) {
+      // the bucket's live pixels: those that composite at or after its start
+      uint16_t *live = s.live[warp];
+      const uint32_t start = (uint32_t)(w0 + 64 * bucket);
+      int nl = 0;
+      for (int i = 0; i < 2 * (blocks / parts); ++i) {   // half a block at a time
+        const int k = part + split * (pp + parts * (i >> 1));
+        const int q = ((k / (TW / 8)) * 8 + (i & 1) * 4 + (lane >> 3)) * TW + (k % (TW / 8)) * 8 + (lane & 7);
+        const bool on = s.stop[q] > start;
+        const uint32_t bal = __ballot_sync(0xffffffffu, on);
+        if (on) live[nl + __popc(bal & lt)] = (uint16_t)q;
+        nl += __popc(bal);
+      }
+      __syncwarp();
+      if (nl > 0) {
+        const int j = 64 * bucket + 2 * lane;
+        SplatEntries e;
+        e.set(w0 + j, s.xy[j], s.xy[j + 1], s.co[j], s.co[j + 1], s.rgb[j], s.rgb[j + 1]);
+        SplatMoments v;
+        splat_walk(e, nl, s.ring[warp], lane, v, [&](int s0, float4 &A, float4 &B) {
+          A = make_float4(0.f, 0.f, 0.f, 0.f);
+          B = make_float4(0.f, 0.f, 1.f, 0.f);
+          if (s0 + lane < nl) {
+            const int p = live[s0 + lane];
+            const float4 g = s.g[p];
+            const float2 k = s.ck[bucket][p];
+            A = make_float4(g.x, g.y, g.z, __uint_as_float(s.stop[p]));
+            B = make_float4((float)(tc.tx * TW + p % TW) + 0.5f, (float)(tc.ty * TH + p / TW) + 0.5f, k.x, k.y);
+          }
+        });
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+          if (j + h < cnt) v.flush(h, s.rec[j + h], conic_o, g_mean2d, g_co, g_rgb);
+      }
+    }
+    if (!more) break;
+    __syncthreads();   // the next window rewrites the entries and the checkpoints
   }
 }
 
@@ -1065,22 +1352,52 @@ static gs_status_t launch_bwd(const gs_proj_t *proj, const gs_bins_t *bins, cons
   GS_CUDA_TRY(cudaMemsetAsync(g->d_mean2d, 0, R * 2 * sizeof(float), s));
   GS_CUDA_TRY(cudaMemsetAsync(g->d_conic_opacity, 0, R * 4 * sizeof(float), s));
   GS_CUDA_TRY(cudaMemsetAsync(g->d_rgb, 0, R * 4 * sizeof(float), s));
-  // 2 pixels per thread: 8 x 8 warp blocks skip more records than 8 x 16 ones
-  // (4 pixels per thread) save in shared per-entry work.
-  constexpr int PX = 2;
   const auto *m2 = reinterpret_cast<const float2 *>(proj->mean2d);
   const auto *co = reinterpret_cast<const float4 *>(proj->conic_opacity);
   const auto *c = reinterpret_cast<const float4 *>(proj->rgb);
   const auto *rg = reinterpret_cast<const uint2 *>(bins->ranges);
+  if ((int64_t)frame->n_tiles * TW * TH >= kTilePixels || proj->n_records < kTileRecords * frame->n_tiles) {
+    // 2 pixels per thread: 8 x 8 warp blocks skip more records than 8 x 16 ones
+    // (4 pixels per thread) save in shared per-entry work.
+    constexpr int PX = 2;
 #define GS_BWD(STOPV, HALFV)                                                                               \
   raster_bwd_kernel<TW, TH, PX, STOPV, HALFV><<<frame->n_tiles, TW * TH / PX, 0, s>>>(                       \
       m2, co, c, bins->vals, rg, frame->cams_dev, frame->n_views, image, d_image, stop, g->d_mean2d,          \
       g->d_conic_opacity, g->d_rgb, (uint64_t)proj->n_records, (uint64_t)bins->capacity)
-  if (stop)
-    half ? GS_BWD(true, true) : GS_BWD(true, false);
-  else
-    half ? GS_BWD(false, true) : GS_BWD(false, false);
+    if (stop)
+      half ? GS_BWD(true, true) : GS_BWD(true, false);
+    else
+      half ? GS_BWD(false, true) : GS_BWD(false, false);
 #undef GS_BWD
+    GS_LAUNCH_CHECK();
+    return GS_OK;
+  }
+  // With few tiles, a CTA takes a half or a quarter of its tile's 8 x 8 blocks, and eight
+  // warps with windows of eight buckets shorten the longest tile's walk; with many, CTAs of four
+  // warps keep more of their warps busy in the forward step (260 tiles: 129 against 158 us
+  // for a training step's kernel; 1014 tiles: 196 against 215. 16 tiles: whole, halves, quarters
+  // 79, 56, 44 us; 260 tiles: 150, 129, 142).
+  constexpr int NB = BwdTile<TW, TH, 1>::NB;
+  const bool few = frame->n_tiles < 2 * num_sms();
+  int split = 1;
+  while (split < 4 && 2 * split <= NB && frame->n_tiles * split < 2 * num_sms()) split *= 2;
+  auto go = [&](auto kern, int threads, size_t smem) -> gs_status_t {
+    GS_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    kern<<<frame->n_tiles * split, threads, smem, s>>>(
+        m2, co, c, bins->vals, rg, frame->cams_dev, frame->n_views, image, d_image, stop, g->d_mean2d,
+        g->d_conic_opacity, g->d_rgb, (uint64_t)proj->n_records, (uint64_t)bins->capacity, split);
+    return GS_OK;
+  };
+  // the staging depth's half: windows of half as many buckets
+#define GS_BWD(STOPV, WB) \
+  go(raster_bwd_tile_kernel<TW, TH, STOPV, WB>, BwdTile<TW, TH, WB>::NW * 32, sizeof(BwdTile<TW, TH, WB>))
+  gs_status_t st;
+  if (stop)
+    st = few && !half ? GS_BWD(true, 8) : (few || !half ? GS_BWD(true, 4) : GS_BWD(true, 2));
+  else
+    st = few && !half ? GS_BWD(false, 8) : (few || !half ? GS_BWD(false, 4) : GS_BWD(false, 2));
+#undef GS_BWD
+  if (st) return st;
   GS_LAUNCH_CHECK();
   return GS_OK;
 }

@@ -12,6 +12,7 @@ import torch
 
 from oracle import raster as oras
 from paper_2507_20239_gb300 import rasterizer as R
+from paper_2507_20239_gb300 import synth
 from tests.gs_fixtures import oracle_lists, oracle_records_fp32, records_to_gpu, rel_l2, scene
 
 pytestmark = pytest.mark.gpu
@@ -163,3 +164,34 @@ def test_raster_full_size_sampled_tiles():
         for k in got:
             e = rel_l2(got[k], g[k])
             assert e < GRAD_TOL, (k, e, st is not None)
+
+
+@pytest.mark.parametrize("use_stop", [False, True])
+@pytest.mark.parametrize("depth", [0, 1])
+@pytest.mark.parametrize("n,size,tile", [
+    (190, (64, 64), (16, 16)),       # 16 tiles: a quarter of a tile per CTA; one short window
+    (2500, (61, 50), (16, 16)),      # lists over several windows, ragged edges
+    (300, (250, 183), (16, 16)),     # 192 tiles: half a tile per CTA; too few records a tile below
+    (2600, (250, 183), (16, 16)),
+    (5000, (333, 301), (16, 16)),    # 399 tiles: whole tiles, four-warp CTAs
+    (900, (37, 64), (8, 8)), (3000, (200, 190), (8, 8)),
+    (3000, (130, 70), (16, 32)), (3000, (70, 130), (32, 16))])
+def test_tile_backward_matches_per_splat_backward(n, size, tile, depth, use_stop):
+    """gs_raster_bwd's paths by frame size against gs_raster_bwd_splat on the same lists:
+    FP32 on both sides, the sums in another order (1e-4, as between the two backwards
+    elsewhere). A wide camera puts 60 to 700 entries in a tile's list: one window and several,
+    with bucket counts that are no multiple of the warps'."""
+    sc = synth.small_scene(n, n=n, width=size[0], height=size[1])
+    frame = R.Frame(sc.cameras, tile=tile)
+    P = R.to_device_params(sc.params())
+    proj = R.project(P, 0, frame)
+    bins = R.bin_sort(proj, frame)
+    ckpt = R.alloc_ckpt(frame, bins)
+    bg = (0.2, 0.1, 0.4)
+    img, _, stop = R.raster_fwd_ckpt(proj, bins, frame, ckpt, bg)
+    d_image = torch.randn(img.shape, generator=torch.Generator("cuda").manual_seed(n), device="cuda")
+    want = R.raster_bwd_splat(proj, bins, frame, img, d_image, stop, ckpt)
+    got = R.raster_bwd(proj, bins, frame, img, d_image, bg, stop=stop if use_stop else None, stage_depth=depth)
+    for k in ("d_mean2d", "d_conic_opacity", "d_rgb"):
+        a, b = getattr(got, k).cpu().numpy(), getattr(want, k).cpu().numpy()
+        assert np.linalg.norm(b) > 0 and rel_l2(a, b) < 1e-4, k
