@@ -40,7 +40,7 @@ typedef enum {
   GS_ERR_INVALID_ARG = 1,
   GS_ERR_CAPACITY = 2,     /* a device-side count exceeded a caller capacity     */
   GS_ERR_CUDA = 3,         /* a CUDA launch or runtime call failed               */
-  GS_ERR_TIMEOUT = 4,      /* a bounded device wait ran out (reserved)           */
+  GS_ERR_TIMEOUT = 4,      /* a bounded device wait ran out (gs_bin_sort's sort) */
   GS_ERR_UNSUPPORTED = 5   /* valid request this build does not implement        */
 } gs_status_t;
 
@@ -73,7 +73,9 @@ typedef struct {
   int32_t max_width, max_height;
   int32_t sort_fused_bits; /* gs_bin_sort: low tile-id bits sorted while emitting
                             * (1..8, at most the tile-id width); 0 = automatic.
-                            * A tuning knob: the order produced is the same. */
+                            * A tuning knob: the order produced is the same. It
+                            * has an effect only on views of more than 20000
+                            * tiles, whose entries are sorted by tile id.     */
 } gs_frame_t;
 
 /* Gaussian parameters, device SoA (Eq. 1: position, scale, rotation, opacity, SH):
@@ -203,7 +205,8 @@ gs_status_t gs_project(const gs_params_t *params, const gs_frame_t *frame, gs_pr
  * entry per tile row of each visible record's rectangle (in practice fewer than M).
  * Device-side: if M or that row count exceeds bins->capacity, GS_ERR_CAPACITY is
  * OR-ed into *d_error, *bins->d_count receives the larger of the two (the capacity
- * needed) and vals holds no lists, every range being [0, 0). */
+ * needed) and vals holds no lists, every range being [0, 0). If a bounded wait of
+ * the depth sort runs out, GS_ERR_TIMEOUT is OR-ed and every range is [0, 0). */
 gs_status_t gs_bin_sort(const gs_proj_t *proj, const gs_frame_t *frame, gs_bins_t *bins,
                         void *ws, size_t ws_bytes, int32_t *d_error, gs_stream_t stream);
 

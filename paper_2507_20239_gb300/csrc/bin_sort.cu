@@ -8,6 +8,10 @@
 // per tile row, the ellipse's x-extent over the row's pixel centres keeps a
 // contiguous run of columns (the exact ellipse-box test, band_span_rn).
 //
+// Two paths give that order. Views whose tiles fit the shared-memory tables of
+// bin_direct.cuh (up to 20000, all but very large views or small tiles) have their entries
+// counted and written straight to their places. The others go the way of this file:
+//
 // Instead of one wide radix sort on (tile << 32 | depth) keys over all duplicates,
 // the order is built in two stable stages that give the same permutation:
 //   1. the visible records (one entry each) are stably sorted by their FP32 depth
@@ -29,6 +33,8 @@
 // Every count is read from device memory (no host round trip), so the whole
 // sequence can be captured into a CUDA graph. All grids are fixed-size and every
 // block derives its share of the work from the device-side count.
+#include <algorithm>
+
 #include "gs_common.cuh"
 #include "scan.cuh"
 
@@ -441,6 +447,12 @@ __device__ __forceinline__ uint32_t band_columns(float xl, float xr, int x0, int
   lo = a;
   return b >= a ? (uint32_t)(b - a + 1) : 0u;
 }
+
+}  // namespace gs
+
+#include "bin_direct.cuh"
+
+namespace gs {
 
 // Binning of 32 depth-ordered records per warp (one batch), one tile row of a
 // record's candidate rectangle (a "unit") at a time: the ellipse's x-extent over the
@@ -917,7 +929,10 @@ extern "C" size_t gs_bin_sort_workspace_size(int64_t n_records, int64_t dup_capa
   if (n_records < 0 || dup_capacity < 0) return 0;
   int tile_bits = 32, fbits = kMaxFusedBits;
   if (frame && !frame_sort_plan(frame, tile_bits, fbits)) return 0;
-  return bin_ws_layout(nullptr, n_records, dup_capacity, fbits).bytes;
+  const size_t pairs = bin_ws_layout(nullptr, n_records, dup_capacity, fbits).bytes;
+  if (!frame) return std::max(pairs, dir_ws_bound(n_records, dup_capacity));
+  const DirPlan plan = dir_plan(frame, n_records, dup_capacity);
+  return plan.ok ? dir_ws_size(frame, n_records, dup_capacity, plan) : pairs;
 }
 
 extern "C" gs_status_t gs_bin_sort(const gs_proj_t *proj, const gs_frame_t *frame, gs_bins_t *bins, void *ws,
@@ -931,9 +946,11 @@ extern "C" gs_status_t gs_bin_sort(const gs_proj_t *proj, const gs_frame_t *fram
   if ((reinterpret_cast<uintptr_t>(ws) & 255u) != 0) return GS_ERR_INVALID_ARG;
   int tile_bits, fbits;
   if (!frame_sort_plan(frame, tile_bits, fbits)) return GS_ERR_INVALID_ARG;
+  cudaStream_t s = as_stream(stream);
+  const DirPlan plan = dir_plan(frame, R, bins->capacity);
+  if (plan.ok) return dir_bin_sort(proj, frame, bins, ws, ws_bytes, plan, d_error, s);
   const BinWs w = bin_ws_layout(ws, R, bins->capacity, fbits);
   if (ws_bytes < w.bytes) return GS_ERR_INVALID_ARG;
-  cudaStream_t s = as_stream(stream);
   const int G = scan_blocks();
   uint32_t *n_vis = w.counters + 0, *m_total = w.counters + 1, *overflow = w.counters + 2;
   GS_CUDA_TRY(cudaMemsetAsync(w.counters, 0, 64, s));

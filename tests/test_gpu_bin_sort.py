@@ -195,3 +195,43 @@ def test_full_view_lists_hold_every_exact_fp64_pair():
                                              proj.radius.cpu().numpy(), cam.width, cam.height, (16, 16), tiles, recs)
     print(f"listed {listed}, exact-with-margin {must}, within the margin {between}")
     assert listed > 10_000_000 and must > 0.99 * listed and between < 1e-3 * listed
+
+
+def _wide(seed, n, width, height, tile=(16, 16), footprint=1.0):
+    cam = synth.Camera(np.eye(3, dtype=np.float32), np.zeros(3, np.float32), 100., 100., width / 2, height / 2,
+                       width, height)
+    return _synthetic_records(seed, n, [cam], tile), cam
+
+
+@pytest.mark.parametrize("n,size,tile", [
+    (1, (16, 16), (16, 16)), (63, (33, 17), (16, 16)), (2047, (300, 200), (16, 16)), (2049, (300, 200), (16, 16)),
+    (70_001, (100, 60), (8, 8)),            # few tiles, long lists: records of one chunk share every tile
+    (320_000, (640, 480), (16, 16)),        # chunks of equal weight instead of equal counts
+    (400_000, (1250, 830), (8, 8)),         # 16328 tiles: one mask word per tile
+    (20_000, (1700, 1300), (8, 8))])        # 34,669 tiles in a view: emitted pairs and radix passes
+def test_bin_sort_paths_by_frame_size(n, size, tile):
+    """Counting and pair paths at the edges of their batches (32 and 256 records), sort
+    partitions (2048), chunks and tables."""
+    recs, cam = _wide(n, n, *size, tile=tile)
+    _check(recs, [cam], tile)
+
+
+def test_bin_sort_many_records_in_one_place():
+    """Every record over the same few tiles, of depths in few values, in a view whose other
+    tiles stay empty: full masks in the emission, one chunk's weight in one place, ties kept in
+    record order; and a view in which nothing is visible beside it."""
+    recs, cam = _wide(21, 330_000, 400, 300)
+    r = recs[0]
+    n = len(r["radius"])
+    rng = np.random.default_rng(5)
+    r["mean2d"][:] = np.stack([rng.uniform(100, 130, n), rng.uniform(90, 120, n)], 1).astype(np.float32)
+    r["conic_f"][:] = [1 / 36.0, 0.0, 1 / 36.0]
+    r["q_max"][:] = np.float32(2 * np.log(255 * 0.5))
+    half = oproj.footprint_half(r["conic_f"].astype(np.float64), r["q_max"].astype(np.float64)).astype(np.float32)
+    r["rect"][:] = oproj.tile_rect(r["mean2d"], half, 16, 16, *r["grid"])
+    r["radius"][:] = 20
+    r["depth"][:] = rng.choice(np.float32([0.5, 1.0, 1.0000001, 7.25, 3e7]), n)
+    empty = {k: (v.copy() if isinstance(v, np.ndarray) else v) for k, v in r.items()}
+    for k in ("radius", "depth", "rect"):
+        empty[k][:] = 0
+    _check([r, empty], [cam, cam], (16, 16))
