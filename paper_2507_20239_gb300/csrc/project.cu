@@ -255,11 +255,12 @@ __global__ void __launch_bounds__(256) project_fwd_kernel(gs_params_t P, const g
 // Projection VJP, geometric part: conic, pixel mean and opacity gradients of every
 // view -> means (through t = W mu + t_w and J), log-scales, quaternion, opacity
 // logit; the densification statistic is fused. The colour part is project_bwd_sh.
-// Every input is requested at entry, before the visibility test (with several views
-// the per-view records follow it): the parameters of a Gaussian no view sees are read
-// and not used, but a thread waits for one round trip instead of two.
+// Every input is requested at entry, before the visibility test, and with several views
+// each record a view ahead: what belongs to a view that does not see the Gaussian is read
+// and not used, but a thread does not wait for a radius before it asks for the rest
+// (5M Gaussians, 4 views: GEOM_FIGURES).
 template <bool ONE_VIEW>
-__global__ void __launch_bounds__(128, 5) project_bwd_geom_kernel(gs_params_t P, const gs_camera_t *__restrict__ cams,
+__global__ void __launch_bounds__(128, ONE_VIEW ? 5 : 4) project_bwd_geom_kernel(gs_params_t P, const gs_camera_t *__restrict__ cams,
                                                                int n_views, gs_proj_t proj, gs_rec_grads_t rg,
                                                                gs_param_grads_t out, float *accum, int32_t *count) {
   const int64_t n = P.n;
@@ -269,14 +270,10 @@ __global__ void __launch_bounds__(128, 5) project_bwd_geom_kernel(gs_params_t P,
     const float4 q = reinterpret_cast<const float4 *>(P.quats)[g];
     const float ls0 = P.log_scales[3 * g + 0], ls1 = P.log_scales[3 * g + 1], ls2 = P.log_scales[3 * g + 2];
     const float logit = P.opacity_logits[g];
-    int rad1 = 0;
-    float2 gm1 = make_float2(0.f, 0.f);
-    float4 gco1 = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (ONE_VIEW) {
-      rad1 = proj.radius[g];
-      gm1 = reinterpret_cast<const float2 *>(rg.d_mean2d)[g];
-      gco1 = reinterpret_cast<const float4 *>(rg.d_conic_opacity)[g];
-    }
+    // the first view's record; with several, each is requested a view ahead
+    int rad1 = proj.radius[g];
+    float2 gm1 = reinterpret_cast<const float2 *>(rg.d_mean2d)[g];
+    float4 gco1 = reinterpret_cast<const float4 *>(rg.d_conic_opacity)[g];
     float d_mean[3] = {0.f, 0.f, 0.f};
     float dM[9] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};   // dL/dM, M = R S
     float d_logit = 0.f;
@@ -287,8 +284,16 @@ __global__ void __launch_bounds__(128, 5) project_bwd_geom_kernel(gs_params_t P,
     float qinv = 0.f, s0 = 0.f, s1 = 0.f, s2 = 0.f, M[9];
     Rot Rq;
     for (int v = 0; v < (ONE_VIEW ? 1 : n_views); ++v) {
-      const int64_t r = (int64_t)v * n + g;
-      if ((ONE_VIEW ? rad1 : proj.radius[r]) <= 0) continue;
+      const int rad = rad1;
+      const float2 gm = gm1;
+      const float4 gco = gco1;
+      if (!ONE_VIEW && v + 1 < n_views) {
+        const int64_t r = (int64_t)(v + 1) * n + g;
+        rad1 = proj.radius[r];
+        gm1 = reinterpret_cast<const float2 *>(rg.d_mean2d)[r];
+        gco1 = reinterpret_cast<const float4 *>(rg.d_conic_opacity)[r];
+      }
+      if (rad <= 0) continue;
       const gs_camera_t &cam = cams[v];
       if (!any) {
         any = true;
@@ -302,8 +307,6 @@ __global__ void __launch_bounds__(128, 5) project_bwd_geom_kernel(gs_params_t P,
       ProjGeom G;
       camera_space(cam, mx, my, mz, G.tx, G.ty, G.tz);
       project_cov(cam, M, G);
-      const float2 gm = ONE_VIEW ? gm1 : reinterpret_cast<const float2 *>(rg.d_mean2d)[r];
-      const float4 gco = ONE_VIEW ? gco1 : reinterpret_cast<const float4 *>(rg.d_conic_opacity)[r];
       if (accum) {
         const float gx = __fmul_rn(gm.x, 0.5f * (float)cam.width);
         const float gy = __fmul_rn(gm.y, 0.5f * (float)cam.height);
@@ -414,82 +417,94 @@ __global__ void __launch_bounds__(128, 5) project_bwd_geom_kernel(gs_params_t P,
 
 // Projection VJP, colour part: SH coefficient gradients (zero through a clamped
 // channel) and the colour's dependence on the viewing direction, added to the
-// mean gradients that project_bwd_geom_kernel wrote. STAGED (sh_stride ==
-// (DEG+1)^2): each warp moves the SH rows of its 32 Gaussians and their gradients
-// between global and shared memory with coalesced accesses (rows padded by one float).
-// ONE_VIEW: with a single view each coefficient's gradient is written once, right
-// after the coefficient has been read, so it overwrites the staged row in place and
-// one shared buffer suffices (twice the resident blocks).
-template <int DEG, bool STAGED, bool ONE_VIEW>
-__global__ void __launch_bounds__(128, ONE_VIEW ? 8 : 4) project_bwd_sh_kernel(
+// mean gradients that project_bwd_geom_kernel wrote. Bound by HBM. Each warp moves the SH rows
+// of its 32 Gaussians and their gradients between global and shared memory with coalesced
+// accesses (rows padded by one float); a Gaussian's gradient row takes the place of its
+// coefficients there. WIDE: the rows hold more coefficients than the degree in use (sh_stride >
+// (DEG+1)^2, as through most of a training run): only the used ones are read, and the whole
+// gradient row is written, zero beyond them (each thread reading and writing its own row in
+// global memory took SH_WIDE_FIGURES).
+// ONE_VIEW: each coefficient's gradient is written once, right after the coefficient has been
+// read. With several views it is summed in registers (SH_MULTI_FIGURES).
+template <int DEG, bool WIDE, bool ONE_VIEW>
+__global__ void __launch_bounds__(128, ONE_VIEW ? 8 : 5) project_bwd_sh_kernel(
     gs_params_t P, const gs_camera_t *__restrict__ cams, int n_views, gs_proj_t proj, gs_rec_grads_t rg,
     gs_param_grads_t out, bool vec) {
   constexpr int K = (DEG + 1) * (DEG + 1);
-  constexpr int RW = 3 * K, RP = RW + 1;
-  constexpr bool IN_PLACE = STAGED && ONE_VIEW;
-  __shared__ float s_sh[STAGED ? 4 * 32 * RP : 1];
-  __shared__ float s_dsh[IN_PLACE ? 1 : 4 * 32 * RP];
+  constexpr int RW = 3 * K, RP = RW + 1, R4 = (RW + 3) / 4;
+  __shared__ float s_sh[4 * 32 * RP];
   const int64_t n = P.n;
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  float *wsh = s_sh + (STAGED ? wib * 32 * RP : 0);
-  float *dsh_row = IN_PLACE ? wsh + lane * RP : s_dsh + (wib * 32 + lane) * RP;
+  const int gw = WIDE ? 3 * P.sh_stride : RW;   // floats per row in global memory
+  float *wsh = s_sh + wib * 32 * RP;
+  float *row = wsh + lane * RP;
   for (int64_t base = blockIdx.x * (int64_t)blockDim.x; base < n; base += (int64_t)gridDim.x * blockDim.x) {
     const int64_t g = base + threadIdx.x;
     const int64_t g0 = base + wib * 32;
     const int rows = (int)(n - g0 < 0 ? 0 : (n - g0 > 32 ? 32 : n - g0));
-    // with one view, the record's inputs are requested before the row staging, so
-    // they arrive while it runs
+    // the first view's record is requested before the row staging, so that it arrives while that
+    // runs; with several views each is requested a view ahead
     int rad1 = 0;
-    float mx1 = 0.f, my1 = 0.f, mz1 = 0.f;
+    float mx = 0.f, my = 0.f, mz = 0.f;
     float4 grgb1 = make_float4(0.f, 0.f, 0.f, 0.f);
     uint8_t cl1 = 0;
-    if (ONE_VIEW && g < n) {
+    bool seen = false;
+    if (g < n) {
       rad1 = proj.radius[g];
-      mx1 = P.means[3 * g + 0]; my1 = P.means[3 * g + 1]; mz1 = P.means[3 * g + 2];
+      mx = P.means[3 * g + 0]; my = P.means[3 * g + 1]; mz = P.means[3 * g + 2];
       grgb1 = reinterpret_cast<const float4 *>(rg.d_rgb)[g];
       cl1 = proj.clamped[g];
+      seen = rad1 > 0;
+      if (!ONE_VIEW)
+        for (int v = 1; v < n_views && !seen; ++v) seen = proj.radius[(int64_t)v * n + g] > 0;
     }
-    if (STAGED) {
-      // rows of Gaussians culled in every view are not read: their coefficients are
-      // never used and their gradient rows are zero
-      bool seen = false;
-      if (ONE_VIEW)
-        seen = rad1 > 0;
-      else if (g < n)
-        for (int v = 0; v < n_views && !seen; ++v) seen = proj.radius[(int64_t)v * n + g] > 0;
-      const uint32_t vmask = __ballot_sync(0xffffffffu, seen);
-      const float *src = P.sh + g0 * RW;
-      if (RW % 4 == 0 && vec) {   // rows of 3K floats, K = 4 or 16: whole float4s, none across rows
-        for (int f4 = lane; f4 < rows * RW / 4; f4 += 32) {
-          const int row = (4 * f4) / RW;
-          if (!((vmask >> row) & 1u)) continue;
-          const float4 x = reinterpret_cast<const float4 *>(src)[f4];
-          float *d = wsh + row * RP + (4 * f4) % RW;
-          d[0] = x.x; d[1] = x.y; d[2] = x.z; d[3] = x.w;
-        }
-      } else {
-        for (int f = lane; f < rows * RW; f += 32)
-          if ((vmask >> (f / RW)) & 1u) wsh[(f / RW) * RP + (f % RW)] = src[f];
+    // rows of Gaussians culled in every view are not read: their coefficients are
+    // never used and their gradient rows are zero
+    const uint32_t vmask = __ballot_sync(0xffffffffu, seen);
+    const float *src = P.sh + g0 * gw;
+    if (!WIDE && RW % 4 == 0 && vec) {   // rows of 3K floats, K = 4 or 16: whole float4s, none across rows
+      for (int f4 = lane; f4 < rows * RW / 4; f4 += 32) {
+        const int i = (4 * f4) / RW;
+        if (!((vmask >> i) & 1u)) continue;
+        const float4 x = reinterpret_cast<const float4 *>(src)[f4];
+        float *d = wsh + i * RP + (4 * f4) % RW;
+        d[0] = x.x; d[1] = x.y; d[2] = x.z; d[3] = x.w;
       }
-      __syncwarp();
+    } else if (WIDE && vec) {            // the float4s that the used coefficients reach into
+      for (int f4 = lane; f4 < rows * R4; f4 += 32) {
+        const int i = f4 / R4, c = 4 * (f4 - i * R4);
+        if (!((vmask >> i) & 1u)) continue;
+        const float4 x = *reinterpret_cast<const float4 *>(src + (int64_t)i * gw + c);
+        float *d = wsh + i * RP + c;
+        d[0] = x.x;
+        if (c + 1 < RW) d[1] = x.y;
+        if (c + 2 < RW) d[2] = x.z;
+        if (c + 3 < RW) d[3] = x.w;
+      }
+    } else {
+      for (int f = lane; f < rows * RW; f += 32)
+        if ((vmask >> (f / RW)) & 1u) wsh[(f / RW) * RP + (f % RW)] = src[(int64_t)(f / RW) * gw + (f % RW)];
     }
+    __syncwarp();
     if (g < n) {
-      const float *sh = STAGED ? wsh + lane * RP : P.sh + (int64_t)g * P.sh_stride * 3;
-      if (!IN_PLACE) {
-#pragma unroll
-        for (int k = 0; k < RW; ++k) dsh_row[k] = 0.f;
-      }
-      const float mx = ONE_VIEW ? mx1 : P.means[3 * g + 0], my = ONE_VIEW ? my1 : P.means[3 * g + 1],
-                  mz = ONE_VIEW ? mz1 : P.means[3 * g + 2];
       float dm0 = 0.f, dm1 = 0.f, dm2 = 0.f;
-      bool any = false;
+      float acc[ONE_VIEW ? 1 : RW];
+      if (!ONE_VIEW) {
+#pragma unroll
+        for (int k = 0; k < RW; ++k) acc[k] = 0.f;
+      }
       for (int v = 0; v < (ONE_VIEW ? 1 : n_views); ++v) {
-        const int64_t r = (int64_t)v * n + g;
-        if ((ONE_VIEW ? rad1 : proj.radius[r]) <= 0) continue;
-        any = true;
+        const int rad = rad1;
+        const float4 grgb = grgb1;
+        const uint8_t cl = cl1;
+        if (!ONE_VIEW && v + 1 < n_views) {
+          const int64_t r = (int64_t)(v + 1) * n + g;
+          rad1 = proj.radius[r];
+          grgb1 = reinterpret_cast<const float4 *>(rg.d_rgb)[r];
+          cl1 = proj.clamped[r];
+        }
+        if (rad <= 0) continue;
         const gs_camera_t &cam = cams[v];
-        const float4 grgb = ONE_VIEW ? grgb1 : reinterpret_cast<const float4 *>(rg.d_rgb)[r];
-        const uint8_t cl = ONE_VIEW ? cl1 : proj.clamped[r];
         const float g0c = (cl & 1) ? 0.f : grgb.x, g1c = (cl & 2) ? 0.f : grgb.y, g2c = (cl & 4) ? 0.f : grgb.z;
         float ccx, ccy, ccz;
         camera_centre(cam, ccx, ccy, ccz);
@@ -498,15 +513,15 @@ __global__ void __launch_bounds__(128, ONE_VIEW ? 8 : 4) project_bwd_sh_kernel(
         const float dxn = ex * il, dyn = ey * il, dzn = ez * il;
         float gdx = 0.f, gdy = 0.f, gdz = 0.f;
         sh_visit<DEG>(dxn, dyn, dzn, [&](int k, float Y, float yx, float yy, float yz) {
-          const float wk = g0c * sh[3 * k + 0] + g1c * sh[3 * k + 1] + g2c * sh[3 * k + 2];
-          if (IN_PLACE) {
-            dsh_row[3 * k + 0] = g0c * Y;
-            dsh_row[3 * k + 1] = g1c * Y;
-            dsh_row[3 * k + 2] = g2c * Y;
+          const float wk = g0c * row[3 * k + 0] + g1c * row[3 * k + 1] + g2c * row[3 * k + 2];
+          if (ONE_VIEW) {
+            row[3 * k + 0] = g0c * Y;
+            row[3 * k + 1] = g1c * Y;
+            row[3 * k + 2] = g2c * Y;
           } else {
-            dsh_row[3 * k + 0] += g0c * Y;
-            dsh_row[3 * k + 1] += g1c * Y;
-            dsh_row[3 * k + 2] += g2c * Y;
+            acc[ONE_VIEW ? 0 : 3 * k + 0] += g0c * Y;
+            acc[ONE_VIEW ? 0 : 3 * k + 1] += g1c * Y;
+            acc[ONE_VIEW ? 0 : 3 * k + 2] += g2c * Y;
           }
           gdx = fmaf(wk, yx, gdx);
           gdy = fmaf(wk, yy, gdy);
@@ -518,35 +533,45 @@ __global__ void __launch_bounds__(128, ONE_VIEW ? 8 : 4) project_bwd_sh_kernel(
         dm1 += (gdy - dd * dyn) * il;
         dm2 += (gdz - dd * dzn) * il;
       }
-      if (any) {
+      if (seen) {
         out.d_means[3 * g + 0] += dm0;
         out.d_means[3 * g + 1] += dm1;
         out.d_means[3 * g + 2] += dm2;
-      } else if (IN_PLACE) {
-#pragma unroll
-        for (int k = 0; k < RW; ++k) dsh_row[k] = 0.f;   // culled: zero gradient
       }
-      if (!STAGED) {
-        float *dsh = out.d_sh + (int64_t)g * P.sh_stride * 3;
+      if (!ONE_VIEW || !seen) {
 #pragma unroll
-        for (int k = 0; k < RW; ++k) dsh[k] = dsh_row[k];
-        for (int k = K; k < P.sh_stride; ++k) dsh[3 * k + 0] = dsh[3 * k + 1] = dsh[3 * k + 2] = 0.f;
+        for (int k = 0; k < RW; ++k) row[k] = ONE_VIEW ? 0.f : acc[ONE_VIEW ? 0 : k];   // culled: zero gradient
       }
     }
-    if (STAGED) {
-      __syncwarp();
-      float *dst = out.d_sh + g0 * RW;
-      const float *srow = IN_PLACE ? wsh : s_dsh + wib * 32 * RP;
-      if (RW % 4 == 0 && vec) {
-        for (int f4 = lane; f4 < rows * RW / 4; f4 += 32) {
-          const float *q = srow + ((4 * f4) / RW) * RP + (4 * f4) % RW;
-          reinterpret_cast<float4 *>(dst)[f4] = make_float4(q[0], q[1], q[2], q[3]);
+    __syncwarp();
+    float *dst = out.d_sh + g0 * gw;
+    if (!WIDE && RW % 4 == 0 && vec) {
+      for (int f4 = lane; f4 < rows * RW / 4; f4 += 32) {
+        const float *q = wsh + ((4 * f4) / RW) * RP + (4 * f4) % RW;
+        reinterpret_cast<float4 *>(dst)[f4] = make_float4(q[0], q[1], q[2], q[3]);
+      }
+    } else if (WIDE && vec) {
+      const int w4 = gw / 4, dr = 32 / w4, dc = 32 - dr * w4;   // a step of 32 float4s in rows and columns
+      int i = lane / w4, c = lane - i * w4;
+      for (int f4 = lane; f4 < rows * w4; f4 += 32) {
+        const float *q = wsh + i * RP + 4 * c;
+        const int left = RW - 4 * c;
+        reinterpret_cast<float4 *>(dst)[f4] = make_float4(left > 0 ? q[0] : 0.f, left > 1 ? q[1] : 0.f,
+                                                          left > 2 ? q[2] : 0.f, left > 3 ? q[3] : 0.f);
+        i += dr;
+        c += dc;
+        if (c >= w4) {
+          c -= w4;
+          ++i;
         }
-      } else {
-        for (int f = lane; f < rows * RW; f += 32) dst[f] = srow[(f / RW) * RP + (f % RW)];
       }
-      __syncwarp();
+    } else if (WIDE) {
+      for (int i = 0; i < rows; ++i)
+        for (int f = lane; f < gw; f += 32) dst[(int64_t)i * gw + f] = f < RW ? wsh[i * RP + f] : 0.f;
+    } else {
+      for (int f = lane; f < rows * RW; f += 32) dst[f] = wsh[(f / RW) * RP + (f % RW)];
     }
+    __syncwarp();
   }
 }
 
@@ -570,7 +595,7 @@ __global__ void densify_accum_kernel(const float *__restrict__ d_mean2d, const i
   }
 }
 
-template <int DEG, bool STAGED>
+template <int DEG, bool WIDE>
 static void launch_bwd_k(int grid, cudaStream_t s, const gs_params_t &P, const gs_frame_t *frame, const gs_proj_t &proj,
                          const gs_rec_grads_t &rg, const gs_param_grads_t &out, float *acc, int32_t *cnt) {
   if (frame->n_views == 1)
@@ -578,12 +603,14 @@ static void launch_bwd_k(int grid, cudaStream_t s, const gs_params_t &P, const g
   else
     project_bwd_geom_kernel<false><<<grid, 128, 0, s>>>(P, frame->cams_dev, frame->n_views, proj, rg, out, acc, cnt);
   count_launch();
-  // float4 staging needs both SH arrays on 16-byte boundaries (rows of 3K floats, K = 4 or 16)
-  const bool vec = (reinterpret_cast<uintptr_t>(P.sh) & 15u) == 0 && (reinterpret_cast<uintptr_t>(out.d_sh) & 15u) == 0;
+  // float4 staging needs both SH arrays on 16-byte boundaries, and so their rows (3 sh_stride
+  // floats; without WIDE the kernel itself leaves out K = 1 and 9)
+  const bool vec = (reinterpret_cast<uintptr_t>(P.sh) & 15u) == 0 && (reinterpret_cast<uintptr_t>(out.d_sh) & 15u) == 0 &&
+                   (!WIDE || P.sh_stride % 4 == 0);
   if (frame->n_views == 1)
-    project_bwd_sh_kernel<DEG, STAGED, true><<<grid, 128, 0, s>>>(P, frame->cams_dev, 1, proj, rg, out, vec);
+    project_bwd_sh_kernel<DEG, WIDE, true><<<grid, 128, 0, s>>>(P, frame->cams_dev, 1, proj, rg, out, vec);
   else
-    project_bwd_sh_kernel<DEG, STAGED, false><<<grid, 128, 0, s>>>(P, frame->cams_dev, frame->n_views, proj, rg, out,
+    project_bwd_sh_kernel<DEG, WIDE, false><<<grid, 128, 0, s>>>(P, frame->cams_dev, frame->n_views, proj, rg, out,
                                                                    vec);
 }
 
@@ -647,15 +674,15 @@ extern "C" gs_status_t gs_project_bwd(const gs_params_t *params, const gs_frame_
   const int grid = grid_for(params->n, 128);
   cudaStream_t s = as_stream(stream);
   const int K = (params->sh_degree + 1) * (params->sh_degree + 1);
-  const bool staged = params->sh_stride == K;
+  const bool wide = params->sh_stride > K;
   switch (params->sh_degree) {
-    case 0: staged ? launch_bwd_k<0, true>(grid, s, *params, frame, *proj, *rg, *out, densify_accum, densify_count)
+    case 0: wide ? launch_bwd_k<0, true>(grid, s, *params, frame, *proj, *rg, *out, densify_accum, densify_count)
                   : launch_bwd_k<0, false>(grid, s, *params, frame, *proj, *rg, *out, densify_accum, densify_count); break;
-    case 1: staged ? launch_bwd_k<1, true>(grid, s, *params, frame, *proj, *rg, *out, densify_accum, densify_count)
+    case 1: wide ? launch_bwd_k<1, true>(grid, s, *params, frame, *proj, *rg, *out, densify_accum, densify_count)
                   : launch_bwd_k<1, false>(grid, s, *params, frame, *proj, *rg, *out, densify_accum, densify_count); break;
-    case 2: staged ? launch_bwd_k<2, true>(grid, s, *params, frame, *proj, *rg, *out, densify_accum, densify_count)
+    case 2: wide ? launch_bwd_k<2, true>(grid, s, *params, frame, *proj, *rg, *out, densify_accum, densify_count)
                   : launch_bwd_k<2, false>(grid, s, *params, frame, *proj, *rg, *out, densify_accum, densify_count); break;
-    default: staged ? launch_bwd_k<3, true>(grid, s, *params, frame, *proj, *rg, *out, densify_accum, densify_count)
+    default: wide ? launch_bwd_k<3, true>(grid, s, *params, frame, *proj, *rg, *out, densify_accum, densify_count)
                   : launch_bwd_k<3, false>(grid, s, *params, frame, *proj, *rg, *out, densify_accum, densify_count); break;
   }
   GS_LAUNCH_CHECK();

@@ -161,3 +161,43 @@ def test_project_vjp_clamped_colour_and_fov_clamp():
     want = opipe.project_vjp(p, 0, [cam], [g])
     for k in R.PARAM_KEYS:
         assert rel_l2(out[k].cpu().numpy(), want[k]) < 1e-4, k
+
+
+@pytest.mark.parametrize("degree", [0, 1, 2])
+@pytest.mark.parametrize("views", [1, 3])
+@pytest.mark.parametrize("stored,shift", [(16, 0), (16, 1), (11, 0)])
+@pytest.mark.parametrize("n", [1, 33, 1000])
+def test_project_vjp_of_rows_wider_than_the_degree(n, stored, shift, views, degree):
+    """SH rows that store more coefficients than the degree uses, on 16-byte boundaries or not
+    (shift: one float off) and of widths that are no multiple of four: bit for bit the
+    gradients of exact rows, and zeros beyond them. The exact rows against the oracle."""
+    K = (degree + 1) ** 2
+    sc = scene("orbit_small")
+    cams = [synth.orbit_camera(4.0, 0.3 + 1.9 * v, 15.0, 200 - 40 * v, 150, 180.0) for v in range(views)]
+    sub = {k: np.ascontiguousarray(v[:n]) for k, v in sc.params().items()}
+    exact = dict(sub, sh=np.ascontiguousarray(sub["sh"][:, :K]))
+    frame = R.Frame(cams)
+    P = {k: torch.as_tensor(v).cuda() for k, v in exact.items()}
+    proj = R.project(P, degree, frame)
+    rng = np.random.default_rng(n + degree)
+    gs = [{k: v.astype(np.float32) for k, v in _rand_rec_grads(rng, n).items()} for _ in cams]
+    rec = _rec_grads_gpu(gs)
+    want = R.project_bwd(P, degree, frame, proj, rec)
+    oracle = opipe.project_vjp(exact, degree, cams, gs)
+    for k in R.PARAM_KEYS:
+        w = oracle[k]
+        assert np.linalg.norm(want[k].cpu().numpy() - w) <= 1e-4 * np.linalg.norm(w) + 1e-30, k
+
+    def placed(value):
+        flat = torch.full((n * stored * 3 + 1,), value, device="cuda")
+        return flat[shift:shift + n * stored * 3].view(n, stored, 3)
+
+    wide = dict(P, sh=placed(7.0))
+    wide["sh"][:, :K] = P["sh"]
+    out = {k: torch.empty_like(P[k]) for k in R.PARAM_KEYS}
+    out["sh"] = placed(5.0)
+    R.project_bwd(wide, degree, frame, proj, rec, out=out)
+    for k in R.PARAM_KEYS:
+        got = out[k][:, :K] if k == "sh" else out[k]
+        assert torch.equal(got, want[k]), k
+    assert not out["sh"][:, K:].any()
