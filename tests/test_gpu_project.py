@@ -201,3 +201,23 @@ def test_project_vjp_of_rows_wider_than_the_degree(n, stored, shift, views, degr
         got = out[k][:, :K] if k == "sh" else out[k]
         assert torch.equal(got, want[k]), k
     assert not out["sh"][:, K:].any()
+
+
+@pytest.mark.parametrize("degree,stored", [(0, 1), (1, 4), (2, 9), (2, 16), (3, 16)])
+@pytest.mark.parametrize("n", [1, 127, 3000])
+def test_project_of_several_views_equals_each_view(n, degree, stored):
+    """A frame of several views (of different sizes, some Gaussians behind or outside some of
+    them) against frames of one view, bit for bit: both evaluate the same expressions."""
+    sc = scene("orbit_small")
+    sub = {k: np.ascontiguousarray(v[:n]) for k, v in sc.params().items()}
+    sub["sh"] = np.ascontiguousarray(sub["sh"][:, :stored])
+    P = {k: torch.as_tensor(v).cuda() for k, v in sub.items()}
+    cams = [synth.orbit_camera(4.0 - v, 0.3 + 1.9 * v, 15.0, 200 - 40 * v, 150, 180.0) for v in range(4)]
+    got = R.project(P, degree, R.Frame(cams))
+    seen = 0
+    for v, cam in enumerate(cams):
+        want = R.project(P, degree, R.Frame([cam]))
+        seen += int((want.radius > 0).sum())
+        for k in ("mean2d", "conic_opacity", "rgb", "depth", "radius", "rect", "clamped"):
+            assert torch.equal(getattr(got, k)[v * n:(v + 1) * n], getattr(want, k)), (v, k)
+    assert n < 100 or n < seen < 4 * n
