@@ -35,7 +35,8 @@ struct SelectState {      // scratch of the selection (lives in the caller's wor
   unsigned long long n_keep;   // count after pruning
   uint32_t prefix;             // radix-select prefix of the k-th key
   uint32_t k_rem;              // rank still to find inside the current bucket
-  uint32_t pad[2];
+  uint32_t done;               // blocks of the current kernel that have finished
+  uint32_t pad;
   uint32_t hist[256];
 };
 
@@ -52,11 +53,62 @@ __device__ __forceinline__ void block_add_u64(unsigned long long x, unsigned lon
   }
 }
 
+// The last block to get here (every block of the grid calls it once, with all its results
+// added to the state) goes on with what follows a grid-wide sum, in place of a launch.
+__device__ __forceinline__ bool last_block(SelectState *st) {
+  __shared__ bool s_last;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) s_last = atomicAdd(&st->done, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!s_last) return false;
+  __threadfence();
+  if (threadIdx.x == 0) st->done = 0;
+  return true;
+}
+
+// One block: the bucket of the byte at `shift` that holds rank k_rem, thread b on bucket b (a
+// single thread walking the buckets took 8 us a byte); clears the histogram.
+__device__ __forceinline__ void kth_find(int shift, double ratio, SelectState *st) {
+  static_assert(kSelThreads == 256, "a thread per bucket");
+  const uint32_t b = threadIdx.x;
+  const uint32_t c = __ldcg(&st->hist[b]);
+  uint32_t k;
+  if (shift == 24) {
+    const unsigned long long N = __ldcg(&st->n_post);
+    unsigned long long r = (unsigned long long)floor((double)N * ratio);
+    if (r > N - 1) r = N - 1;
+    k = (uint32_t)r;
+  } else {
+    k = st->k_rem;
+  }
+  const uint32_t prefix = shift == 24 ? 0u : st->prefix;
+  uint32_t all;
+  const uint32_t before = block_exclusive_scan<uint32_t>(c, &all);
+  st->hist[b] = 0;
+  // the first bucket that k falls into; the last one if it falls into none
+  if ((k >= before && k - before < c) || (b == 255 && k >= all)) {
+    st->k_rem = k - before;
+    st->prefix = prefix | b << shift;
+  }
+  __syncthreads();
+}
+
+__device__ __forceinline__ float tau_of(const gs_densify_cfg_t &cfg, const SelectState *st) {
+  return cfg.prune_adaptive ? fminf(from_ordered_bits(st->prefix), cfg.prune_upper_logit) : cfg.prune_logit;
+}
+
+// Masks and the post-densification count; for adaptive pruning also the first step of the
+// radix select (the highest byte's histogram, weighted by multiplicity, and its bucket).
 __global__ void __launch_bounds__(kSelThreads) select_kernel(gs_densify_cfg_t cfg, const float *__restrict__ log_scales,
+                                                             const float *__restrict__ logits,
                                                              const float *__restrict__ accum,
                                                              const int32_t *__restrict__ count, int64_t n,
                                                              uint8_t *__restrict__ split, uint8_t *__restrict__ clone,
-                                                             SelectState *st) {
+                                                             SelectState *st, float *tau) {
+  __shared__ uint32_t h[256];
+  h[threadIdx.x] = 0;
+  __syncthreads();
   unsigned long long post = 0;
   for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < n; g += (int64_t)gridDim.x * blockDim.x) {
     const int32_t c = count[g];
@@ -73,58 +125,42 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(gs_densify_cfg_t cf
     }
     split[g] = sp;
     clone[g] = cl;
-    post += (sp || cl) ? 2 : 1;
+    const uint32_t w = (sp || cl) ? 2u : 1u;
+    post += w;
+    if (cfg.prune_adaptive) atomicAdd(&h[ordered_bits(logits[g]) >> 24], w);
   }
   block_add_u64(post, &st->n_post);
+  __syncthreads();
+  if (h[threadIdx.x]) atomicAdd(&st->hist[threadIdx.x], h[threadIdx.x]);
+  if (!last_block(st)) return;
+  if (cfg.prune_adaptive)
+    kth_find(24, cfg.prune_ratio, st);
+  else if (threadIdx.x == 0)
+    *tau = tau_of(cfg, st);
 }
 
 // Radix select, most significant byte first: histogram of the current byte over
-// the keys that match the prefix found so far, weighted by multiplicity.
-__global__ void __launch_bounds__(kSelThreads) kth_hist_kernel(const float *__restrict__ logits,
+// the keys that match the prefix found so far, weighted by multiplicity, and its bucket; after
+// the last byte the threshold.
+__global__ void __launch_bounds__(kSelThreads) kth_hist_kernel(gs_densify_cfg_t cfg, const float *__restrict__ logits,
                                                                const uint8_t *__restrict__ split,
                                                                const uint8_t *__restrict__ clone, int64_t n,
-                                                               int shift, SelectState *st) {
+                                                               int shift, SelectState *st, float *tau) {
   __shared__ uint32_t h[256];
-  for (int i = threadIdx.x; i < 256; i += blockDim.x) h[i] = 0;
+  h[threadIdx.x] = 0;
   __syncthreads();
   const uint32_t prefix = st->prefix;
-  const uint32_t hi_mask = shift >= 24 ? 0u : (0xffffffffu << (shift + 8));
+  const uint32_t hi_mask = 0xffffffffu << (shift + 8);
   for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < n; g += (int64_t)gridDim.x * blockDim.x) {
     const uint32_t key = ordered_bits(logits[g]);
     if ((key & hi_mask) != (prefix & hi_mask)) continue;
     atomicAdd(&h[(key >> shift) & 0xffu], (split[g] | clone[g]) ? 2u : 1u);
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < 256; i += blockDim.x)
-    if (h[i]) atomicAdd(&st->hist[i], h[i]);
-}
-
-__global__ void kth_find_kernel(int shift, double ratio, SelectState *st) {
-  // single thread: walk the 256 buckets to the one holding rank k_rem
-  if (threadIdx.x != 0) return;
-  if (shift == 24) {
-    const unsigned long long N = st->n_post;
-    unsigned long long k = (unsigned long long)floor((double)N * ratio);
-    if (k > N - 1) k = N - 1;
-    st->k_rem = (uint32_t)k;
-    st->prefix = 0;
-  }
-  uint32_t k = st->k_rem, b = 0;
-  for (; b < 255; ++b) {
-    const uint32_t c = st->hist[b];
-    if (k < c) break;
-    k -= c;
-  }
-  st->k_rem = k;
-  st->prefix |= b << shift;
-  for (int i = 0; i < 256; ++i) st->hist[i] = 0;
-}
-
-__global__ void tau_kernel(gs_densify_cfg_t cfg, SelectState *st, float *tau) {
-  if (threadIdx.x != 0) return;
-  float t = cfg.prune_logit;
-  if (cfg.prune_adaptive) t = fminf(from_ordered_bits(st->prefix), cfg.prune_upper_logit);
-  *tau = t;
+  if (h[threadIdx.x]) atomicAdd(&st->hist[threadIdx.x], h[threadIdx.x]);
+  if (!last_block(st)) return;
+  kth_find(shift, cfg.prune_ratio, st);
+  if (shift == 0 && threadIdx.x == 0) *tau = tau_of(cfg, st);
 }
 
 __global__ void __launch_bounds__(kSelThreads) count_keep_kernel(const float *__restrict__ logits,
@@ -139,31 +175,102 @@ __global__ void __launch_bounds__(kSelThreads) count_keep_kernel(const float *__
     c += split[g] ? 2 : (clone[g] ? 2 : 1);
   }
   block_add_u64(c, &st->n_keep);
-}
-
-__global__ void publish_kernel(SelectState *st, int64_t *d_new_n) {
-  if (threadIdx.x == 0) *d_new_n = (int64_t)st->n_keep;
+  if (last_block(st) && threadIdx.x == 0) *d_new_n = (int64_t)__ldcg(&st->n_keep);
 }
 
 // ------------------------------------------------------------------ compaction
-struct SectionFlag {
+// Positions of the three sections (survivors: kept, not split; clones; split parents) from one
+// reduce-then-scan over all three flags, which reads the logits and masks twice in three
+// launches (a scan per section read them six times in nine: 47 -> 17 us at 1.2M).
+struct Sections {
   const float *logits;
   const uint8_t *split, *clone;
   const float *tau;
   int64_t n;
-  int kind;                // 0: survivor (kept, not split), 1: clone, 2: split parent
-  uint32_t *pos;
-  uint32_t *total_out;
-  __device__ uint64_t count() const { return (uint64_t)n; }
-  __device__ uint32_t value(uint64_t g) const {
-    if (logits[g] < *tau) return 0u;
-    if (kind == 0) return split[g] ? 0u : 1u;
-    if (kind == 1) return clone[g] ? 1u : 0u;
-    return split[g] ? 1u : 0u;
+  uint32_t *pos[3], *totals;
+  __device__ __forceinline__ uint3 flags(int64_t g) const {
+    if (logits[g] < *tau) return make_uint3(0u, 0u, 0u);
+    const uint32_t sp = split[g] ? 1u : 0u;
+    return make_uint3(1u - sp, clone[g] ? 1u : 0u, sp);
   }
-  __device__ void emit(uint64_t g, uint64_t pre, uint32_t) const { pos[g] = (uint32_t)pre; }
-  __device__ void total(uint64_t t) const { *total_out = (uint32_t)t; }
 };
+
+__device__ __forceinline__ uint3 add3(uint3 a, uint3 b) { return make_uint3(a.x + b.x, a.y + b.y, a.z + b.z); }
+
+// Exclusive sums over the block (kScanThreads threads) of three counts; *total: the block's.
+__device__ __forceinline__ uint3 block_exclusive_scan3(uint3 x, uint3 *total) {
+  uint3 r;
+  r.x = block_exclusive_scan<uint32_t>(x.x, &total->x);
+  r.y = block_exclusive_scan<uint32_t>(x.y, &total->y);
+  r.z = block_exclusive_scan<uint32_t>(x.z, &total->z);
+  return r;
+}
+
+__global__ void __launch_bounds__(kScanThreads) sections_reduce_kernel(Sections f, uint3 *sums) {
+  uint64_t begin, end;
+  chunk_of((uint64_t)f.n, gridDim.x, kScanTile, begin, end);
+  uint3 x = make_uint3(0u, 0u, 0u), all;
+#pragma unroll 4
+  for (uint64_t i = begin + threadIdx.x; i < end; i += kScanThreads) x = add3(x, f.flags((int64_t)i));
+  block_exclusive_scan3(x, &all);
+  if (threadIdx.x == 0) sums[blockIdx.x] = all;
+}
+
+// One block of 1024 threads: the blocks' sums to exclusive prefixes (G <= 1024).
+__global__ void __launch_bounds__(1024) sections_top_kernel(Sections f, uint3 *sums, int G) {
+  const int t = threadIdx.x;
+  uint3 all;
+  const uint3 pre = block_exclusive_scan3(t < G ? sums[t] : make_uint3(0u, 0u, 0u), &all);
+  if (t < G) sums[t] = pre;
+  if (t == 0) {
+    f.totals[0] = all.x;
+    f.totals[1] = all.y;
+    f.totals[2] = all.z;
+  }
+}
+
+__global__ void __launch_bounds__(kScanThreads) sections_down_kernel(Sections f, const uint3 *__restrict__ sums) {
+  uint64_t begin, end;
+  chunk_of((uint64_t)f.n, gridDim.x, kScanTile, begin, end);
+  uint3 run = sums[blockIdx.x];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  __shared__ uint3 s_warp[kScanThreads / 32];
+  const uint32_t lt = lanemask_lt();
+  // a warp takes 256 consecutive Gaussians, 32 at a time: coalesced, ranks by ballot
+  for (uint64_t tile = begin; tile < end; tile += kScanTile) {
+    const uint64_t w0 = tile + (uint64_t)warp * (32 * kScanItems);
+    uint32_t bs[kScanItems], bc[kScanItems], bp[kScanItems];
+    uint3 own = make_uint3(0u, 0u, 0u);
+#pragma unroll
+    for (int j = 0; j < kScanItems; ++j) {
+      const uint64_t i = w0 + 32 * j + lane;
+      const uint3 x = i < end ? f.flags((int64_t)i) : make_uint3(0u, 0u, 0u);
+      bs[j] = __ballot_sync(0xffffffffu, x.x);
+      bc[j] = __ballot_sync(0xffffffffu, x.y);
+      bp[j] = __ballot_sync(0xffffffffu, x.z);
+      own = add3(own, make_uint3(__popc(bs[j]), __popc(bc[j]), __popc(bp[j])));
+    }
+    if (lane == 0) s_warp[warp] = own;
+    __syncthreads();
+    uint3 at = run;
+#pragma unroll
+    for (int w = 0; w < kScanThreads / 32; ++w) {
+      if (w < warp) at = add3(at, s_warp[w]);
+      run = add3(run, s_warp[w]);
+    }
+#pragma unroll
+    for (int j = 0; j < kScanItems; ++j) {
+      const uint64_t i = w0 + 32 * j + lane;
+      if (i < end) {
+        f.pos[0][i] = at.x + __popc(bs[j] & lt);
+        f.pos[1][i] = at.y + __popc(bc[j] & lt);
+        f.pos[2][i] = at.z + __popc(bp[j] & lt);
+      }
+      at = add3(at, make_uint3(__popc(bs[j]), __popc(bc[j]), __popc(bp[j])));
+    }
+    __syncthreads();
+  }
+}
 
 constexpr int kMaxExtra = 16;
 struct ExtraList {
@@ -387,7 +494,7 @@ __global__ void __launch_bounds__(kScatThreads) scatter_kernel(
 struct DensWs {
   SelectState *st;
   uint32_t *pos_s, *pos_c, *pos_p, *totals;
-  uint64_t *block_sums;
+  uint3 *block_sums;
   size_t bytes;
 };
 
@@ -407,7 +514,7 @@ static DensWs dens_layout(void *base, int64_t n) {
   w.pos_c = (uint32_t *)take(4 * (size_t)n + 16);
   w.pos_p = (uint32_t *)take(4 * (size_t)n + 16);
   w.totals = (uint32_t *)take(16);
-  w.block_sums = (uint64_t *)take(8 * kMaxBlocks);
+  w.block_sums = (uint3 *)take(sizeof(uint3) * kMaxBlocks);
   w.bytes = off;
   return w;
 }
@@ -416,6 +523,26 @@ static int dgrid(int64_t n) {
   int64_t g = (n + kSelThreads - 1) / kSelThreads;
   const int64_t cap = (int64_t)num_sms() * 8;
   return (int)(g < 1 ? 1 : (g > cap ? cap : g));
+}
+
+// The selection on a cleared state: masks, then for adaptive pruning the threshold byte by byte,
+// then the new count. What follows each grid-wide sum is done by the kernel's last block:
+// five launches for adaptive pruning (thirteen with one for every such step: 80 -> 54 us at 1.2M).
+static gs_status_t select_launches(const gs_densify_cfg_t &cfg, const float *log_scales, const float *logits,
+                                   const float *accum, const int32_t *count, int64_t n, uint8_t *split, uint8_t *clone,
+                                   float *tau, int64_t *d_new_n, SelectState *st, cudaStream_t s) {
+  const int G = dgrid(n);
+  select_kernel<<<G, kSelThreads, 0, s>>>(cfg, log_scales, logits, accum, count, n, split, clone, st, tau);
+  GS_LAUNCH_CHECK();
+  if (cfg.prune_adaptive) {
+    for (int shift = 16; shift >= 0; shift -= 8) {
+      kth_hist_kernel<<<G, kSelThreads, 0, s>>>(cfg, logits, split, clone, n, shift, st, tau);
+      GS_LAUNCH_CHECK();
+    }
+  }
+  count_keep_kernel<<<G, kSelThreads, 0, s>>>(logits, split, clone, n, tau, st, d_new_n);
+  GS_LAUNCH_CHECK();
+  return GS_OK;
 }
 
 }  // namespace gs
@@ -441,24 +568,7 @@ extern "C" gs_status_t gs_densify_select(const gs_densify_cfg_t *cfg, const floa
   if (ws_bytes < w.bytes) return GS_ERR_INVALID_ARG;
   cudaStream_t s = as_stream(stream);
   GS_CUDA_TRY(cudaMemsetAsync(w.st, 0, sizeof(SelectState), s));
-  const int G = dgrid(n);
-  select_kernel<<<G, kSelThreads, 0, s>>>(*cfg, log_scales, accum, count, n, split, clone, w.st);
-  GS_LAUNCH_CHECK();
-  if (cfg->prune_adaptive) {
-    for (int shift = 24; shift >= 0; shift -= 8) {
-      kth_hist_kernel<<<G, kSelThreads, 0, s>>>(opacity_logits, split, clone, n, shift, w.st);
-      GS_LAUNCH_CHECK();
-      kth_find_kernel<<<1, 32, 0, s>>>(shift, cfg->prune_ratio, w.st);
-      GS_LAUNCH_CHECK();
-    }
-  }
-  tau_kernel<<<1, 32, 0, s>>>(*cfg, w.st, d_tau_logit);
-  GS_LAUNCH_CHECK();
-  count_keep_kernel<<<G, kSelThreads, 0, s>>>(opacity_logits, split, clone, n, d_tau_logit, w.st, d_new_n);
-  GS_LAUNCH_CHECK();
-  publish_kernel<<<1, 32, 0, s>>>(w.st, d_new_n);
-  GS_LAUNCH_CHECK();
-  return GS_OK;
+  return select_launches(*cfg, log_scales, opacity_logits, accum, count, n, split, clone, d_tau_logit, d_new_n, w.st, s);
 }
 
 extern "C" gs_status_t gs_densify_apply(const gs_densify_cfg_t *cfg, const gs_params_t *in, const uint8_t *split,
@@ -492,11 +602,13 @@ extern "C" gs_status_t gs_densify_apply(const gs_densify_cfg_t *cfg, const gs_pa
   }
   cudaStream_t s = as_stream(stream);
   const int G = scan_blocks();
-  for (int kind = 0; kind < 3; ++kind) {
-    uint32_t *pos = kind == 0 ? w.pos_s : (kind == 1 ? w.pos_c : w.pos_p);
-    SectionFlag f{in->opacity_logits, split, clone, d_tau_logit, in->n, kind, pos, w.totals + kind};
-    if (gs_status_t st = run_scan(f, w.block_sums, G, s)) return st;
-  }
+  const Sections sec{in->opacity_logits, split, clone, d_tau_logit, in->n, {w.pos_s, w.pos_c, w.pos_p}, w.totals};
+  sections_reduce_kernel<<<G, kScanThreads, 0, s>>>(sec, w.block_sums);
+  GS_LAUNCH_CHECK();
+  sections_top_kernel<<<1, 1024, 0, s>>>(sec, w.block_sums, G);
+  GS_LAUNCH_CHECK();
+  sections_down_kernel<<<G, kScanThreads, 0, s>>>(sec, w.block_sums);
+  GS_LAUNCH_CHECK();
   int sg = (int)((in->n + 32 * (kScatThreads / 32) - 1) / (32 * (kScatThreads / 32)));
   // at most the blocks the device keeps resident: with more, a second partial wave
   // of the grid-stride loop runs on a part of the GPU
@@ -565,22 +677,5 @@ extern "C" gs_status_t gs_densify_select_static(const gs_densify_cfg_t *cfg, con
   cudaStream_t s = as_stream(stream);
   // the previous call's contents are still there: clear the counters and histogram
   GS_CUDA_TRY(cudaMemsetAsync(st, 0, sizeof(SelectState), s));
-  const int G = dgrid(n);
-  select_kernel<<<G, kSelThreads, 0, s>>>(*cfg, log_scales, accum, count, n, split, clone, st);
-  GS_LAUNCH_CHECK();
-  if (cfg->prune_adaptive) {
-    for (int shift = 24; shift >= 0; shift -= 8) {
-      kth_hist_kernel<<<G, kSelThreads, 0, s>>>(opacity_logits, split, clone, n, shift, st);
-      GS_LAUNCH_CHECK();
-      kth_find_kernel<<<1, 32, 0, s>>>(shift, cfg->prune_ratio, st);
-      GS_LAUNCH_CHECK();
-    }
-  }
-  tau_kernel<<<1, 32, 0, s>>>(*cfg, st, d_tau_logit);
-  GS_LAUNCH_CHECK();
-  count_keep_kernel<<<G, kSelThreads, 0, s>>>(opacity_logits, split, clone, n, d_tau_logit, st, d_new_n);
-  GS_LAUNCH_CHECK();
-  publish_kernel<<<1, 32, 0, s>>>(st, d_new_n);
-  GS_LAUNCH_CHECK();
-  return GS_OK;
+  return select_launches(*cfg, log_scales, opacity_logits, accum, count, n, split, clone, d_tau_logit, d_new_n, st, s);
 }

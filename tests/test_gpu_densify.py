@@ -122,3 +122,41 @@ def test_densify_apply_capacity_overflow():
     out, ex, got_n, err = R.densify_apply(cfg, P, 1, split, clone, tau, need - 1, ws=ws)
     torch.cuda.synchronize()
     assert int(err.item()) == 2 and int(got_n.item()) == need
+
+
+@pytest.mark.parametrize("n", [1, 2, 33, 255, 257, 2047, 2049, 300_001])
+@pytest.mark.parametrize("ratio", [None, 1e-6, 0.03, 0.999])
+@pytest.mark.parametrize("equal", [False, True])
+def test_densify_event_at_block_edges(n, ratio, equal):
+    """Selection and compaction at the edges of their warps (32), blocks (256) and scan tiles
+    (2048), with the threshold's rank first, inside and last, and all logits equal."""
+    p, accum, count, thr_s = _select_inputs(11, max(n, 200))
+    p = {k: np.ascontiguousarray(v[:n]) for k, v in p.items()}
+    accum, count = accum[:n].copy(), count[:n].copy()
+    if equal:
+        p["opacity_logits"][:] = np.float32(-0.75)
+    P = {k: torch.as_tensor(v).cuda() for k, v in p.items()}
+    kw = dict(prune_ratio=ratio, prune_upper_logit=np.float32(3.0)) if ratio else \
+        dict(prune_logit=oden.logit_threshold(0.3))
+    cfg = R.densify_cfg(mode=0, log_scale_threshold=thr_s, seed=77, event=3, **kw)
+    acc, cnt = torch.as_tensor(accum).cuda(), torch.as_tensor(count).cuda()
+    split, clone, tau, new_n, ws = R.densify_select(cfg, P, acc, cnt)
+    ws_, wc = oden.select(accum, count, p["log_scales"], 0, np.float32(2e-4), thr_s)
+    assert np.array_equal(split.cpu().numpy().astype(bool), ws_) and np.array_equal(clone.cpu().numpy().astype(bool), wc)
+    want_tau = oden.prune_threshold(p["opacity_logits"], ws_, wc, p=ratio, tau_u=1 / (1 + math.exp(-3.0))) if ratio \
+        else oden.prune_threshold(p["opacity_logits"], ws_, wc, fixed_tau=0.3)
+    assert abs(float(tau.item()) - float(want_tau)) <= 1e-6 * abs(float(want_tau))   # tau_u's logit rounds either way
+    idx = np.where(p["opacity_logits"] < np.float32(tau.item()), 0, 1 + (ws_ | wc))
+    assert int(new_n.item()) == idx.sum()
+    cap = max(1, int(new_n.item()))
+    m1 = np.arange(n * 4, dtype=np.float32).reshape(n, 4)
+    out, ex, got_n, err = R.densify_apply(cfg, P, 1, split, clone, tau, cap, extra={"m1": torch.as_tensor(m1).cuda()},
+                                          ws=ws)
+    want, wex, _ = oden.apply(p, ws_, wc, np.float32(tau.item()), 77, 3, extra={"m1": m1})
+    k = int(got_n.item())
+    assert int(err.item()) == 0 and k == idx.sum() == len(want["means"])
+    for key in ("log_scales", "quats", "opacity_logits", "sh"):
+        assert np.array_equal(out[key][:k].cpu().numpy(), want[key]), key
+    assert np.array_equal(ex["m1"][:k].cpu().numpy(), wex["m1"])
+    if k:
+        assert np.abs(out["means"][:k].cpu().numpy() - want["means"]).max() < 1e-5
