@@ -417,25 +417,42 @@ __global__ void __launch_bounds__(kDirThreads) direct_order_kernel(const DirArgs
   const int64_t seg = (int64_t)v * a.n;
   uint32_t *weights = a.weights + (int64_t)v * a.groups;
   const int t = threadIdx.x;
-  __shared__ uint32_t s_w[kDirWarps];
-  for (uint32_t g = b; g < ng; g += blocks_per_view) {
-    const uint32_t k = g * kDirThreads + t;
-    uint32_t w = 0;
-    if (k < nv) {
-      const uint32_t off = a.v1[seg + k];
-      const uint2 h = GS_CHECK(off < a.unit_cap, 4, off) ? a.units[off] : make_uint2(0u, 0u);
-      a.ordered[seg + k] = make_uint2(off, h.y >> 16);
-      a.k1[seg + k] = h.x;
-      w = (h.y & 0xffffu) + kRecordWeight;
+  // four groups a turn: a record's header is a gather from a random place, and with one group the
+  // block waited out a round trip per record (20M records, 15M of them visible: 319 -> 289 us; 12 views
+  // 73 -> 58)
+  constexpr int kTurn = 4;
+  __shared__ uint32_t s_w[kTurn][kDirWarps];
+  for (uint32_t g = kTurn * b; g < ng; g += kTurn * blocks_per_view) {
+    uint32_t off[kTurn];
+    uint2 h[kTurn];
+#pragma unroll
+    for (int i = 0; i < kTurn; ++i) {
+      const uint32_t k = (g + i) * kDirThreads + t;
+      off[i] = k < nv ? a.v1[seg + k] : 0u;
     }
-    w = __reduce_add_sync(0xffffffffu, w);
-    if ((t & 31) == 0) s_w[t >> 5] = w;
+#pragma unroll
+    for (int i = 0; i < kTurn; ++i) {
+      const bool on = (g + i) * kDirThreads + t < nv;
+      h[i] = on && GS_CHECK(off[i] < a.unit_cap, 4, off[i]) ? a.units[off[i]] : make_uint2(0u, 0u);
+    }
+#pragma unroll
+    for (int i = 0; i < kTurn; ++i) {
+      const uint32_t k = (g + i) * kDirThreads + t;
+      uint32_t w = 0;
+      if (k < nv) {
+        a.ordered[seg + k] = make_uint2(off[i], h[i].y >> 16);
+        a.k1[seg + k] = h[i].x;
+        w = (h[i].y & 0xffffu) + kRecordWeight;
+      }
+      w = __reduce_add_sync(0xffffffffu, w);
+      if ((t & 31) == 0) s_w[i][t >> 5] = w;
+    }
     __syncthreads();
-    if (t == 0) {
+    if (t < kTurn && g + t < ng) {
       uint32_t sum = 0;
 #pragma unroll
-      for (int i = 0; i < kDirWarps; ++i) sum += s_w[i];
-      weights[g] = sum;
+      for (int i = 0; i < kDirWarps; ++i) sum += s_w[t][i];
+      weights[g + t] = sum;
     }
     __syncthreads();
   }
@@ -934,7 +951,7 @@ inline size_t dir_ws_bound(int64_t R, int64_t cap) {
   p.unit_grid = kUnitBlocks * num_sms();
   const DirWs w = dir_layout(nullptr, R, cap, kDirMaxViews, kDirMatrix, p);
   return w.bytes + 4 * (size_t)kDirPasses * 256 * ((size_t)R / kDirTile + kDirMaxViews + 1) +
-         4 * ((size_t)R / kDirThreads + 8 * (size_t)num_sms() + 4 * kDirMaxViews) + 1024;
+         4 * ((size_t)R / kDirThreads + 16 * (size_t)num_sms() + 4 * kDirMaxViews) + 1024;
 }
 
 inline gs_status_t dir_bin_sort(const gs_proj_t *proj, const gs_frame_t *f, gs_bins_t *bins, void *ws, size_t ws_bytes,

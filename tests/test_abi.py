@@ -169,3 +169,21 @@ def test_debug_status_entry_point(lib):
     dbg = _abi.load(gbuild.build(debug=True))
     missing = [n for n in declared_functions() if not hasattr(dbg, n)]
     assert not missing, missing
+
+
+def test_bin_sort_workspace_without_a_frame_is_enough_for_any():
+    """gs_bin_sort_workspace_size(NULL frame) against frames of one to many views, few to
+    many tiles, on both binning paths."""
+    lib = _abi.load()
+    for n_views, w, h, tile in [(1, 16, 16, 16), (1, 1246, 826, 16), (12, 623, 413, 16), (4, 1600, 1060, 8),
+                                (1000, 64, 48, 8), (1025, 64, 48, 8), (1, 20000, 20000, 8), (300, 1920, 1080, 16)]:
+        cams = (_abi.GsCamera * n_views)()
+        for c in cams:
+            c.fx = c.fy = 100.0
+            c.width, c.height, c.near_plane = w, h, 0.2
+        fr = _abi.GsFrame()
+        assert lib.gs_frame_init(cams, n_views, tile, tile, C.byref(fr)) == 0
+        for n in (0, 1, 1000, 100_000):
+            for cap in (0, 1, 5_000_000):
+                size = lib.gs_bin_sort_workspace_size(n * n_views, cap, C.byref(fr))
+                assert 0 < size <= lib.gs_bin_sort_workspace_size(n * n_views, cap, None), (n_views, w, n, cap)
