@@ -170,7 +170,7 @@ __device__ __forceinline__ int warp_select(const float4 *s_rgb, int cnt, int war
 // entries at a time. Lane l gathers entry base + l, tests it against the warp's
 // 8x8 block (the ellipse's x-extent over the block's rows against its columns); the
 // passing entries are closed up in the warp's shared slots and composited in list
-// order, two per turn of the loop. A warp leaves as soon as its 64 pixels have
+// order, U per turn of the loop. A warp leaves as soon as its 64 pixels have
 // stopped, so neither barriers nor finished neighbours hold it (one-warp CTAs,
 // which also free a finished warp's slot, measured no faster).
 struct FwdArgs {
@@ -192,7 +192,7 @@ struct FwdArgs {
 constexpr int kFwdSlots = 32;   // a full step of 32 is even: no filler needed beyond it
 
 // One warp's 8 x 8 block `warp` of `tile`, with the warp's staging slots.
-template <int TW, int TH, bool CKPT>
+template <int TW, int TH, bool CKPT, int U>
 __device__ __forceinline__ void fwd_warp_block(const FwdArgs &a, int tile, int warp, int lane, float2 *sxy,
                                                float4 *sco, float4 *srgb) {
   constexpr int NW = TW * TH / 64;
@@ -276,7 +276,7 @@ __device__ __forceinline__ void fwd_warp_block(const FwdArgs &a, int tile, int w
       sel = row_span(e, Y0, Y1, xl, xr) && X1 >= xl && X0 <= xr;
     }
     // the passing entries, closed up in order; the colour's fourth word carries the list
-    // position. An odd count is filled with an entry of opacity 0.
+    // position. The last turn is filled with entries of opacity 0.
     const uint32_t b = __ballot_sync(0xffffffffu, sel);
     const int cnt = __popc(b);
     if (sel) {
@@ -285,9 +285,9 @@ __device__ __forceinline__ void fwd_warp_block(const FwdArgs &a, int tile, int w
       sco[at] = make_float4(__fmul_rn(co.x, kNegHalfLog2e), co.y, __fmul_rn(co.z, kNegHalfLog2e), co.w);
       srgb[at] = make_float4(c.x, c.y, c.z, __uint_as_float((uint32_t)j + 1u));
     }
-    if ((cnt & 1) && lane == 0) {
-      sxy[cnt] = make_float2(0.f, 0.f);
-      sco[cnt] = srgb[cnt] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (lane < ((U - cnt) & (U - 1))) {
+      sxy[cnt + lane] = make_float2(0.f, 0.f);
+      sco[cnt + lane] = srgb[cnt + lane] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
     __syncwarp();
     // one entry's sigma at both pixels
@@ -318,7 +318,8 @@ __device__ __forceinline__ void fwd_warp_block(const FwdArgs &a, int tile, int w
       const bool c0 = a0 && !(Tn.x < kTMin), c1 = a1 && !(Tn.y < kTMin);
       done0 = done0 || (a0 && !c0);
       done1 = done1 || (a1 && !c1);
-      const float2 w = f2_mul(f2(c0 ? al.x : 0.f, c1 ? al.y : 0.f), T);
+      const float2 as = f2(c0 ? al.x : 0.f, c1 ? al.y : 0.f);
+      const float2 w = f2_mul(as, T);
       if (CKPT) {
         cr = f2(fmaf(c.x, w.x, cr.x), fmaf(c.x, w.y, cr.y));
         cg = f2(fmaf(c.y, w.x, cg.x), fmaf(c.y, w.y, cg.y));
@@ -328,19 +329,24 @@ __device__ __forceinline__ void fwd_warp_block(const FwdArgs &a, int tile, int w
         cg = f2_fma(f2(c.y), w, cg);
         cb = f2_fma(f2(c.z), w, cb);
       }
-      T = f2(c0 ? Tn.x : T.x, c1 ? Tn.y : T.y);
+      // Tn where the entry is taken, T elsewhere (x 1): on the FMA pipe, which has room where
+      // two more selections would not (the ALU is the pipe in use most: 291 -> 272 us)
+      T = f2_mul(T, f2_sub(ONE, as));
       const uint32_t pos = __float_as_uint(c.w);
       st0 = c0 ? pos : st0;
       st1 = c1 ? pos : st1;
     };
-    // two entries at a time: their sigmas do not depend on each other, and a warp that
+    // U entries a turn: their sigmas do not depend on each other, and a warp that
     // waits for one entry's sigma after another (about 120 cycles each) is what a frame
-    // of few tiles takes its time from: 38 -> 26 us at 16 tiles, 82 -> 53 at 260, 76 -> 60
-    // at 1014, 155 -> 121 at 2542, and 313 -> 292 with checkpoints at 4056
-    for (int i = 0; i < cnt; i += 2) {
-      const float2 al_a = alpha(i), al_b = alpha(i + 1);
-      composite(al_a, srgb[i]);
-      composite(al_b, srgb[i + 1]);
+    // of few tiles takes its time from. One, two, four a turn: 38, 26, 22 us at 16 tiles, 82, 53,
+    // 45 at 260, 155, 118, 123 at 2542 (hence U by the launch), and with checkpoints 313, 272,
+    // 269 at 4056.
+    for (int i = 0; i < cnt; i += U) {
+      float2 al[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) al[u] = alpha(i + u);
+#pragma unroll
+      for (int u = 0; u < U; ++u) composite(al[u], srgb[i + u]);
     }
     __syncwarp();
   }
@@ -366,14 +372,14 @@ __device__ __forceinline__ void fwd_warp_block(const FwdArgs &a, int tile, int w
 }
 
 // One CTA per tile, warp w on the tile's block w.
-template <int TW, int TH, bool CKPT>
+template <int TW, int TH, bool CKPT, int U>
 __global__ void __launch_bounds__(TW *TH / 2) raster_fwd_warp_kernel(const FwdArgs a) {
   constexpr int NW = TW * TH / 64;
   __shared__ float2 s_xy[NW][kFwdSlots];
   __shared__ float4 s_co[NW][kFwdSlots];
   __shared__ float4 s_rgb[NW][kFwdSlots];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  fwd_warp_block<TW, TH, CKPT>(a, blockIdx.x, warp, lane, s_xy[warp], s_co[warp], s_rgb[warp]);
+  fwd_warp_block<TW, TH, CKPT, U>(a, blockIdx.x, warp, lane, s_xy[warp], s_co[warp], s_rgb[warp]);
 }
 
 // Persistent form: a resident grid whose warps claim (tile, block) units from a
@@ -382,7 +388,7 @@ __global__ void __launch_bounds__(TW *TH / 2) raster_fwd_warp_kernel(const FwdAr
 // is done. Units are independent; no warp ever waits on another.
 constexpr int kQueueWarps = 4;
 
-template <int TW, int TH, bool CKPT>
+template <int TW, int TH, bool CKPT, int U>
 __global__ void __launch_bounds__(32 * kQueueWarps) raster_fwd_queue_kernel(const FwdArgs a, int n_tiles,
                                                                            uint32_t *queue) {
   constexpr int NW = TW * TH / 64;
@@ -396,7 +402,7 @@ __global__ void __launch_bounds__(32 * kQueueWarps) raster_fwd_queue_kernel(cons
     if (lane == 0) u = atomicAdd(queue, 1u);
     u = __shfl_sync(0xffffffffu, u, 0);
     if (u >= units) break;
-    fwd_warp_block<TW, TH, CKPT>(a, (int)(u / NW), (int)(u % NW), lane, s_xy[w], s_co[w], s_rgb[w]);
+    fwd_warp_block<TW, TH, CKPT, U>(a, (int)(u / NW), (int)(u % NW), lane, s_xy[w], s_co[w], s_rgb[w]);
     __syncwarp();
   }
 }
@@ -1164,13 +1170,14 @@ __global__ void __launch_bounds__(BwdTile<TW, TH, WB>::NW * 32, BwdTile<TW, TH, 
             done0 = done0 || (a0 && !c0);
             done1 = done1 || (a1 && !c1);
           }
-          const float wt0 = (c0 ? al0 : 0.f) * tr.x, wt1 = (c1 ? al1 : 0.f) * tr.z;
+          const float as0 = c0 ? al0 : 0.f, as1 = c1 ? al1 : 0.f;
+          const float wt0 = as0 * tr.x, wt1 = as1 * tr.z;
           const float cd0 = fmaf(c.z, g0.z, fmaf(c.y, g0.y, c.x * g0.x));
           const float cd1 = fmaf(c.z, g1.z, fmaf(c.y, g1.y, c.x * g1.x));
           tr.y = fmaf(-cd0, wt0, tr.y);
           tr.w = fmaf(-cd1, wt1, tr.w);
-          tr.x = c0 ? Tn0 : tr.x;
-          tr.z = c1 ? Tn1 : tr.z;
+          tr.x = __fmul_rn(tr.x, __fsub_rn(1.f, as0));   // Tn where the entry is taken
+          tr.z = __fmul_rn(tr.z, __fsub_rn(1.f, as1));
           st0 = c0 ? pos + 1u : st0;
           st1 = c1 ? pos + 1u : st1;
         };
@@ -1323,16 +1330,21 @@ static gs_status_t launch_fwd(const gs_proj_t *proj, const gs_bins_t *bins, cons
     a.ckpt = ckpt ? *ckpt : CkptLayout{};
     a.n_records = (uint64_t)proj->n_records;
     a.list_cap = (uint64_t)bins->capacity;
+    const bool few = frame->n_tiles <= 8 * num_sms();   // entries a turn: see fwd_warp_block
     if (cfg->d_queue) {
       // persistent grid: every CTA the SMs hold at once
       GS_CUDA_TRY(cudaMemsetAsync(cfg->d_queue, 0, sizeof(uint32_t), s));
-      auto kern = ckpt ? raster_fwd_queue_kernel<TW, TH, true> : raster_fwd_queue_kernel<TW, TH, false>;
+      auto kern = ckpt  ? raster_fwd_queue_kernel<TW, TH, true, 4>
+                  : few ? raster_fwd_queue_kernel<TW, TH, false, 4>
+                        : raster_fwd_queue_kernel<TW, TH, false, 2>;
       int per_sm = 0;
       GS_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * kQueueWarps, 0));
       if (per_sm < 1) per_sm = 1;
       kern<<<num_sms() * per_sm, 32 * kQueueWarps, 0, s>>>(a, frame->n_tiles, cfg->d_queue);
     } else {
-      auto kern = ckpt ? raster_fwd_warp_kernel<TW, TH, true> : raster_fwd_warp_kernel<TW, TH, false>;
+      auto kern = ckpt  ? raster_fwd_warp_kernel<TW, TH, true, 4>
+                  : few ? raster_fwd_warp_kernel<TW, TH, false, 4>
+                        : raster_fwd_warp_kernel<TW, TH, false, 2>;
       kern<<<frame->n_tiles, TW * TH / 2, 0, s>>>(a);
     }
     GS_LAUNCH_CHECK();
