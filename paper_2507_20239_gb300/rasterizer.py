@@ -212,9 +212,10 @@ def bin_sort(proj: Projected, frame: Frame, capacity: Optional[int] = None, want
     """Bin and sort; on duplicate-capacity overflow, grow to the reported count and redo."""
     R = proj.mean2d.shape[0]
     if bins is None:
-        bins = alloc_bins(frame, R, capacity or max(1 << 16, 8 * R), want_keys)
-    for _ in range(3):
+        bins = alloc_bins(frame, R, capacity or max(1 << 16, 8 * R), want_keys)   # its error word is zero
+    else:
         bins.error.zero_()
+    for _ in range(3):
         bin_sort_into(proj, frame, bins)
         if int(bins.error.item()) == 0:
             return bins
