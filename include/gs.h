@@ -134,7 +134,8 @@ typedef struct {
   float bg[3];             /* background colour (default black)                   */
   int32_t store_stop;      /* write the per-pixel stop index in gs_raster_fwd     */
   int32_t stage_depth;     /* gs_raster_bwd: list entries staged per CTA step,
-                            * 0 = one per thread, 1 = half as many. A tuning
+                            * 0 = the full step (one per thread; on small frames
+                            * a window of 256 or 512), 1 = half as many. A tuning
                             * knob: gradients agree up to summation order. */
   uint32_t *d_queue;       /* gs_raster_fwd / gs_raster_fwd_ckpt: NULL = one CTA
                             * per tile; else a device word (overwritten) that a
@@ -240,8 +241,9 @@ gs_status_t gs_l1_loss_grad(const gs_frame_t *frame, const float *image, const f
  * with NULL the stop position is recomputed from the transmittance cut-off. Uses
  * dL/dsigma_i = T_i <c_i, g> - (<out, g> - sum_{j<=i} <c_j, g> sigma_j T_j) / (1 - sigma_i),
  * out being the forward's image; zero through the 0.99 clamp. Per-pixel terms are
- * summed per Gaussian in registers, across the warp and the CTA, then added once
- * per (tile, record) into grads (see gs_rec_grads_t). */
+ * summed per Gaussian in registers, across the warp and the CTA (on frames of few
+ * tiles by the walk of gs_raster_bwd_splat, from states kept in shared memory), then
+ * added once per (tile or part of a tile, record) into grads (see gs_rec_grads_t). */
 gs_status_t gs_raster_bwd(const gs_proj_t *proj, const gs_bins_t *bins, const gs_frame_t *frame,
                           const gs_raster_cfg_t *cfg, const float *image, const float *d_image,
                           const uint32_t *stop, gs_rec_grads_t *grads, gs_stream_t stream);
