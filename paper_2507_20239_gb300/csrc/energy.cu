@@ -124,63 +124,64 @@ __device__ __forceinline__ void load_twiddles(float2 *s_tw, const float2 *__rest
 }
 
 // Both passes are a direct O(N^2) sum per coefficient, in the order n = 0, 1, ..., on the
-// FP32 pipes. A thread keeps kDftRows lines (rows, or columns) of kDftK frequencies in
-// registers, so a twiddle serves kDftRows lines and a line's value kDftK frequencies.
+// FP32 pipes. A thread keeps 8 or 16 lines (rows, or columns) of one or two (KK) frequencies in
+// registers, so a twiddle serves all of its lines and a line's value its frequencies; neighbouring
+// lines are packed pairs (f32x2: the same operations and roundings at half the issue slots).
 // With one line and one frequency per thread the passes ran at the rate of their
 // shared-memory loads (a conflicted twiddle per two FMAs).
 // The input is real, so X[h][W - k] = conj X[h][k] and column W - k has the magnitudes of
 // column k: only k = 0 .. W / 2 are computed, the others counted with weight 2.
-// 3 x 826 x 1246: row pass ~1770 -> 234 us, column pass ~1390 -> 251 us (82% of issue
-// slots; 229 us of FMAs in the two at the FP32 peak); same bits up to the FP64 sum's order.
+// 3 x 826 x 1246: row pass ~1770 -> 216 us unpacked, 187 packed; column pass ~1390 -> 247 and 237
+// (229 us of FMAs in the two at the FP32 peak), pairs of (re, im) instead of two columns, which
+// need every value twice, 274; 3 x 207 x 312: 30 -> 14 and 21 -> 14. Same bits up to the FP64 sum's order.
 constexpr int kDftThreads = 64;
-constexpr int kDftK = 2;                        // frequencies per thread
-constexpr int kDftRows = 16;                    // rows per thread (row pass)
 constexpr int kDftCols = 8;                     // columns per thread (column pass)
 constexpr int kDftChunk = 64;                   // line positions staged at a time
-constexpr int kDftPad = kDftRows + 4;           // staged row position: 16-byte aligned, 4-way at most when filled
 
 // X[line][k] = sum_n I[line][n] exp(-2 pi i n k / W), line = channel * H + row.
-__global__ void __launch_bounds__(kDftThreads, 8) dft_rows_kernel(const float *__restrict__ img, int64_t lines, int W,
-                                                               int K, const float2 *__restrict__ tw,
-                                                               float2 *__restrict__ X) {
+template <int ROWS, int KK>
+__global__ void __launch_bounds__(kDftThreads, ROWS * KK > 16 ? 6 : 12) dft_rows_kernel(
+    const float *__restrict__ img, int64_t lines, int W, int K, const float2 *__restrict__ tw, float2 *__restrict__ X) {
+  constexpr int kPad = ROWS + 4;   // staged position: 16-byte aligned, 4-way at most when filled
   extern __shared__ float4 s_raw[];
-  float *s_x = reinterpret_cast<float *>(s_raw);                               // [kDftChunk][kDftPad]
-  float2 *s_tw = reinterpret_cast<float2 *>(s_x + kDftChunk * kDftPad);
-  const int64_t l0 = (int64_t)blockIdx.x * kDftRows;
+  float *s_x = reinterpret_cast<float *>(s_raw);                               // [kDftChunk][kPad]
+  float2 *s_tw = reinterpret_cast<float2 *>(s_x + kDftChunk * kPad);
+  const int64_t l0 = (int64_t)blockIdx.x * ROWS;
   load_twiddles(s_tw, tw, W);
-  int k[kDftK], q[kDftK];
-  float re[kDftK][kDftRows], im[kDftK][kDftRows];
+  int k[KK], q[KK];
+  float2 re[KK][ROWS / 2], im[KK][ROWS / 2];
 #pragma unroll
-  for (int j = 0; j < kDftK; ++j) {
-    const int kk = (blockIdx.y * kDftK + j) * kDftThreads + threadIdx.x;
+  for (int j = 0; j < KK; ++j) {
+    const int kk = (blockIdx.y * KK + j) * kDftThreads + threadIdx.x;
     k[j] = kk < K ? kk : 0;
     q[j] = 0;
 #pragma unroll
-    for (int r = 0; r < kDftRows; ++r) re[j][r] = im[j][r] = 0.f;
+    for (int r = 0; r < ROWS / 2; ++r) re[j][r] = im[j][r] = make_float2(0.f, 0.f);
   }
   for (int n0 = 0; n0 < W; n0 += kDftChunk) {
     const int cnt = min(kDftChunk, W - n0);
     __syncthreads();
-    for (int i = threadIdx.x; i < kDftChunk * kDftRows; i += kDftThreads) {
+    for (int i = threadIdx.x; i < kDftChunk * ROWS; i += kDftThreads) {
       const int r = i / kDftChunk, n = i - r * kDftChunk;
-      s_x[n * kDftPad + r] = n < cnt && l0 + r < lines ? img[(l0 + r) * W + n0 + n] : 0.f;
+      s_x[n * kPad + r] = n < cnt && l0 + r < lines ? img[(l0 + r) * W + n0 + n] : 0.f;
     }
     __syncthreads();
-#pragma unroll 2
+#pragma unroll 4
     for (int n = 0; n < cnt; ++n) {
-      float x[kDftRows];
+      float2 x[ROWS / 2];
 #pragma unroll
-      for (int r = 0; r < kDftRows; r += 4) {
-        const float4 v = *reinterpret_cast<const float4 *>(s_x + n * kDftPad + r);
-        x[r] = v.x; x[r + 1] = v.y; x[r + 2] = v.z; x[r + 3] = v.w;
+      for (int r = 0; r < ROWS / 2; r += 2) {
+        const float4 v = *reinterpret_cast<const float4 *>(s_x + n * kPad + 2 * r);
+        x[r] = make_float2(v.x, v.y);
+        x[r + 1] = make_float2(v.z, v.w);
       }
 #pragma unroll
-      for (int j = 0; j < kDftK; ++j) {
+      for (int j = 0; j < KK; ++j) {
         const float2 t = s_tw[tw_slot(q[j])];
 #pragma unroll
-        for (int r = 0; r < kDftRows; ++r) {
-          re[j][r] = fmaf(x[r], t.x, re[j][r]);
-          im[j][r] = fmaf(x[r], t.y, im[j][r]);
+        for (int r = 0; r < ROWS / 2; ++r) {
+          re[j][r] = f2_fma(x[r], f2(t.x), re[j][r]);
+          im[j][r] = f2_fma(x[r], f2(t.y), im[j][r]);
         }
         q[j] += k[j];
         q[j] = (int)min((uint32_t)q[j], (uint32_t)(q[j] - W));   // q mod W (q < 2 W)
@@ -188,12 +189,14 @@ __global__ void __launch_bounds__(kDftThreads, 8) dft_rows_kernel(const float *_
     }
   }
 #pragma unroll
-  for (int j = 0; j < kDftK; ++j) {
-    const int kk = (blockIdx.y * kDftK + j) * kDftThreads + threadIdx.x;
+  for (int j = 0; j < KK; ++j) {
+    const int kk = (blockIdx.y * KK + j) * kDftThreads + threadIdx.x;
     if (kk >= K) continue;
 #pragma unroll
-    for (int r = 0; r < kDftRows; ++r)
-      if (l0 + r < lines) X[(l0 + r) * K + kk] = make_float2(re[j][r], im[j][r]);
+    for (int r = 0; r < ROWS; ++r)
+      if (l0 + r < lines)
+        X[(l0 + r) * K + kk] = r & 1 ? make_float2(re[j][r / 2].y, im[j][r / 2].y)
+                                     : make_float2(re[j][r / 2].x, im[j][r / 2].x);
   }
 }
 
@@ -218,49 +221,51 @@ __device__ __forceinline__ void add_magnitude(float re, float im, float weight, 
 
 // Y[m] = sum_h X[h][k] exp(-2 pi i h m / H) of kDftCols adjacent columns k (of the K kept)
 // of one channel; adds sum |Y[m]| to *sum, columns that stand for W - k too twice.
-__global__ void __launch_bounds__(kDftThreads, 10) dft_cols_l1_kernel(const float2 *__restrict__ X, int H, int W, int K,
-                                                                  const float2 *__restrict__ tw, double *sum) {
+template <int KK>
+__global__ void __launch_bounds__(kDftThreads, KK > 1 ? 8 : 12) dft_cols_l1_kernel(
+    const float2 *__restrict__ X, int H, int W, int K, const float2 *__restrict__ tw, double *sum) {
   extern __shared__ float4 s_raw[];
-  float2 *s_x = reinterpret_cast<float2 *>(s_raw);                            // [kDftChunk][kDftCols]
-  float2 *s_tw = s_x + kDftChunk * kDftCols;
+  float4 *s_x = s_raw;                          // [kDftChunk][kDftCols / 2]: (re, re, im, im) of two columns
+  float2 *s_tw = reinterpret_cast<float2 *>(s_x + kDftChunk * kDftCols / 2);
   const int col_blocks = (K + kDftCols - 1) / kDftCols;
   const int ch = blockIdx.x / col_blocks, c0 = (blockIdx.x - ch * col_blocks) * kDftCols;
   const float2 *src = X + (int64_t)ch * H * K;
   load_twiddles(s_tw, tw, H);
-  int m[kDftK], q[kDftK];
-  float re[kDftK][kDftCols], im[kDftK][kDftCols];
+  int m[KK], q[KK];
+  float2 re[KK][kDftCols / 2], im[KK][kDftCols / 2];
 #pragma unroll
-  for (int j = 0; j < kDftK; ++j) {
-    const int mm = (blockIdx.y * kDftK + j) * kDftThreads + threadIdx.x;
+  for (int j = 0; j < KK; ++j) {
+    const int mm = (blockIdx.y * KK + j) * kDftThreads + threadIdx.x;
     m[j] = mm < H ? mm : 0;
     q[j] = 0;
 #pragma unroll
-    for (int c = 0; c < kDftCols; ++c) re[j][c] = im[j][c] = 0.f;
+    for (int c = 0; c < kDftCols / 2; ++c) re[j][c] = im[j][c] = f2(0.f);
   }
   for (int h0 = 0; h0 < H; h0 += kDftChunk) {
     const int cnt = min(kDftChunk, H - h0);
     __syncthreads();
     for (int i = threadIdx.x; i < kDftChunk * kDftCols; i += kDftThreads) {
       const int h = i / kDftCols, c = i - h * kDftCols;
-      s_x[i] = h < cnt && c0 + c < K ? src[(int64_t)(h0 + h) * K + c0 + c] : make_float2(0.f, 0.f);
+      const float2 x = h < cnt && c0 + c < K ? src[(int64_t)(h0 + h) * K + c0 + c] : make_float2(0.f, 0.f);
+      float *to = reinterpret_cast<float *>(s_x + i / 2) + (c & 1);
+      to[0] = x.x;
+      to[2] = x.y;
     }
     __syncthreads();
-#pragma unroll 2
+#pragma unroll 4
     for (int h = 0; h < cnt; ++h) {
-      float2 x[kDftCols];
+      float4 x[kDftCols / 2];
 #pragma unroll
-      for (int c = 0; c < kDftCols; c += 2) {
-        const float4 v = *reinterpret_cast<const float4 *>(s_x + h * kDftCols + c);
-        x[c] = make_float2(v.x, v.y);
-        x[c + 1] = make_float2(v.z, v.w);
-      }
+      for (int c = 0; c < kDftCols / 2; ++c) x[c] = s_x[h * (kDftCols / 2) + c];
 #pragma unroll
-      for (int j = 0; j < kDftK; ++j) {
+      for (int j = 0; j < KK; ++j) {
         const float2 t = s_tw[tw_slot(q[j])];
+        const float2 tx = f2(t.x), ty = f2(t.y), ny = f2(-t.y);
 #pragma unroll
-        for (int c = 0; c < kDftCols; ++c) {
-          re[j][c] = fmaf(x[c].x, t.x, fmaf(-x[c].y, t.y, re[j][c]));
-          im[j][c] = fmaf(x[c].x, t.y, fmaf(x[c].y, t.x, im[j][c]));
+        for (int c = 0; c < kDftCols / 2; ++c) {
+          const float2 xr = f2(x[c].x, x[c].y), xi = f2(x[c].z, x[c].w);
+          re[j][c] = f2_fma(xr, tx, f2_fma(xi, ny, re[j][c]));
+          im[j][c] = f2_fma(xr, ty, f2_fma(xi, tx, im[j][c]));
         }
         q[j] += m[j];
         q[j] = (int)min((uint32_t)q[j], (uint32_t)(q[j] - H));
@@ -270,12 +275,14 @@ __global__ void __launch_bounds__(kDftThreads, 10) dft_cols_l1_kernel(const floa
   float part = 0.f, part_c = 0.f;
   double wide = 0.0;
 #pragma unroll
-  for (int j = 0; j < kDftK; ++j) {
-    if ((blockIdx.y * kDftK + j) * kDftThreads + threadIdx.x >= H) continue;
+  for (int j = 0; j < KK; ++j) {
+    if ((blockIdx.y * KK + j) * kDftThreads + threadIdx.x >= H) continue;
 #pragma unroll
     for (int c = 0; c < kDftCols; ++c) {
       const int k = c0 + c;
-      if (k < K) add_magnitude(re[j][c], im[j][c], k == 0 || 2 * k == W ? 1.f : 2.f, part, part_c, wide);
+      const float2 r = re[j][c / 2], i = im[j][c / 2];
+      if (k < K)
+        add_magnitude(c & 1 ? r.y : r.x, c & 1 ? i.y : i.x, k == 0 || 2 * k == W ? 1.f : 2.f, part, part_c, wide);
     }
   }
   if (wide != 0.0) atomicAdd(sum, wide);
@@ -329,24 +336,40 @@ extern "C" gs_status_t gs_spectrum_l1(const float *image, int32_t C, int32_t H, 
   cudaStream_t s = as_stream(stream);
   const int K = W / 2 + 1;
   const int64_t lines = (int64_t)C * H;
-  const int64_t row_blocks = (lines + kDftRows - 1) / kDftRows;
   const int64_t col_blocks = (int64_t)C * ((K + kDftCols - 1) / kDftCols);
+  const int64_t row_blocks = (lines + 15) / 16;   // of 16 lines
   if (row_blocks > 0x7fffffffll || col_blocks > 0x7fffffffll) return GS_ERR_INVALID_ARG;
   float2 *X = static_cast<float2 *>(ws);
   float2 *tw_w = X + lines * K, *tw_h = tw_w + W;
-  const size_t smem_rows = sizeof(float) * kDftChunk * kDftPad + sizeof(float2) * tw_slots(W);
-  const size_t smem_cols = sizeof(float2) * kDftChunk * kDftCols + sizeof(float2) * tw_slots(H);
-  static_assert(sizeof(float2) * (kDftChunk * kDftCols + kEnergyMaxDim + kEnergyMaxDim / 16 + 1) <= 48 * 1024,
-                "fits the default shared-memory limit");
   GS_CUDA_TRY(cudaMemsetAsync(d_sum, 0, sizeof(double), s));
   twiddles_kernel<<<(W + H + 127) / 128, 128, 0, s>>>(tw_w, W, tw_h, H);
   GS_LAUNCH_CHECK();
-  constexpr int kPer = kDftThreads * kDftK;
-  dft_rows_kernel<<<dim3((unsigned)row_blocks, (K + kPer - 1) / kPer), kDftThreads, smem_rows, s>>>(image, lines, W, K,
-                                                                                                tw_w, X);
+  auto rows = [&](auto kernel, int per, int freqs) {
+    const dim3 grid((unsigned)((lines + per - 1) / per), (K + kDftThreads * freqs - 1) / (kDftThreads * freqs));
+    const size_t smem = sizeof(float) * kDftChunk * (per + 4) + sizeof(float2) * tw_slots(W);
+    kernel<<<grid, kDftThreads, smem, s>>>(image, lines, W, K, tw_w, X);
+  };
+  auto cols = [&](auto kernel, int freqs) {
+    const dim3 grid((unsigned)col_blocks, (H + kDftThreads * freqs - 1) / (kDftThreads * freqs));
+    const size_t smem = sizeof(float2) * kDftChunk * kDftCols + sizeof(float2) * tw_slots(H);
+    static_assert(sizeof(float2) * (kDftChunk * kDftCols + kEnergyMaxDim + kEnergyMaxDim / 16 + 1) <= 48 * 1024,
+                  "fits the default shared-memory limit");
+    kernel<<<grid, kDftThreads, smem, s>>>(X, H, W, K, tw_h, d_sum);
+  };
+  // The larger tiles reuse more per load, the smaller ones keep more warps at work, and on
+  // images of few blocks, whose threads wait for one sum after another, that counts for more. Larger
+  // and smaller, us: rows, at 9.2, 5.1, 3.0, 1.5, 0.8, 0.5 blocks of 16 x 128 per SM, 378 / 569,
+  // 187 / 277, 95 / 114, 43 / 44, 35 / 29, 23 / 14; columns, at 10.8, 5.6, 5.0, 3.1, 1.5, 0.8 blocks of
+  // 8 x 128, 237 / 259, 97 / 109, 84 / 85, 48 / 40, 24 / 20, 19 / 14.
+  if (row_blocks * ((K + 2 * kDftThreads - 1) / (2 * kDftThreads)) >= num_sms())
+    rows(dft_rows_kernel<16, 2>, 16, 2);
+  else
+    rows(dft_rows_kernel<8, 1>, 8, 1);
   GS_LAUNCH_CHECK();
-  dft_cols_l1_kernel<<<dim3((unsigned)col_blocks, (H + kPer - 1) / kPer), kDftThreads, smem_cols, s>>>(
-      X, H, W, K, tw_h, d_sum);
+  if (col_blocks * ((H + 2 * kDftThreads - 1) / (2 * kDftThreads)) >= 4 * num_sms())
+    cols(dft_cols_l1_kernel<2>, 2);
+  else
+    cols(dft_cols_l1_kernel<1>, 1);
   GS_LAUNCH_CHECK();
   return GS_OK;
 }

@@ -47,6 +47,13 @@ def test_spectrum_l1_at_tile_edges(shape):
     assert abs(got - want) <= 1e-5 * want
 
 
+@pytest.mark.parametrize("shape", [(8, 397, 333), (9, 259, 515), (3, 530, 255)])
+def test_spectrum_l1_larger_tiles(shape):
+    """Images of blocks enough for the passes' larger tiles (16 rows, two frequencies a
+    thread), with ragged last tiles; tolerance as above."""
+    test_spectrum_l1_at_tile_edges(shape)
+
+
 @pytest.mark.parametrize("shape,r", [((3, 207, 311), 16), ((2, 207, 311), 17), ((1, 207, 311), 40), ((2, 5, 33), 2),
                                      ((1, 9, 64), 2), ((1, 40, 3), 8)])
 def test_downscale_filter_widths(shape, r):
