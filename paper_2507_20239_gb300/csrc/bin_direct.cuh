@@ -17,8 +17,8 @@
 // instead of 8 bytes out, 8 in and 8 out again, the gathers in depth order touch one place per
 // record (its header and runs) instead of four, no two warps claim work from one
 // counter, and a frame takes 9 or 10 launches instead of 21. gs_bin_sort, that path -> this one,
-// kernel times: 5M Gaussians in 4 views of 1600 x 1060 (72.8M entries) 6.03 -> 3.73 ms, 500k in
-// 12 mixed views (34.7M) 1.46 -> 1.09 ms, 1.5M in one 1246 x 826 view (16.5M) 430 -> 424 us, 600k
+// kernel times: 5M Gaussians in 4 views of 1600 x 1060 (72.8M entries) 6.03 -> 3.65 ms, 500k in
+// 12 mixed views (34.7M) 1.46 -> 1.07 ms, 1.5M in one 1246 x 826 view (16.5M) 430 -> 416 us, 600k
 // on 979 x 653 192 -> 185, 100k on 312 x 207 85 -> 65, 2k on 64 x 64 75 -> 38. The emission is half
 // of it at the larger sizes; without its scattered 4-byte stores it takes 149 of 203 us (1.5M).
 #pragma once
@@ -689,7 +689,9 @@ __global__ void __launch_bounds__(kDirScanThreads) direct_scan_kernel(const DirA
 // a population count of the bits below it, with a third barrier for the cursors, 210 / 1967,
 // and with the hits spread evenly over the lanes first, 242 / 1849; groups of 32, 64 or 128
 // records, 256 or 512 threads 203 to 216 / 1650 to 2130; a warp writing a tile's entries together
-// where there are more than 4 or 8, 273 and 237 / 2513 and 2221.
+// where there are more than 4 or 8, 273 and 237 / 2513 and 2221. One warp per chunk with cursors
+// of its own and no barriers: a record's rectangle over the lanes, record after record, 345 / 4198; the
+// hits spread over the lanes, those of a tile ranked by match.any, 234 / 1809.
 // W words of mask per tile: 4 W + 4 + 2 1/8 bytes of shared memory per tile of the view.
 constexpr int kEmitThreads = 256;
 constexpr uint32_t kEmitStage = 3 * kEmitThreads;   // units staged at a time, three loads a thread in flight
