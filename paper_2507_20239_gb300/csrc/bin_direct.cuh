@@ -878,13 +878,17 @@ inline uint64_t dir_unit_cap(int64_t R, int64_t cap, int64_t unit_grid) {
 // sixteen with several views, whose sizes may differ (12 views of a quarter to full size: 1165
 // us for the whole binning with eight, 1086 with sixteen; one view of 4056 tiles 426 and 447,
 // the matrix being longer to scan), of at least 64 records, and a matrix within its bound. Refused: views of more
-// tiles than the emission has shared memory for, and sizes beyond the counters'.
+// tiles than the emission has shared memory for, sizes beyond the counters', less than a record a
+// view, and frames whose layout gs_frame_init has not written (a view's tables in shared memory
+// are sized by the largest view: max_width and max_height have to cover every view's tiles).
 inline DirPlan dir_plan(const gs_frame_t *f, int64_t R, int64_t cap) {
   DirPlan p{};
-  if (f->n_views > kDirMaxViews || R < 1) return p;
+  if (f->n_views < 1 || f->n_views > kDirMaxViews || R < f->n_views || f->n_tiles < 1) return p;
+  if (f->tile_w < 1 || f->tile_h < 1 || f->max_width < 1 || f->max_height < 1) return p;
   const int64_t n = R / f->n_views;
-  const int64_t gx = (f->max_width + f->tile_w - 1) / f->tile_w, gy = (f->max_height + f->tile_h - 1) / f->tile_h;
-  if (gx * gy > kDirMaxTiles || n >= (1ll << 30)) return p;
+  const int64_t gx = ((int64_t)f->max_width + f->tile_w - 1) / f->tile_w;
+  const int64_t gy = ((int64_t)f->max_height + f->tile_h - 1) / f->tile_h;
+  if (gx * gy > kDirMaxTiles || gx * gy * f->n_views < f->n_tiles || n >= (1ll << 30)) return p;
   p.max_tiles = (int)(gx * gy);
   int64_t chunks = ((f->n_views > 1 ? 16ll : 8ll) * num_sms() + f->n_views - 1) / f->n_views;
   const int64_t groups = (n + kDirThreads - 1) / kDirThreads, by_matrix = kDirMatrix / f->n_tiles;

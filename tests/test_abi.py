@@ -187,3 +187,31 @@ def test_bin_sort_workspace_without_a_frame_is_enough_for_any():
             for cap in (0, 1, 5_000_000):
                 size = lib.gs_bin_sort_workspace_size(n * n_views, cap, C.byref(fr))
                 assert 0 < size <= lib.gs_bin_sort_workspace_size(n * n_views, cap, None), (n_views, w, n, cap)
+
+
+def test_bin_sort_workspace_of_frames_and_counts_without_a_plan():
+    """Fewer records than views, no view at all, a frame that gs_frame_init has not filled: a size
+    (the general path's), in a process of its own, which a division by zero would end."""
+    import sys
+    code = """
+import ctypes as C
+from paper_2507_20239_gb300 import _abi
+lib = _abi.load()
+cams = (_abi.GsCamera * 4)()
+for c in cams:
+    c.fx = c.fy = 100.0
+    c.width, c.height, c.near_plane = 100, 60, 0.2
+fr = _abi.GsFrame()
+assert lib.gs_frame_init(cams, 4, 16, 16, C.byref(fr)) == 0
+sizes = [lib.gs_bin_sort_workspace_size(n, 1000, C.byref(fr)) for n in (0, 1, 3, 4)]
+for field, value in (("n_views", 0), ("n_views", -1), ("n_tiles", 0), ("tile_w", 0), ("tile_h", 0), ("max_width", 0),
+                     ("max_height", 0)):
+    f = _abi.GsFrame.from_buffer_copy(fr)
+    setattr(f, field, value)
+    sizes.append(lib.gs_bin_sort_workspace_size(1000, 1000, C.byref(f)))
+sizes.append(lib.gs_bin_sort_workspace_size(1000, 1000, C.byref(_abi.GsFrame())))
+assert all(s > 4 * 1000 for s in sizes), sizes
+"""
+    r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True,
+                       cwd=os.path.dirname(os.path.dirname(HEADER)))
+    assert r.returncode == 0, (r.returncode, r.stderr)
