@@ -156,3 +156,10 @@ class GsError(RuntimeError):
 def check(code, where):
     if code != 0:
         raise GsError(code, where)
+
+
+def check_error_word(word, where):
+    """Raise for a device error word, in which a call ORs its status bits. A wait that ran out
+    goes before a capacity: the counts beside it are not ones to size a buffer by."""
+    if word != 0:
+        raise GsError(4 if word & 4 else 2 if word & 2 else word, where)

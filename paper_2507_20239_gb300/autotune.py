@@ -17,6 +17,7 @@ from typing import Callable, Optional, Sequence
 
 import torch
 
+from . import _abi
 from .rasterizer import lib
 from .step import StepConfig, TrainStep
 
@@ -115,8 +116,7 @@ def autotune(params: dict, sh_degree: int, cameras, target_images, candidates: S
             return None
         step = TrainStep(params, sh_degree, cameras, target_images, cfg, device=device)
         ms = time_step(step, reps=reps)
-        if step.error() != 0:
-            raise RuntimeError("duplicate capacity exceeded")
+        _abi.check_error_word(step.error(), "duplicates or checkpoints")
         img = step.image.clone()
         if ref_image[0] is None:
             ref_image[0] = img

@@ -209,7 +209,8 @@ def bin_sort_into(proj: Projected, frame: Frame, bins: Bins, stream=None):
 
 def bin_sort(proj: Projected, frame: Frame, capacity: Optional[int] = None, want_keys=False,
              bins: Optional[Bins] = None) -> Bins:
-    """Bin and sort; on duplicate-capacity overflow, grow to the reported count and redo."""
+    """Bin and sort; on duplicate-capacity overflow, grow to the reported count and redo. Any other
+    device error is raised."""
     R = proj.mean2d.shape[0]
     if bins is None:
         bins = alloc_bins(frame, R, capacity or max(1 << 16, 8 * R), want_keys)   # its error word is zero
@@ -217,8 +218,11 @@ def bin_sort(proj: Projected, frame: Frame, capacity: Optional[int] = None, want
         bins.error.zero_()
     for _ in range(3):
         bin_sort_into(proj, frame, bins)
-        if int(bins.error.item()) == 0:
+        word = int(bins.error.item())
+        if word == 0:
             return bins
+        if word & ~2:
+            _abi.check_error_word(word, "gs_bin_sort")
         need = int(bins.count.item())
         bins = alloc_bins(frame, R, int(need * 1.1) + 1024, want_keys)
     raise _abi.GsError(2, "gs_bin_sort capacity")

@@ -21,6 +21,7 @@ from dataclasses import dataclass
 
 import torch
 
+from . import _abi
 from . import rasterizer as R
 from .autograd import DensifyStats
 
@@ -91,8 +92,7 @@ class TrainStep:
                 R.bin_sort_into(self.proj, f, self.bins)
                 R.raster_fwd_ckpt(self.proj, self.bins, f, probe, image=self.image, T_final=self.T, stop=self.stop)
                 R.ckpt_usage(f, self.bins, probe, out=self.ckpt_use)
-                if int(self.bins.error.item()) != 0:
-                    raise RuntimeError("TrainStep: duplicate capacity exceeded while sizing the checkpoints")
+                _abi.check_error_word(int(self.bins.error.item()), "TrainStep: binning while sizing the checkpoints")
                 slots = int(int(self.ckpt_use[0].item()) * headroom) + 4 * 256
                 del probe
             self.ckpt = R.alloc_ckpt(f, self.bins, slots)
@@ -150,7 +150,8 @@ class TrainStep:
         return g
 
     def error(self) -> int:
-        """gs_bin_sort's device error word (0: every list fitted the capacity), with
+        """gs_bin_sort's device error word (0: every list fitted the capacity; else GS_ERR_CAPACITY,
+        and GS_ERR_TIMEOUT if a wait of its sort ran out), with
         GS_ERR_CAPACITY also set when the per-splat forward ran out of checkpoint slots."""
         err = int(self.bins.error.item())
         if self.ckpt is not None:
