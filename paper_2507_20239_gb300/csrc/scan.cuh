@@ -25,10 +25,10 @@ __device__ __forceinline__ uint32_t lanemask_lt() {
   return m;
 }
 
-// Exclusive scan over the block (kScanThreads threads); returns the block total in *total.
+// Exclusive scan over the block (whole warps, up to 1024 threads); returns the block total in *total.
 template <typename T>
 __device__ __forceinline__ T block_exclusive_scan(T x, T *total) {
-  __shared__ T warp_sums[32];
+  __shared__ T warp_sums[33];   // [32]: the total
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   T incl = x;
 #pragma unroll
@@ -48,11 +48,11 @@ __device__ __forceinline__ T block_exclusive_scan(T x, T *total) {
       if (lane >= o) wi += y;
     }
     if (lane < nw) warp_sums[lane] = wi - w;
-    if (lane == nw - 1) warp_sums[31] = wi;
+    if (lane == nw - 1) warp_sums[32] = wi;
   }
   __syncthreads();
   const T res = warp_sums[warp] + incl - x;
-  *total = warp_sums[31];
+  *total = warp_sums[32];
   __syncthreads();
   return res;
 }
