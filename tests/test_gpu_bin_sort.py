@@ -235,3 +235,72 @@ def test_bin_sort_many_records_in_one_place():
     for k in ("radius", "depth", "rect"):
         empty[k][:] = 0
     _check([r, empty], [cam, cam], (16, 16))
+
+
+# ---- the general path (emitted pairs and radix passes): views of more than 20000 tiles, or more than
+# 1024 views, with the cases that smaller frames give the counting path
+
+def _large_views(seed, n, views=1):
+    """8 x 8 tiles: 34,669 of a view, with smaller ones beside it."""
+    sizes = [(1700, 1300), (425, 325), (850, 650)][:views]
+    cams = [synth.Camera(np.eye(3, dtype=np.float32), np.zeros(3, np.float32), 100., 100., w / 2, h / 2, w, h)
+            for w, h in sizes]
+    return _synthetic_records(seed, n, cams, (8, 8)), cams
+
+
+@pytest.mark.parametrize("fused_bits", [0, 1, 3, 8])
+def test_pair_path_fused_bits_and_views(fused_bits):
+    recs, cams = _large_views(31, 6000, views=3)
+    _check(recs, cams, (8, 8), fused_bits=fused_bits)
+
+
+def test_pair_path_capacity_overflow_reports_and_retries():
+    recs, cams = _large_views(32, 3000)
+    frame, proj = R.Frame(cams, tile=(8, 8)), records_to_gpu(recs)
+    _, vals, _ = _oracle_bins(recs, frame)
+    bins = R.alloc_bins(frame, proj.mean2d.shape[0], capacity=len(vals) // 2)
+    R.bin_sort_into(proj, frame, bins)
+    torch.cuda.synchronize()
+    assert int(bins.error.item()) == 2 and int(bins.count.item()) == max(len(vals), _rect_rows(recs))
+    assert np.all(bins.ranges.cpu().numpy() == 0)
+    _check(recs, cams, (8, 8), capacity=len(vals) // 2)
+
+
+def test_pair_path_rectangle_rows_beyond_the_entry_count():
+    recs, cams = _large_views(33, 2000)
+    r, n = recs[0], 2000
+    rng = np.random.default_rng(98)
+    tx, ty = rng.integers(0, 212, n), rng.integers(0, 162, n)
+    r["mean2d"][:] = np.stack([8 * tx + 4, 8 * ty + 4], 1).astype(np.float32)
+    r["conic_f"][:] = [4.0, 0.0, 4.0]
+    r["q_max"][:] = np.float32(2 * np.log(255 * 0.5))
+    r["rect"][:] = np.stack([tx, np.zeros(n), tx + 1, np.full(n, 163)], 1).astype(r["rect"].dtype)
+    r["radius"][:] = 2
+    r["depth"][:] = rng.uniform(1.0, 5.0, n).astype(np.float32)
+    frame = R.Frame(cams, tile=(8, 8))
+    bins = R.alloc_bins(frame, n, capacity=8 * n)
+    R.bin_sort_into(records_to_gpu(recs), frame, bins)
+    torch.cuda.synchronize()
+    assert int(bins.error.item()) == 2 and int(bins.count.item()) == _rect_rows(recs) == 163 * n
+    assert _check(recs, cams, (8, 8), capacity=8 * n) >= n
+
+
+def test_pair_path_ties_and_empty_views():
+    recs, cams = _large_views(34, 4000, views=2)
+    for r in recs:
+        r["depth"][r["radius"] > 0] = 2.5
+    _check(recs, cams, (8, 8))                       # ties: record order
+    for k in ("radius", "depth", "rect"):
+        recs[0][k][:] = 0
+    _check(recs, cams, (8, 8))                       # nothing visible in one view
+    for k in ("radius", "depth", "rect"):
+        recs[1][k][:] = 0
+    assert _check(recs, cams, (8, 8)) == 0           # nor in the other
+
+
+@pytest.mark.parametrize("views", [1024, 1025])      # the counting path's most views, and one more
+def test_bin_sort_of_many_small_views(views):
+    cams = [synth.Camera(np.eye(3, dtype=np.float32), np.zeros(3, np.float32), 30., 30., w / 2, 9., w, 17)
+            for w in (15 + v % 20 for v in range(views))]
+    recs = _synthetic_records(40, 40, cams, (16, 16))
+    assert _check(recs, cams, (16, 16)) > views
