@@ -8,8 +8,8 @@
 // normalised to sum 1; rows likewise.
 //
 // ||E(I)||_1: a 2D DFT of each channel as two 1D DFT passes -- rows (real input) and
-// columns (complex input, the magnitudes summed in FP64 per block and added once per
-// block), each a direct sum with twiddles from a shared table indexed by n k mod N, the
+// columns (complex input, the magnitudes to about 2^-46 in FP32 pairs, summed as such per
+// warp and added once per warp in FP64), each a direct sum with twiddles from a shared table indexed by n k mod N, the
 // index advanced incrementally; no FFT library is used. The direct sum keeps every
 // coefficient's FP32 rounding sequence independent of how N factors.
 #include <algorithm>
@@ -133,7 +133,7 @@ __device__ __forceinline__ void load_twiddles(float2 *s_tw, const float2 *__rest
 // column k: only k = 0 .. W / 2 are computed, the others counted with weight 2.
 // 3 x 826 x 1246: row pass ~1770 -> 216 us unpacked, 187 packed; column pass ~1390 -> 247 and 237
 // (229 us of FMAs in the two at the FP32 peak), pairs of (re, im) instead of two columns, which
-// need every value twice, 274; 3 x 207 x 312: 30 -> 14 and 21 -> 14. Same bits up to the FP64 sum's order.
+// need every value twice, 274; 3 x 207 x 312: 30 -> 14 and 21 -> 14. The coefficients have the same bits.
 constexpr int kDftThreads = 64;
 constexpr int kDftCols = 8;                     // columns per thread (column pass)
 constexpr int kDftChunk = 64;                   // line positions staged at a time
@@ -202,21 +202,22 @@ __global__ void __launch_bounds__(kDftThreads, ROWS * KK > 16 ? 6 : 12) dft_rows
 
 // (s, c) += weight |z|, |z| to about 2^-46 in FP32 pairs (the FP64 square root ran for
 // longer than the DFT): z's squares as hi + lo exactly but for lo's last bits, m ~ sqrt(hi)
-// and its correction (hi + lo - m^2) / (2 m). Outside the range where no term of that under-
-// or overflows, the FP64 root, into `wide`. weight: 1 or 2.
+// and its correction (hi + lo - m^2) / (2 m), one rounding per operation as written (a
+// contracted product would count its own rounding error twice). Outside the range where no term of
+// that under- or overflows, the FP64 root, into `wide`. weight: 1 or 2.
 __device__ __forceinline__ void add_magnitude(float re, float im, float weight, float &s, float &c, double &wide) {
   const float a = fmaxf(fabsf(re), fabsf(im)), b = fminf(fabsf(re), fabsf(im));
   if (!(a >= 1e-12f && fabsf(re) <= 1e15f && fabsf(im) <= 1e15f)) {
     if (re != 0.f || im != 0.f) wide += (double)weight * sqrt((double)re * re + (double)im * im);
     return;
   }
-  const float a2 = a * a, b2 = b * b;
-  const float hi = a2 + b2;
-  const float lo = (b2 - (hi - a2)) + (fmaf(a, a, -a2) + fmaf(b, b, -b2));
-  const float m = sqrtf(hi);
-  const float e = (fmaf(-m, m, hi) + lo) * (0.5f / m);
-  pair_add(s, c, weight * m);
-  c += weight * e;
+  const float a2 = __fmul_rn(a, a), b2 = __fmul_rn(b, b);
+  const float hi = __fadd_rn(a2, b2);
+  const float lo = __fadd_rn(__fsub_rn(b2, __fsub_rn(hi, a2)), __fadd_rn(__fmaf_rn(a, a, -a2), __fmaf_rn(b, b, -b2)));
+  const float m = __fsqrt_rn(hi);
+  const float e = __fmul_rn(__fadd_rn(__fmaf_rn(-m, m, hi), lo), __fdiv_rn(0.5f, m));
+  pair_add(s, c, __fmul_rn(weight, m));
+  c = __fadd_rn(c, __fmul_rn(weight, e));
 }
 
 // Y[m] = sum_h X[h][k] exp(-2 pi i h m / H) of kDftCols adjacent columns k (of the K kept)

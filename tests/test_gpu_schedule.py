@@ -102,3 +102,41 @@ def test_energy_schedule_drives_training():
     tr = Trainer(synth.surface_scene(3, 10_000, 3).params(), views, sched, extent=4.4)
     hist = tr.run(log_every=100)
     assert tr.event == 3 and hist[-1][2] < hist[0][2]
+
+
+def _column_spectrum(x0, x1):
+    """||E||_1 of the one-column image (x0, x1, 0, 0), whose DFT takes one rounding per coefficient: the
+    twiddles are 1, -i, -1 and i, so Y = (x0 + x1, x0 - i x1, x0 - x1, x0 + i x1) in FP32."""
+    a, b = np.float32(x0), np.float32(x1)
+    with np.errstate(all="ignore"):
+        return abs(np.float64(a + b)) + abs(np.float64(a - b)) + 2 * np.hypot(np.float64(a), np.float64(b))
+
+
+@pytest.mark.parametrize("seed", range(8))
+def test_spectrum_magnitudes_beyond_fp32(seed):
+    """The sum of exactly known coefficients: each magnitude within 2^-46 of its value and the sums in
+    pairs of 2^-47 and FP64, so 2^-43 with room for 16 terms; an FP32 root would be off by 2^-25."""
+    rng = np.random.default_rng(seed)
+    x = (rng.uniform(0.5, 1.0, (4, 2)) * 2.0 ** rng.integers(-3, 3, (4, 2))).astype(np.float32)
+    for c in (1, 4):
+        img = np.zeros((c, 4, 1), np.float32)
+        img[:, :2, 0] = x[:c]
+        want = sum(_column_spectrum(*v) for v in x[:c])
+        got = S.spectrum_l1(torch.as_tensor(img).cuda())
+        assert abs(got - want) <= 2.0 ** -43 * want, (c, got, want)
+
+
+@pytest.mark.parametrize("x0,x1", [(3e-13, 4e-13), (3e-20, 4e-20), (1.5e-30, 1e-31), (1e-12, 3e-25), (3e16, 4e16),
+                                   (2e30, 1.25e31), (1e15, 1e-3), (3.0, 4e-20), (0.0, 2e-15), (0.0, 0.0)])
+def test_spectrum_magnitudes_over_the_range(x0, x1):
+    """Magnitudes around and outside the range that the FP32 pairs take (1e-12 to 1e15)."""
+    img = np.array([x0, x1, 0, 0], np.float32).reshape(1, 4, 1)
+    got, want = S.spectrum_l1(torch.as_tensor(img).cuda()), _column_spectrum(x0, x1)
+    assert abs(got - want) <= 2.0 ** -43 * want, (got, want)
+
+
+@pytest.mark.parametrize("bad", [np.nan, np.inf, -np.inf])
+def test_spectrum_of_images_with_non_finite_values(bad):
+    img = np.ones((1, 8, 8), np.float32)
+    img[0, 3, 5] = bad
+    assert np.isnan(S.spectrum_l1(torch.as_tensor(img).cuda()))
