@@ -309,8 +309,10 @@ extern "C" gs_status_t gs_downscale(const float *image, int32_t C, int32_t H, in
                                     gs_stream_t stream) {
   if (!image || !out || C <= 0 || H <= 0 || W <= 0 || r < 1) return GS_ERR_INVALID_ARG;
   const int Hr = gs_downscaled_size(H, r), Wr = gs_downscaled_size(W, r);
-  // taps per axis: at most 2 s + 1 with s = W / Wr <= 1.5 r (Wr rounds W / r down to half)
-  const int64_t taps = 2 * (int64_t)std::max((W + Wr - 1) / Wr, (H + Hr - 1) / Hr) + 1;
+  // taps per axis: at most 2 s + 1 with s = W / Wr <= 1.5 r (Wr rounds W / r down to half), and
+  // one more by the FP32 rounding of the positions up to 2^22 columns or rows; beyond, any number
+  int64_t taps = kMaxTaps + 1;
+  if (W <= 1 << 22 && H <= 1 << 22) taps = 2 * (int64_t)std::max((W + Wr - 1) / Wr, (H + Hr - 1) / Hr) + 2;
   const dim3 blocks((Wr + kDsX - 1) / kDsX, (Hr + kDsY - 1) / kDsY, C);
   if (taps <= kMaxTaps && blocks.y <= 65535 && blocks.z <= 65535) {
     downscale_taps_kernel<<<blocks, dim3(kDsX, kDsY), 0, as_stream(stream)>>>(image, H, W, out, Hr, Wr);

@@ -140,3 +140,25 @@ def test_spectrum_of_images_with_non_finite_values(bad):
     img = np.ones((1, 8, 8), np.float32)
     img[0, 3, 5] = bad
     assert np.isnan(S.spectrum_l1(torch.as_tensor(img).cuda()))
+
+
+def test_downscale_of_an_image_wider_than_fp32_positions():
+    """2^28 columns at scale 17: the positions' FP32 rounding widens some filters to 37 taps, one more
+    than the tabulated kernel has room for. Sampled columns against the filter's definition in FP32,
+    whose position (j + 1/2) s - 1/2 may be one or two roundings."""
+    n, r, f = 1 << 28, 17, np.float32
+    x = torch.rand(1, 1, n, generator=torch.Generator("cuda").manual_seed(5), device="cuda")
+    got = S.downscale(x, r)[0, 0]
+    m = got.shape[0]
+    rng = np.random.default_rng(6)
+    s = f(n) / f(m)
+    widest = 0
+    for j in np.concatenate([rng.integers(0, m, 300), np.arange(m - 100, m)]):
+        err = []
+        for c in ((f(j) + f(0.5)) * s - f(0.5), f(np.float64(f(j) + f(0.5)) * np.float64(s) - 0.5)):
+            k0, k1 = max(0, int(np.ceil(c - s))), min(n - 1, int(np.floor(c + s)))
+            w = np.maximum(f(0), f(1) - np.abs(np.arange(k0, k1 + 1).astype(f) - c) / s).astype(np.float64)
+            err.append(abs(float(got[j]) - (w * x[0, 0, k0:k1 + 1].cpu().numpy().astype(np.float64)).sum() / w.sum()))
+            widest = max(widest, k1 - k0 + 1)
+        assert min(err) < 1e-5, j
+    assert widest == 37
