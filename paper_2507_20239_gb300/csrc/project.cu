@@ -140,7 +140,7 @@ __device__ __forceinline__ void camera_centre(const gs_camera_t &cam, float &cx,
   cz = -(W[2] * cam.t[0] + W[5] * cam.t[1] + W[8] * cam.t[2]);
 }
 
-// One view (kept in one piece: through the functions below it took 87 instead of 81 us at 1.5M
+// A thread per record: one view, and several views of few Gaussians (kept in one piece: through the functions below it took 87 instead of 81 us at 1.5M
 // Gaussians, degree 3). VEC: the SH rows start on 16-byte boundaries (sh_stride a multiple of 4), so a
 // thread reads its row as float4s: 4 coefficients x 3 channels per three loads.
 template <int DEG, bool VEC>
@@ -339,10 +339,10 @@ __device__ __forceinline__ void view_direction(const gs_camera_t &cam, float mx,
   dz *= il;
 }
 
-// Several views: a thread takes a Gaussian through all of them, so that its parameters are read
-// and its covariance factor formed once (its SH row when the first view sees it), not once per
-// view from HBM. Bound by the records written. 5M Gaussians, 4 views: 830 -> 533 us; 500k, 12
-// views: 239 -> 133
+// Several views of many Gaussians (views_at_once): a thread takes a Gaussian through all of them, so
+// that its parameters are read and its covariance factor formed once (its SH row when the first view
+// sees it), not once per view from HBM. Bound by the records written. 5M Gaussians, 4 views:
+// 830 -> 533 us; 500k, 12 views: 239 -> 133.
 template <int DEG, bool VEC>
 __global__ void __launch_bounds__(128, 4) project_fwd_views_kernel(gs_params_t P, const gs_camera_t *__restrict__ cams,
                                                                   int n_views, int tile_w, int tile_h, gs_proj_t out) {
@@ -772,6 +772,16 @@ static int grid_for(int64_t n, int threads) {
   return (int)(want < 1 ? 1 : (want > cap ? cap : want));
 }
 
+// Whether a thread takes its Gaussian through every view (project_fwd_views_kernel) or one record
+// (project_fwd_kernel). With few Gaussians the views in turn are what it costs: per record -> all
+// views at 2k Gaussians, degree 3, 5.1 -> 7.9 us (4 views), 5.0 -> 15.1 (12), 8.8 -> 64.6 (64); at 20k
+// 7.8 -> 8.3, 13.4 -> 17.0, 46.6 -> 73.9. Half a round of threads (of 512 an SM) makes up for it where the
+// rows are long: 40k, degree 3, 10.9 -> 9.4, 21.2 -> 18.7, 89.6 -> 82.9; with the short rows of degrees 0
+// and 1 two rounds do (degree 0, 64 views: 75 -> 92 at 60k, 142 -> 162 at 120k, 188 -> 186 at 160k).
+static bool views_at_once(int n_views, int64_t n, int degree) {
+  return n_views > 1 && n >= (degree >= 2 ? 256 : 1024) * (int64_t)num_sms();
+}
+
 }  // namespace gs
 
 using namespace gs;
@@ -788,9 +798,10 @@ extern "C" gs_status_t gs_project(const gs_params_t *params, const gs_frame_t *f
   cudaStream_t s = as_stream(stream);
   const bool vec = params->sh_stride % 4 == 0 && aligned16(params->sh);
 #define GS_PROJ_FWD(D)                                                                                          \
-  if (frame->n_views == 1) {                                                                                    \
+  if (!views_at_once(frame->n_views, params->n, D)) {                                                           \
     auto kern = vec ? project_fwd_kernel<D, true> : project_fwd_kernel<D, false>;                               \
-    kern<<<grid_for(params->n, 256), 256, 0, s>>>(*params, frame->cams_dev, 1, frame->tile_w, frame->tile_h, *out); \
+    kern<<<grid_for(R, 256), 256, 0, s>>>(*params, frame->cams_dev, frame->n_views, frame->tile_w,               \
+                                          frame->tile_h, *out);                                                  \
   } else {                                                                                                      \
     auto kern = vec ? project_fwd_views_kernel<D, true> : project_fwd_views_kernel<D, false>;                    \
     kern<<<grid_for(params->n, 128), 128, 0, s>>>(*params, frame->cams_dev, frame->n_views, frame->tile_w,       \

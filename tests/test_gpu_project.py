@@ -221,3 +221,24 @@ def test_project_of_several_views_equals_each_view(n, degree, stored):
         for k in ("mean2d", "conic_opacity", "rgb", "depth", "radius", "rect", "clamped"):
             assert torch.equal(getattr(got, k)[v * n:(v + 1) * n], getattr(want, k)), (v, k)
     assert n < 100 or n < seen < 4 * n
+
+
+@pytest.mark.parametrize("degree,stored", [(0, 1), (1, 4), (2, 9), (3, 16)])
+@pytest.mark.parametrize("more", [-1, 0, 129])
+def test_project_of_several_views_around_the_line_between_its_kernels(degree, stored, more):
+    """Counts on both sides of views_at_once's line, bit for bit the records of one-view frames."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    n = (256 if degree >= 2 else 1024) * sms + more
+    g = torch.Generator("cuda").manual_seed(7)
+    norm = lambda *s: torch.randn(*s, generator=g, device="cuda")   # noqa: E731
+    P = dict(means=1.5 * norm(n, 3), log_scales=-4 + 0.7 * norm(n, 3), quats=norm(n, 4), opacity_logits=norm(n) - 2,
+             sh=0.3 * norm(n, stored, 3))
+    cams = [synth.orbit_camera(4.0 - v, 0.3 + 1.9 * v, 15.0, 200 - 40 * v, 150, 180.0) for v in range(3)]
+    got = R.project(P, degree, R.Frame(cams))
+    seen = 0
+    for v, cam in enumerate(cams):
+        want = R.project(P, degree, R.Frame([cam]))
+        seen += int((want.radius > 0).sum())
+        for k in ("mean2d", "conic_opacity", "rgb", "depth", "radius", "rect", "clamped"):
+            assert torch.equal(getattr(got, k)[v * n:(v + 1) * n], getattr(want, k)), (v, k)
+    assert 0.3 * n < seen < 2.9 * n
