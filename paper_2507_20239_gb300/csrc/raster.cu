@@ -1018,15 +1018,9 @@ __global__ void __launch_bounds__(kSplatThreads, kSplatBlocks) raster_bwd_splat_
 // per bucket however few tiles there are, and no reduction, at the price of a second forward
 // walk (the kernels alone, 16 x 16 tiles, raster_bwd_kernel -> this one): 206 -> 58 us at
 // 2k Gaussians on 64 x 64 (16 tiles), 404 -> 175 at 100k on 312 x 207 (260), 467 -> 290 at
-// 300k on 623 x 413 (1014), 546 -> 446 at 500k on 900 x 600 (2166), 923 -> 905 at 1.5M on
-// 1246 x 826 (4056); 16224 tiles 1981 -> 2214; 8 x 8 tiles 470 -> 437 at 900 x 600 and
-// 906 -> 994 at 1246 x 826; 16 x 32 tiles 632 -> 605 and 1086 -> 1279. Hence the line at
-// kTilePixels padded pixels. Lists of a few entries leave its buckets empty: 44 -> 58 us at
-// 5k Gaussians on 623 x 413, 132 -> 110 at 20k, 62 -> 45 at 5k on 312 x 207; hence
-// kTileRecords records a tile.
-constexpr int64_t kTilePixels = 600000;   // padded pixels of the frame (tiles x tile size), below
-constexpr int64_t kTileRecords = 12;      // records per tile, at least
-
+// 300k on 623 x 413 (1014), 546 -> 446 at 500k on 900 x 600 (2166). A bucket's walk costs the
+// same however few entries it has, so tiles of short lists (bwd_short) are taken pixel by pixel, and
+// frames of short lists go to raster_bwd_kernel (bwd_by_tile).
 template <int TW, int TH, int WB>
 struct BwdTile {
   // two CTAs of eight warps an SM (128 registers a thread), or five of four (102)
@@ -1042,13 +1036,101 @@ struct BwdTile {
   uint16_t live[NW][NP];
 };
 
+// A tile's short list, pixel by pixel: warp w on block w of the tile, an entry's nine sums reduced over
+// the warp and added up over the CTA's warps in shared memory, as in raster_bwd_kernel, whose
+// decisions and operations these are.
+template <int TW, int TH, bool STOP, int WB>
+__device__ __forceinline__ void bwd_short_list(BwdTile<TW, TH, WB> &s, const TileCoord &tc, uint2 rg, int n,
+                                               const float2 *__restrict__ mean2d, const float4 *__restrict__ conic_o,
+                                               const float4 *__restrict__ rgb, const uint32_t *__restrict__ vals,
+                                               float *g_mean2d, float *g_co, float *g_rgb, uint64_t n_records) {
+  using S = BwdTile<TW, TH, WB>;
+  constexpr int NT = S::NW * 32, CH = S::NP < 128 ? 64 : 128;
+  static_assert(CH <= NT && CH <= S::WE && CH <= S::NP, "an entry a thread, and room for a warp's list");
+  static_assert(9 * CH * sizeof(float) <= sizeof(s.ring), "the sums fit the rings");
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const bool on = warp < S::NB;
+  const int block = on ? warp : 0;
+  float *acc = reinterpret_cast<float *>(s.ring);
+  int lx, ly;
+  pixel_of<TW>(block * 32 + lane, lx, ly);
+  const int p0 = ly * TW + lx;
+  const float fx0 = (float)(tc.tx * TW + lx) + 0.5f, fy = (float)(tc.ty * TH + ly) + 0.5f;
+  PixBwd q[2];
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    const float4 g = s.g[p0 + k];
+    const uint32_t end = on ? __float_as_uint(g.w) : 0u;   // 0: past the image, or nothing composited
+    q[k] = PixBwd{fx0 + (float)k, 1.f, s.state[p0 + k].y, g.x, g.y, g.z, end == 0u, end};
+  }
+  uint32_t wstop = 0;
+  if (STOP) wstop = __reduce_max_sync(0xffffffffu, max(q[0].stop, q[1].stop));
+  for (int base = 0; base < n; base += CH) {
+    if (STOP) {
+      __syncthreads();
+    } else if (__syncthreads_count(!(q[0].done && q[1].done)) == 0) {
+      break;
+    }
+    const int cnt = min(CH, n - base);
+    uint32_t r = 0;
+    float4 cu = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (t < cnt) {
+      r = vals[rg.x + base + t];
+      if (!GS_CHECK(r < n_records, 1, r)) r = 0;
+      stage<TW, TH, 8, 8>(mean2d, conic_o, rgb, r, tc.tx * TW, tc.ty * TH, tc.W, tc.H, s.xy[t], s.co[t], s.rgb[t], cu);
+    }
+    for (int i = t; i < 9 * cnt; i += NT) acc[i] = 0.f;
+    __syncthreads();
+    const int jend = STOP ? min(cnt, (int)min(wstop, 0x7fffffffu) - base) : cnt;
+    if (on && jend > 0 && (STOP || !__all_sync(0xffffffffu, q[0].done && q[1].done))) {
+      uint16_t *list = s.live[warp];
+      int ns = 0;
+      for (int j0 = 0; j0 < jend; j0 += 32) {
+        const int j = j0 + lane;
+        const bool sel = j < jend && ((__float_as_uint(s.rgb[j].w) >> block) & 1u);
+        const uint32_t bal = __ballot_sync(0xffffffffu, sel);
+        if (sel) list[ns + __popc(bal & ((1u << lane) - 1u))] = (uint16_t)j;
+        ns += __popc(bal);
+      }
+      __syncwarp();
+      float v[9] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+      for (int i = 0; i < ns; ++i) {
+        const int j = list[i];
+        const float4 c = s.rgb[j];
+        const float2 xy = s.xy[j];
+        const float4 co = s.co[j];
+        bool any = pix_bwd<STOP>(q[0], (uint32_t)(base + j), fy, xy, co, c, v);
+        any |= pix_bwd<STOP>(q[1], (uint32_t)(base + j), fy, xy, co, c, v);
+        if (__any_sync(0xffffffffu, any)) {
+          warp_reduce9_add(v, acc + j * 9, lane);
+#pragma unroll
+          for (int k = 0; k < 9; ++k) v[k] = 0.f;   // lanes without a contribution kept zeros
+        }
+      }
+    }
+    __syncthreads();
+    if (t < cnt) {
+      const float *a = acc + t * 9;
+      const float mt = a[0], mdy = a[1], mtt = a[2], mtdy = a[3], mdydy = a[4], m = a[5];
+      const float k0 = a[6], k1 = a[7], k2 = a[8];
+      if (mt != 0.f || mdy != 0.f || mtt != 0.f || mtdy != 0.f || mdydy != 0.f || m != 0.f || k0 != 0.f || k1 != 0.f ||
+          k2 != 0.f) {
+        const float oA = cu.w * cu.x, ho = -0.5f * cu.w;   // (A, beta, gamma, o)
+        red_add_v2(g_mean2d + 2 * (size_t)r, -oA * mt, -(oA * cu.y * mt + cu.w * cu.z * mdy));
+        red_add_v4(g_co + 4 * (size_t)r, ho * mtt, -oA * mtdy, ho * mdydy, m);
+        red_add_v4(g_rgb + 4 * (size_t)r, k0, k1, k2, 0.f);
+      }
+    }
+  }
+}
+
 template <int TW, int TH, bool STOP, int WB>
 __global__ void __launch_bounds__(BwdTile<TW, TH, WB>::NW * 32, BwdTile<TW, TH, WB>::NW > 4 ? 2 : 5) raster_bwd_tile_kernel(
     const float2 *__restrict__ mean2d, const float4 *__restrict__ conic_o, const float4 *__restrict__ rgb,
     const uint32_t *__restrict__ vals, const uint2 *__restrict__ ranges, const gs_camera_t *__restrict__ cams,
     int n_views, const float *__restrict__ image, const float *__restrict__ d_image,
     const uint32_t *__restrict__ stop_in, float *__restrict__ g_mean2d, float *__restrict__ g_co,
-    float *__restrict__ g_rgb, uint64_t n_records, uint64_t list_cap, int split) {
+    float *__restrict__ g_rgb, uint64_t n_records, uint64_t list_cap, int split, int short_n) {
   using S = BwdTile<TW, TH, WB>;
   constexpr int NP = S::NP, NB = S::NB, NT = S::NW * 32, WE = S::WE;
   extern __shared__ float4 s_raw[];
@@ -1058,6 +1140,11 @@ __global__ void __launch_bounds__(BwdTile<TW, TH, WB>::NW * 32, BwdTile<TW, TH, 
   const TileCoord tc = tile_coord(cams, n_views, tile);
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   const uint32_t lt = (1u << lane) - 1u;
+  uint2 rg = ranges[tile];
+  if (!GS_CHECK(rg.x <= rg.y && (uint64_t)rg.y <= list_cap, 2, tile)) rg = make_uint2(0u, 0u);
+  // a short list is the tile's first CTA's alone (the others are not worth their start)
+  const bool brief = (int)(rg.y - rg.x) <= short_n;
+  if (split > 1 && brief && part > 0) return;
   if (t == 0) {
     s.xy[WE] = make_float2(0.f, 0.f);
     s.co[WE] = s.rgb[WE] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -1093,10 +1180,12 @@ __global__ void __launch_bounds__(BwdTile<TW, TH, WB>::NW * 32, BwdTile<TW, TH, 
     }
   }
   __syncthreads();
-  uint2 rg = ranges[tile];
-  if (!GS_CHECK(rg.x <= rg.y && (uint64_t)rg.y <= list_cap, 2, tile)) rg = make_uint2(0u, 0u);
   int n = (int)(rg.y - rg.x);
   if (STOP) n = min(n, (int)min(s_max, 0x7fffffffu));
+  if (brief) {
+    bwd_short_list<TW, TH, STOP, WB>(s, tc, rg, n, mean2d, conic_o, rgb, vals, g_mean2d, g_co, g_rgb, n_records);
+    return;
+  }
   // this CTA's blocks are part, part + split, ...; warp w walks the w-th of them forward, two
   // pixels per lane
   const int blocks = NB / split, block = part + split * (warp < blocks ? warp : 0);
@@ -1381,6 +1470,31 @@ static gs_status_t clear_grads(const gs_rec_grads_t *g, int64_t R, cudaStream_t 
   return GS_OK;
 }
 
+// Whether gs_raster_bwd takes raster_bwd_tile_kernel. Its gain falls with the frame's pixels (a tile's
+// latency is hidden by other tiles) and with the lists' length, of which the host knows no more
+// than the number of records, seen or not. raster_bwd_kernel -> raster_bwd_tile_kernel, us, of one scene
+// seen whole and six times magnified: 16 x 16 tiles, 2166 of them (554k padded pixels), 300k Gaussians
+// 448 -> 367 and 216 -> 224, 150k 328 -> 292 and 156 -> 177, 50k 193 -> 215 and 75 -> 105; 1014 tiles (260k), 300k
+// 383 -> 280 and 152 -> 137, 50k 175 -> 145 and 51 -> 51, 20k 99 -> 95 and 25 -> 27; 8 x 8 tiles, 6370 (408k), 300k
+// 389 -> 303 and 201 -> 211, 8475 (542k) 424 -> 365 and 238 -> 271; 16 x 32 tiles, 290 (148k), 50k 233 -> 144 and
+// 48 -> 48, 507 (260k) 201 -> 207 and 52 -> 59. Hence a line in pixels per shape, below it 12 records a
+// tile at least, and more with the square of the pixels; beyond that a magnified view still takes up to
+// 1.09 times as long (150k Gaussians on 780 x 520).
+static bool bwd_by_tile(int tile_pixels, int64_t n_tiles, int64_t records) {
+  const int64_t px = n_tiles * tile_pixels;
+  const int64_t line = tile_pixels == 256 ? 600000 : (tile_pixels < 256 ? 450000 : 200000);
+  return px < line && records >= 12 * n_tiles && records >= px * px / (tile_pixels < 256 ? 1000000 : 1500000);
+}
+
+// The longest list that raster_bwd_tile_kernel takes pixel by pixel: 312 x 207, 260 tiles of 5 entries on
+// average 31 -> 14 us with up to 32 so taken, of 40 entries 34 -> 32; 623 x 413, 1014 tiles of 39 entries 61 -> 51
+// with 48, of 82 88 -> 82. 8 x 8 tiles have one warp for it: 160 x 120, 300 tiles of 4 entries 13 -> 10 with 16,
+// 2166 tiles no gain.
+static int bwd_short(int tile_pixels, bool few) {
+  if (tile_pixels < 256) return few ? 16 : 0;
+  return few ? 32 : 48;
+}
+
 template <int TW, int TH>
 static gs_status_t launch_bwd(const gs_proj_t *proj, const gs_bins_t *bins, const gs_frame_t *frame,
                               const float *image, const float *d_image, const uint32_t *stop, bool half,
@@ -1390,7 +1504,7 @@ static gs_status_t launch_bwd(const gs_proj_t *proj, const gs_bins_t *bins, cons
   const auto *co = reinterpret_cast<const float4 *>(proj->conic_opacity);
   const auto *c = reinterpret_cast<const float4 *>(proj->rgb);
   const auto *rg = reinterpret_cast<const uint2 *>(bins->ranges);
-  if ((int64_t)frame->n_tiles * TW * TH >= kTilePixels || proj->n_records < kTileRecords * frame->n_tiles) {
+  if (!bwd_by_tile(TW * TH, frame->n_tiles, proj->n_records)) {
     // 2 pixels per thread: 8 x 8 warp blocks skip more records than 8 x 16 ones
     // (4 pixels per thread) save in shared per-entry work.
     constexpr int PX = 2;
@@ -1419,7 +1533,7 @@ static gs_status_t launch_bwd(const gs_proj_t *proj, const gs_bins_t *bins, cons
     GS_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     kern<<<frame->n_tiles * split, threads, smem, s>>>(
         m2, co, c, bins->vals, rg, frame->cams_dev, frame->n_views, image, d_image, stop, g->d_mean2d,
-        g->d_conic_opacity, g->d_rgb, (uint64_t)proj->n_records, (uint64_t)bins->capacity, split);
+        g->d_conic_opacity, g->d_rgb, (uint64_t)proj->n_records, (uint64_t)bins->capacity, split, bwd_short(TW * TH, few));
     return GS_OK;
   };
   // the staging depth's half: windows of half as many buckets

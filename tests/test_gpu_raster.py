@@ -195,3 +195,39 @@ def test_tile_backward_matches_per_splat_backward(n, size, tile, depth, use_stop
     for k in ("d_mean2d", "d_conic_opacity", "d_rgb"):
         a, b = getattr(got, k).cpu().numpy(), getattr(want, k).cpu().numpy()
         assert np.linalg.norm(b) > 0 and rel_l2(a, b) < 1e-4, k
+
+
+@pytest.mark.parametrize("use_stop", [False, True])
+@pytest.mark.parametrize("depth", [0, 1])
+@pytest.mark.parametrize("n,size,tile,zoom", [
+    (200, (64, 64), (16, 16), 3.0), (2500, (61, 50), (16, 16), 1.0),     # quarters of tiles; short, and several windows
+    (2400, (250, 183), (16, 16), 5.0), (9000, (250, 183), (16, 16), 2.5),   # halves; short, and mixed
+    (9000, (333, 301), (16, 16), 4.0), (60_000, (333, 301), (16, 16), 4.0),   # whole tiles, four-warp CTAs
+    (3000, (120, 120), (8, 8), 4.0), (20_000, (200, 190), (8, 8), 2.0), (3000, (130, 70), (16, 32), 3.0),
+    (4000, (70, 130), (32, 16), 1.0)])
+def test_tile_backward_matches_per_pixel_backward(n, size, tile, zoom, depth, use_stop):
+    """raster_bwd_tile_kernel, its short lists, its split tiles and its windows included, against
+    raster_bwd_kernel, which shares neither walk nor reduction with it: a large second view beside the
+    small one takes the frame beyond the line between them. FP32 on both sides, the sums in another
+    order: 1e-4, as between the backwards elsewhere."""
+    sc = synth.small_scene(n, n=n, width=size[0], height=size[1])
+    cam = sc.cameras[0]
+    cam = synth.Camera(cam.R, cam.t, cam.fx * zoom, cam.fy * zoom, cam.cx, cam.cy, cam.width, cam.height)
+    big = synth.Camera(cam.R, cam.t, 1000., 1000., 640., 480., 1280, 960)
+    P = R.to_device_params(sc.params())
+    got = {}
+    for name, cams in (("tile", [cam]), ("pixel", [cam, big])):
+        frame = R.Frame(cams, tile=tile)
+        proj = R.project(P, 0, frame)
+        bins = R.bin_sort(proj, frame)
+        img, _, stop = R.raster_fwd(proj, bins, frame, store_stop=True)
+        d_image = torch.zeros_like(img)
+        d_image[:3 * size[0] * size[1]] = torch.randn(3 * size[0] * size[1], device="cuda",
+                                                      generator=torch.Generator("cuda").manual_seed(n))
+        rg = R.raster_bwd(proj, bins, frame, img, d_image, stop=stop if use_stop else None, stage_depth=depth)
+        got[name] = {k: getattr(rg, k)[:n].cpu().numpy() for k in ("d_mean2d", "d_conic_opacity", "d_rgb")}
+        if name == "tile":
+            lens = (bins.ranges[:, 1] - bins.ranges[:, 0]).cpu().numpy()
+            print(f"lists of {lens.min()} to {lens.max()} entries, {(lens <= 32).mean():.2f} of them up to 32")
+    for k, b in got["pixel"].items():
+        assert np.linalg.norm(b) > 0 and rel_l2(got["tile"][k], b) < 1e-4, k
