@@ -428,12 +428,15 @@ __device__ __forceinline__ void adam_group(int grp, const gs_params_out_t &P, co
 // Bound by HBM. The grid is what the device keeps resident, and takes one group after the other:
 // a grid of eight blocks per SM and group ran as one full round and a partial one
 // (1.2M Gaussians, degree 3, 64% seen: 306 -> 274 us, 300k 91 -> 79; six blocks per SM and group
-// 348 us, 64 of them 419, four resident instead of five 300).
+// 348 us, 64 of them 419, four resident instead of five 300). With few parameters each group
+// has blocks of its own (gridDim.y): one group after the other is then five round trips to memory
+// in turn (500 Gaussians, degree 3, 30% seen, 8.0 -> 5.1 us; 10k of degree 0 7.8 -> 5.4; at 10k of
+// degree 3 one after the other 9.8 against 20).
 __global__ void __launch_bounds__(256, 5) adam_kernel(gs_params_out_t P, gs_param_grads_t G, gs_adam_state_t S, int64_t n, int32_t sh_width,
                             float5_t step_size, float beta1, float beta2, float eps, float sqrt_bc2,
                             const int32_t *__restrict__ radius, int32_t n_views) {
 #pragma unroll 1
-  for (int grp = 0; grp < 5; ++grp)
+  for (int grp = blockIdx.y; grp < 5; grp += gridDim.y)
     adam_group(grp, P, G, S, n, sh_width, step_size.v[grp], beta1, beta2, eps, sqrt_bc2, radius, n_views);
 }
 
@@ -499,8 +502,10 @@ extern "C" gs_status_t gs_adam_step(const gs_adam_cfg_t *cfg, gs_params_out_t *p
   const int64_t widest = n * 3 * (int64_t)sh_stride;
   int per_sm = 0;
   GS_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, adam_kernel, 256, 0));
-  const int gx = (int)std::min<int64_t>((widest + 255) / 256, (int64_t)num_sms() * std::max(per_sm, 1));
-  adam_kernel<<<gx, 256, 0, as_stream(stream)>>>(*params, *grads, *state, n, 3 * sh_stride, ss, (float)cfg->beta1,
+  const int64_t blocks = (widest + 255) / 256;
+  const bool few = blocks <= 2 * num_sms();   // five groups of them: two rounds at most
+  const dim3 grid((unsigned)std::min<int64_t>(blocks, (int64_t)num_sms() * std::max(per_sm, 1)), few ? 5 : 1);
+  adam_kernel<<<grid, 256, 0, as_stream(stream)>>>(*params, *grads, *state, n, 3 * sh_stride, ss, (float)cfg->beta1,
                                                  (float)cfg->beta2, cfg->eps, (float)std::sqrt(bc2), radius, n_views);
   GS_LAUNCH_CHECK();
   return GS_OK;

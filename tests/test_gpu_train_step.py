@@ -108,3 +108,32 @@ def test_opacity_reset_matches_oracle():
     assert np.array_equal(P["opacity_logits"].cpu().numpy(), want)
     assert np.allclose(want, oopt.opacity_reset(lg), atol=1e-7)
     assert float(opt.m["opacity_logits"].abs().max()) == 0.0
+
+
+@pytest.mark.parametrize("sparse", [False, True])
+@pytest.mark.parametrize("K", [1, 9, 16])
+@pytest.mark.parametrize("side", ["one", "below", "above"])
+def test_adam_step_around_the_line_between_its_grids(side, K, sparse):
+    """A group per block row up to two blocks an SM of SH values, one group after the other beyond; every
+    element against the FP64 update, tolerances as above."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    line = 2 * sms * 256 // (3 * K)
+    n = dict(one=1, below=line, above=line + 1)[side]
+    rng = np.random.default_rng(n + K)
+    p = {k: v.astype(np.float32) for k, v in _params(rng, n, K).items()}
+    g = {k: rng.normal(size=v.shape).astype(np.float32) for k, v in p.items()}
+    lrs = {"means": 7e-4, "log_scales": 5e-3, "quats": 1e-3, "opacity_logits": 5e-2, "sh": 2.5e-3}
+    radius = np.where(rng.uniform(size=n) < 0.5, 3, 0).astype(np.int32)
+    dev = lambda a: torch.as_tensor(np.ascontiguousarray(a)).cuda()
+    P = {k: dev(v) for k, v in p.items()}
+    opt = O.Adam(P, lrs)
+    opt.m = {k: dev(np.full_like(v, 1e-3)) for k, v in p.items()}
+    opt.v = {k: dev(np.full_like(v, 1e-2)) for k, v in p.items()}
+    opt.t = 4
+    opt.step(P, {k: dev(v) for k, v in g.items()}, radius=dev(radius) if sparse else None)
+    for k in p:
+        wp, wm, wv = oopt.adam_step(p[k], g[k], np.full_like(p[k], 1e-3), np.full_like(p[k], 1e-2), lrs[k], 5,
+                                    visible=radius > 0 if sparse else None)
+        for got, want in ((P[k], wp), (opt.m[k], wm), (opt.v[k], wv)):
+            got = got.cpu().numpy()
+            assert np.all(np.abs(got - want) <= 2e-6 * (np.abs(want) + np.abs(g[k]))), k
