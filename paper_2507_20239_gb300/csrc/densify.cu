@@ -94,21 +94,22 @@ __device__ __forceinline__ void kth_find(int shift, double ratio, SelectState *s
   __syncthreads();
 }
 
-__device__ __forceinline__ float tau_of(const gs_densify_cfg_t &cfg, const SelectState *st) {
-  return cfg.prune_adaptive ? fminf(from_ordered_bits(st->prefix), cfg.prune_upper_logit) : cfg.prune_logit;
-}
-
-// Masks and the post-densification count; for adaptive pruning also the first step of the
-// radix select (the highest byte's histogram, weighted by multiplicity, and its bucket).
+// Masks; for adaptive pruning (ADAPT) also the post-densification count and the first step of the
+// radix select (the highest byte's histogram, weighted by multiplicity, and its bucket), else the
+// threshold, which is given (a sum and a last block for it too took 2 us).
+template <bool ADAPT>
 __global__ void __launch_bounds__(kSelThreads) select_kernel(gs_densify_cfg_t cfg, const float *__restrict__ log_scales,
                                                              const float *__restrict__ logits,
                                                              const float *__restrict__ accum,
                                                              const int32_t *__restrict__ count, int64_t n,
                                                              uint8_t *__restrict__ split, uint8_t *__restrict__ clone,
                                                              SelectState *st, float *tau) {
-  __shared__ uint32_t h[256];
-  h[threadIdx.x] = 0;
-  __syncthreads();
+  __shared__ uint32_t h[ADAPT ? 256 : 1];
+  if (!ADAPT && blockIdx.x == 0 && threadIdx.x == 0) *tau = cfg.prune_logit;
+  if (ADAPT) {
+    h[threadIdx.x] = 0;
+    __syncthreads();
+  }
   unsigned long long post = 0;
   for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < n; g += (int64_t)gridDim.x * blockDim.x) {
     const int32_t c = count[g];
@@ -127,16 +128,14 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(gs_densify_cfg_t cf
     clone[g] = cl;
     const uint32_t w = (sp || cl) ? 2u : 1u;
     post += w;
-    if (cfg.prune_adaptive) atomicAdd(&h[ordered_bits(logits[g]) >> 24], w);
+    if (ADAPT) atomicAdd(&h[ordered_bits(logits[g]) >> 24], w);
   }
-  block_add_u64(post, &st->n_post);
-  __syncthreads();
-  if (h[threadIdx.x]) atomicAdd(&st->hist[threadIdx.x], h[threadIdx.x]);
-  if (!last_block(st)) return;
-  if (cfg.prune_adaptive)
-    kth_find(24, cfg.prune_ratio, st);
-  else if (threadIdx.x == 0)
-    *tau = tau_of(cfg, st);
+  if (ADAPT) {
+    block_add_u64(post, &st->n_post);
+    __syncthreads();
+    if (h[threadIdx.x]) atomicAdd(&st->hist[threadIdx.x], h[threadIdx.x]);
+    if (last_block(st)) kth_find(24, cfg.prune_ratio, st);
+  }
 }
 
 // Radix select, most significant byte first: histogram of the current byte over
@@ -160,7 +159,7 @@ __global__ void __launch_bounds__(kSelThreads) kth_hist_kernel(gs_densify_cfg_t 
   if (h[threadIdx.x]) atomicAdd(&st->hist[threadIdx.x], h[threadIdx.x]);
   if (!last_block(st)) return;
   kth_find(shift, cfg.prune_ratio, st);
-  if (shift == 0 && threadIdx.x == 0) *tau = tau_of(cfg, st);
+  if (shift == 0 && threadIdx.x == 0) *tau = fminf(from_ordered_bits(st->prefix), cfg.prune_upper_logit);
 }
 
 __global__ void __launch_bounds__(kSelThreads) count_keep_kernel(const float *__restrict__ logits,
@@ -532,7 +531,8 @@ static gs_status_t select_launches(const gs_densify_cfg_t &cfg, const float *log
                                    const float *accum, const int32_t *count, int64_t n, uint8_t *split, uint8_t *clone,
                                    float *tau, int64_t *d_new_n, SelectState *st, cudaStream_t s) {
   const int G = dgrid(n);
-  select_kernel<<<G, kSelThreads, 0, s>>>(cfg, log_scales, logits, accum, count, n, split, clone, st, tau);
+  auto select = cfg.prune_adaptive ? select_kernel<true> : select_kernel<false>;
+  select<<<G, kSelThreads, 0, s>>>(cfg, log_scales, logits, accum, count, n, split, clone, st, tau);
   GS_LAUNCH_CHECK();
   if (cfg.prune_adaptive) {
     for (int shift = 16; shift >= 0; shift -= 8) {
