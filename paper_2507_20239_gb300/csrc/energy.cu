@@ -103,8 +103,14 @@ __global__ void __launch_bounds__(kDsX *kDsY) downscale_taps_kernel(const float 
 
 // tw[q] = exp(-2 pi i q / N), q in [0, N), of the rows (N = W) and of the columns (N = H),
 // computed once per call: the double-precision sines, done by every block of a DFT pass,
-// cost more than the pass (FP64 runs at 1/64 of the FP32 rate here).
-__global__ void twiddles_kernel(float2 *__restrict__ tw_w, int W, float2 *__restrict__ tw_h, int H) {
+// cost more than the pass (FP64 runs at 1/64 of the FP32 rate here). Blocks of one warp: the FP64
+// pipes of many SMs instead of one. Clears the sum as well (a launch less; the two together 64 x 64
+// 16.3 -> 12.8 us for the call, 3 x 623 x 413 90.6 -> 87.8).
+constexpr int kTwThreads = 32;
+
+__global__ void __launch_bounds__(kTwThreads) twiddles_kernel(float2 *__restrict__ tw_w, int W,
+                                                              float2 *__restrict__ tw_h, int H, double *sum) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) *sum = 0.0;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= W + H) return;
   const int N = i < W ? W : H, q = i < W ? i : i - W;
@@ -344,8 +350,7 @@ extern "C" gs_status_t gs_spectrum_l1(const float *image, int32_t C, int32_t H, 
   if (row_blocks > 0x7fffffffll || col_blocks > 0x7fffffffll) return GS_ERR_INVALID_ARG;
   float2 *X = static_cast<float2 *>(ws);
   float2 *tw_w = X + lines * K, *tw_h = tw_w + W;
-  GS_CUDA_TRY(cudaMemsetAsync(d_sum, 0, sizeof(double), s));
-  twiddles_kernel<<<(W + H + 127) / 128, 128, 0, s>>>(tw_w, W, tw_h, H);
+  twiddles_kernel<<<(W + H + kTwThreads - 1) / kTwThreads, kTwThreads, 0, s>>>(tw_w, W, tw_h, H, d_sum);
   GS_LAUNCH_CHECK();
   auto rows = [&](auto kernel, int per, int freqs) {
     const dim3 grid((unsigned)((lines + per - 1) / per), (K + kDftThreads * freqs - 1) / (kDftThreads * freqs));
