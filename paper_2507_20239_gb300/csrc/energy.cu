@@ -320,7 +320,13 @@ extern "C" gs_status_t gs_downscale(const float *image, int32_t C, int32_t H, in
   int64_t taps = kMaxTaps + 1;
   if (W <= 1 << 22 && H <= 1 << 22) taps = 2 * (int64_t)std::max((W + Wr - 1) / Wr, (H + Hr - 1) / Hr) + 2;
   const dim3 blocks((Wr + kDsX - 1) / kDsX, (Hr + kDsY - 1) / kDsY, C);
-  if (taps <= kMaxTaps && blocks.y <= 65535 && blocks.z <= 65535) {
+  // Steps of whole 32-byte sectors put 8 or 16 lanes of a load on one bank. On large images that is what both
+  // kernels take their time from, and the general one, whose blocks read along one row, takes less of it:
+  // tabulated and general, us, scale 8, 1 channel 4096 x 4096 94 / 84, 6000 x 4000 112 / 96, 3 channels 4096 x 3000
+  // 166 / 138, 6000 x 4000 299 / 273; 3200 x 2400 46 / 43 and 116 / 116, 2600 x 2000 36 / 34 and 87 / 92; scale 16, 3
+  // channels 4096 x 4096 422 / 392, 6000 x 4000 771 / 586. Other scales take the tables at any size.
+  const bool conflicts = r % 8 == 0 && (int64_t)H * W >= 7000000;
+  if (taps <= kMaxTaps && !conflicts && blocks.y <= 65535 && blocks.z <= 65535) {
     downscale_taps_kernel<<<blocks, dim3(kDsX, kDsY), 0, as_stream(stream)>>>(image, H, W, out, Hr, Wr);
   } else {
     const int64_t total = (int64_t)Hr * Wr;

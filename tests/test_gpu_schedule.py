@@ -162,3 +162,13 @@ def test_downscale_of_an_image_wider_than_fp32_positions():
             widest = max(widest, k1 - k0 + 1)
         assert min(err) < 1e-5, j
     assert widest == 37
+
+
+@pytest.mark.parametrize("shape,r", [((1, 2600, 2688), 8), ((1, 2600, 2696), 8), ((2, 2650, 2650), 16)])
+def test_downscale_of_large_images(shape, r):
+    """Scales of whole 32-byte steps below and above seven million pixels (the tabulated and the general
+    kernel); tolerance as above."""
+    img = _image(9, *shape)
+    got = S.downscale(torch.as_tensor(img).cuda(), r).cpu().numpy()
+    want = osch.downscale(img, r)
+    assert got.shape == want.shape and np.abs(got - want).max() < 1e-5
