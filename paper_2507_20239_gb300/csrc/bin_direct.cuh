@@ -693,8 +693,9 @@ __global__ void __launch_bounds__(kDirScanThreads) direct_scan_kernel(const DirA
 // of its own and no barriers: a record's rectangle over the lanes, record after record, 345 / 4198; the
 // hits spread over the lanes, those of a tile ranked by match.any, 234 / 1809.
 // W words of mask per tile: 4 W + 4 + 2 1/8 bytes of shared memory per tile of the view.
-constexpr int kEmitThreads = 256;
-constexpr uint32_t kEmitStage = 3 * kEmitThreads;   // units staged at a time, three loads a thread in flight
+// T threads a block: 256, and with one word of mask (more than 7,250 tiles a view, of which one or
+// two blocks fit an SM) 512: 5M-class frames of 10,736 tiles 3.56 -> 3.25 ms (1.5M in 4 views), of 16,224
+// 4.45 -> 4.00, 300k on 13,110 313 -> 290 us.
 
 inline size_t emit_smem(int words, int tiles) {
   return (4 * (size_t)words + 4 + 2) * tiles + 4 * (((size_t)tiles + 31) / 32) + 16;
@@ -713,9 +714,10 @@ __device__ __forceinline__ void take_mask(uint32_t *s, uint32_t m[W]) {
   }
 }
 
-template <int W>
-__global__ void __launch_bounds__(kEmitThreads, 1024 / kEmitThreads) direct_emit_kernel(const DirArgs a, uint32_t *__restrict__ vals) {
-  constexpr int kGroup = 32 * W, kGroups = kEmitThreads / kGroup;
+template <int W, int T>
+__global__ void __launch_bounds__(T, 1024 / T) direct_emit_kernel(const DirArgs a, uint32_t *__restrict__ vals) {
+  constexpr int kEmitThreads = T, kGroup = 32 * W, kGroups = kEmitThreads / kGroup;
+  constexpr uint32_t kEmitStage = 3 * kEmitThreads;   // units staged at a time, three loads a thread in flight
   extern __shared__ uint4 s_raw4[];
   __shared__ uint32_t s_pre[kEmitThreads + 1], s_off[kEmitThreads], s_rid[kEmitThreads];
   __shared__ uint32_t s_warp[kEmitThreads / 32];
@@ -743,7 +745,7 @@ __global__ void __launch_bounds__(kEmitThreads, 1024 / kEmitThreads) direct_emit
   OrderedRec next = begin + t < end ? ordered_record(a, seg, begin + t) : OrderedRec{0u, 0u, 0u};
   uint32_t turn = 0;
   for (uint32_t k0 = begin; k0 < end; k0 += kEmitThreads) {
-    // 512 records and the prefix of their rows
+    // the block's next records (one a thread) and the prefix of their rows
     const OrderedRec rec = next;
     const uint32_t kn = k0 + kEmitThreads + t;
     next = kn < end ? ordered_record(a, seg, kn) : OrderedRec{0u, 0u, 0u};
@@ -776,7 +778,7 @@ __global__ void __launch_bounds__(kEmitThreads, 1024 / kEmitThreads) direct_emit
       for (uint32_t from = u0; from < u1;) {
         if (from >= se || (u1 > se && from == u0)) {
           // units from here on: each the last record whose rows start at or before it, and its
-          // run there, as (tile | length << 16, record of the 512)
+          // run there, as (tile | length << 16, record of the block's)
           sb = from;
           se = min(all, sb + kEmitStage);
           __syncthreads();   // the previous units have been read
@@ -877,10 +879,19 @@ inline uint64_t dir_unit_cap(int64_t R, int64_t cap, int64_t unit_grid) {
 // Whether a frame takes this path, and its chunks: eight blocks per SM in all,
 // sixteen with several views, whose sizes may differ (12 views of a quarter to full size: 1165
 // us for the whole binning with eight, 1086 with sixteen; one view of 4056 tiles 426 and 447,
-// the matrix being longer to scan), of at least 64 records, and a matrix within its bound. Refused: views of more
-// tiles than the emission has shared memory for, sizes beyond the counters', less than a record a
-// view, and frames whose layout gs_frame_init has not written (a view's tables in shared memory
-// are sized by the largest view: max_width and max_height have to cover every view's tiles).
+// the matrix being longer to scan), of at least 64 records, 128 where a view has more than 10,000 tiles
+// and 4096 records (20k records in 4 views of 13,110 tiles 220 -> 184 us), and a matrix within its bound. Refused:
+//  - views of more tiles than the emission has shared memory for, sizes beyond the counters', less
+//    than a record a view, and frames whose layout gs_frame_init has not written (a view's tables in
+//    shared memory are sized by the largest view: max_width and max_height have to cover every view's);
+//  - more than 65,536 tiles in all and fewer than 12 records to each: what a chunk costs in tables and
+//    in the matrix goes by the tiles (general path -> this one: 2k records in each of 32 views of 4056 tiles
+//    127 -> 219 us, 20k 277 -> 364, 50k, 12.3 a tile, 564 -> 561; 20k in 12 views of 6700 203 -> 254, 100k 572 -> 551);
+//  - views of unequal sizes, the largest of more than 10,000 tiles, of 10k records and more: the small
+//    views' blocks hold as much shared memory as the large one's and have as many hits on few tiles
+//    (3 views of 10,736 tiles, a quarter and a sixteenth of that: 20k 136 -> 109 us, 100k 188 -> 250, 500k 503 -> 713;
+//    12 such views 20k 207 -> 247, 100k 519 -> 639; where the largest has 8475, 3 views 455 -> 505 at 500k, 12
+//    views 485 -> 455 at 100k, 2330 -> 1717 at 500k).
 inline DirPlan dir_plan(const gs_frame_t *f, int64_t R, int64_t cap) {
   DirPlan p{};
   if (f->n_views < 1 || f->n_views > kDirMaxViews || R < f->n_views || f->n_tiles < 1) return p;
@@ -889,6 +900,9 @@ inline DirPlan dir_plan(const gs_frame_t *f, int64_t R, int64_t cap) {
   const int64_t gx = ((int64_t)f->max_width + f->tile_w - 1) / f->tile_w;
   const int64_t gy = ((int64_t)f->max_height + f->tile_h - 1) / f->tile_h;
   if (gx * gy > kDirMaxTiles || gx * gy * f->n_views < f->n_tiles || n >= (1ll << 30)) return p;
+  if (f->n_tiles > 65536 && R < 12 * (int64_t)f->n_tiles) return p;
+  const bool large = gx * gy > 10000;
+  if (large && 4 * (int64_t)f->n_tiles < 3 * gx * gy * f->n_views && n >= 10000) return p;
   p.max_tiles = (int)(gx * gy);
   int64_t chunks = ((f->n_views > 1 ? 16ll : 8ll) * num_sms() + f->n_views - 1) / f->n_views;
   const int64_t groups = (n + kDirThreads - 1) / kDirThreads, by_matrix = kDirMatrix / f->n_tiles;
@@ -897,7 +911,7 @@ inline DirPlan dir_plan(const gs_frame_t *f, int64_t R, int64_t cap) {
   p.groups = (int)groups;
   p.ordered = chunks < groups;
   if (!p.ordered) {   // few records: equal shares of whole 64s, as many as fill the chunks
-    p.share = (uint32_t)(((n + chunks - 1) / chunks + 63) / 64 * 64);
+    p.share = (uint32_t)std::max<int64_t>(((n + chunks - 1) / chunks + 63) / 64 * 64, large && n >= 4096 ? 128 : 64);
     chunks = (n + p.share - 1) / p.share;
   }
   const int64_t batches = (n + 31) / 32 * f->n_views, grid = (batches + kDirWarps - 1) / kDirWarps;
@@ -1006,7 +1020,8 @@ inline gs_status_t dir_bin_sort(const gs_proj_t *proj, const gs_frame_t *f, gs_b
   // two words where two blocks or more fit an SM
   const int w = emit_smem(2, plan.max_tiles) <= 100 * 1024 ? 2 : 1;
   const size_t smem_e = emit_smem(w, plan.max_tiles);
-  auto emit = w == 2 ? direct_emit_kernel<2> : direct_emit_kernel<1>;
+  const int et = w == 2 ? 256 : 512;
+  auto emit = w == 2 ? direct_emit_kernel<2, 256> : direct_emit_kernel<1, 512>;
   GS_CUDA_TRY(cudaFuncSetAttribute(emit, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                    (int)emit_smem(1, kDirMaxTiles)));
   direct_count_kernel<<<cg, kDirThreads, smem_c, s>>>(a);
@@ -1016,7 +1031,7 @@ inline gs_status_t dir_bin_sort(const gs_proj_t *proj, const gs_frame_t *f, gs_b
   else
     direct_scan_kernel<32><<<(f->n_tiles + 31) / 32, kDirScanThreads, 0, s>>>(a, bins->d_count, d_error);
   GS_LAUNCH_CHECK();
-  emit<<<cg, kEmitThreads, smem_e, s>>>(a, bins->vals);
+  emit<<<cg, et, smem_e, s>>>(a, bins->vals);
   GS_LAUNCH_CHECK();
   if (bins->keys) {
     direct_keys_kernel<<<num_sms() * 8, 256, 0, s>>>(a.ranges, bins->vals, proj->depth, f->n_tiles, bins->keys);

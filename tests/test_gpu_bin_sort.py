@@ -304,3 +304,15 @@ def test_bin_sort_of_many_small_views(views):
             for w in (15 + v % 20 for v in range(views))]
     recs = _synthetic_records(40, 40, cams, (16, 16))
     assert _check(recs, cams, (16, 16)) > views
+
+
+@pytest.mark.parametrize("n,sizes", [
+    (3000, [(1000, 700)] * 2),                              # 11,000 tiles each: blocks of 512 threads
+    (60_000, [(700, 660)]),                                 # 7304 tiles: one word of mask, two blocks an SM
+    (9_900, [(1000, 700), (500, 350), (250, 175)]),         # unequal views, counted
+    (10_100, [(1000, 700), (500, 350), (250, 175)]),        # unequal views of more records: pairs
+    (700, [(840, 800)] * 7), (120_100, [(840, 800)] * 7)])  # 73,500 tiles in all: pairs; counted from 12 records a tile
+def test_bin_sort_on_both_sides_of_the_plans_lines(n, sizes):
+    cams = [synth.Camera(np.eye(3, dtype=np.float32), np.zeros(3, np.float32), 100., 100., w / 2, h / 2, w, h)
+            for w, h in sizes]
+    _check(_synthetic_records(50, n, cams, (8, 8)), cams, (8, 8))
