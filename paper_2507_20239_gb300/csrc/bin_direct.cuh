@@ -38,6 +38,9 @@ constexpr int kDirPasses = 4;                       // 8-bit digits of the depth
 constexpr int kDirMaxTiles = 20000;                 // per view: 10 1/8 bytes of shared memory each in the emission
 constexpr int kDirMaxViews = 1024;
 constexpr int64_t kDirMatrix = 1 << 24;             // entries of the (chunk, tile) matrix, at most
+constexpr int64_t kDirMostRecords = (1ll << 30) - 1;   // per view: the look-back words count in 30 bits
+// the lines of dir_plan's rule: see there
+constexpr int64_t kDirTilesFew = 65536, kDirTileRecords = 12, kDirUnequalRecords = 10000;
 constexpr uint32_t kDirSpins = 1u << 20;            // polls of a look-back word before the frame is given up
 
 // Device words shared by the kernels of a frame, zeroed before the first.
@@ -58,6 +61,7 @@ struct DirArgs {
   float inv_tw;
   uint64_t cap;           // list capacity (rows and hits)
   uint64_t unit_cap;      // units that the buffer holds (dir_unit_cap)
+  uint32_t stretch;       // units that a warp draws at a time (0: what each batch needs)
   int parts;              // sort partitions per view
   int chunks;             // chunks per view
   int n_tiles;
@@ -87,13 +91,20 @@ __device__ __forceinline__ bool dir_stopped(const DirArgs &a) {
 // ------------------------------------------------------------------ runs of tiles
 // A block takes a run of records view by view, its warps 32 records at a time in record order,
 // each with the next 32 records' inputs on their way; a warp's rows are spread over its
-// lanes (each finds its record by a search over the lanes' row prefix). Units come from a
-// stretch that the warp draws from the frame's counter when its last one is used up, so
-// that neither a barrier nor the counter is on a batch's path: with one draw and five
-// barriers per 256 records the kernel took 67 us at 1.5M records and 589 us at 20M, now 70 and
-// 560: issue (69% of the slots, the exact roundings' square roots and divisions) is what is left.
-constexpr uint32_t kDirStretch = 1024, kDirOwnDraw = 256;   // a batch of more units draws its own
+// lanes (each finds its record by a search over the lanes' row prefix). On frames of more than a
+// million records units come from a stretch of 1024 that the warp draws from the frame's counter when
+// its last one is used up, so that neither a barrier nor the counter is on a batch's path: with one draw
+// and five barriers per 256 records the kernel took 67 us at 1.5M records and 589 us at 20M, now 70
+// and 560: issue (69% of the slots, the exact roundings' square roots and divisions) is what is left.
+// With fewer records a batch draws what it needs: the stretches' rests would be most of the workspace (100k
+// records of 312 x 207 37.9 MB -> 12.2, 600k of 979 x 653 129 -> 65), for 0 to 3 us of the whole binning at 600k.
+constexpr uint32_t kDirStretch = 1024;
+constexpr int64_t kStretchRecords = 1 << 20;   // more of them: stretches
 constexpr int kUnitBlocks = 5;            // per SM
+
+inline uint32_t dir_stretch(int64_t R) { return R > kStretchRecords ? kDirStretch : 0u; }
+// The units up to which a batch draws on the warp's stretch; a batch of more draws its own.
+__host__ __device__ inline uint32_t own_draw(uint32_t stretch) { return stretch / 4; }
 
 __device__ __forceinline__ uint32_t dir_header(uint32_t rows, uint32_t tiles) {
   return rows << 16 | min(tiles, 0xffffu);   // rows <= 65535: rect is 16-bit
@@ -126,6 +137,7 @@ __global__ void __launch_bounds__(kDirThreads, kUnitBlocks) direct_units_kernel(
   const int64_t b0 = total * blockIdx.x / gridDim.x, b1 = total * (blockIdx.x + 1) / gridDim.x;
   uint64_t rows = 0, hits = 0;
   uint64_t at = 0, at_end = 0;   // the warp's stretch of units
+  const uint32_t own = own_draw(a.stretch);
   for (int64_t bv = b0; bv < b1;) {
     const int v = (int)(bv / per_view);
     const int64_t v0 = (int64_t)v * per_view, ve = min(b1, v0 + per_view);
@@ -199,17 +211,17 @@ __global__ void __launch_bounds__(kDirThreads, kUnitBlocks) direct_units_kernel(
       rows += n_units;
       const uint32_t need = n_units + n_vis;
       uint64_t from = at;
-      if (need > kDirOwnDraw || at + need > at_end) {
-        const uint32_t draw = need > kDirOwnDraw ? need : kDirStretch;
+      if (need > own || at + need > at_end) {
+        const uint32_t draw = need > own ? need : a.stretch;
         unsigned long long got = 0;
         if (lane == 0) got = atomicAdd(&a.words->alloc, (unsigned long long)draw);
         from = __shfl_sync(0xffffffffu, got, 0);
-        if (need <= kDirOwnDraw) {
+        if (need <= own) {
           at = from;
           at_end = from + draw;
         }
       }
-      if (need <= kDirOwnDraw) at += need;
+      if (need <= own) at += need;
       const bool keep = from + need <= a.unit_cap;   // else the row count ends the frame (dir_unit_cap)
       const uint32_t off = (uint32_t)from + rexcl + __popc(vm & lanemask_lt());
       if (vis && keep) {
@@ -864,16 +876,23 @@ __global__ void direct_keys_kernel(const uint2 *__restrict__ ranges, const uint3
 // ------------------------------------------------------------------ host side
 struct DirPlan {
   int chunks, parts, max_tiles, groups, unit_grid;
+  int most_chunks;        // of any frame like this one with fewer records too
   uint32_t share;
   bool ordered, ok;
 };
 
-// Units that the buffer holds: the lists' capacity in rows and a header per record, times 4/3
-// (a warp gives up at most kDirOwnDraw units of each stretch it draws), and its last
-// stretch. Frames whose rows fit the capacity fit this.
+// Units that the buffer holds: the lists' capacity in rows and a header per record, with stretches
+// times 4/3 (a warp gives up at most own_draw units of each one) and each warp's last. Frames
+// whose rows fit the capacity fit this.
 inline uint64_t dir_unit_cap(int64_t R, int64_t cap, int64_t unit_grid) {
-  static_assert(4 * kDirOwnDraw <= kDirStretch, "at least 3/4 of a stretch is used");
-  return ((uint64_t)cap + (uint64_t)R) * 4 / 3 + (uint64_t)unit_grid * kDirWarps * kDirStretch + 1;
+  const uint64_t used = (uint64_t)cap + (uint64_t)R, stretch = dir_stretch(R);
+  static_assert(kDirStretch % 4 == 0, "at least 3/4 of a stretch is used");
+  return (stretch ? used * 4 / 3 + (uint64_t)unit_grid * kDirWarps * stretch : used) + 1;
+}
+
+// Entries of the (chunk, tile) matrix, at most: in proportion to what is sorted, up to a bound.
+inline int64_t dir_matrix_cap(int64_t R, int64_t cap) {
+  return std::min<int64_t>(kDirMatrix, 4 * (R + cap) + (1 << 18));
 }
 
 // Whether a frame takes this path, and its chunks: eight blocks per SM in all,
@@ -899,15 +918,16 @@ inline DirPlan dir_plan(const gs_frame_t *f, int64_t R, int64_t cap) {
   const int64_t n = R / f->n_views;
   const int64_t gx = ((int64_t)f->max_width + f->tile_w - 1) / f->tile_w;
   const int64_t gy = ((int64_t)f->max_height + f->tile_h - 1) / f->tile_h;
-  if (gx * gy > kDirMaxTiles || gx * gy * f->n_views < f->n_tiles || n >= (1ll << 30)) return p;
-  if (f->n_tiles > 65536 && R < 12 * (int64_t)f->n_tiles) return p;
+  if (gx * gy > kDirMaxTiles || gx * gy * f->n_views < f->n_tiles || n > kDirMostRecords) return p;
+  if (f->n_tiles > kDirTilesFew && R < kDirTileRecords * f->n_tiles) return p;
   const bool large = gx * gy > 10000;
-  if (large && 4 * (int64_t)f->n_tiles < 3 * gx * gy * f->n_views && n >= 10000) return p;
+  if (large && 4 * (int64_t)f->n_tiles < 3 * gx * gy * f->n_views && n >= kDirUnequalRecords) return p;
   p.max_tiles = (int)(gx * gy);
   int64_t chunks = ((f->n_views > 1 ? 16ll : 8ll) * num_sms() + f->n_views - 1) / f->n_views;
-  const int64_t groups = (n + kDirThreads - 1) / kDirThreads, by_matrix = kDirMatrix / f->n_tiles;
+  const int64_t groups = (n + kDirThreads - 1) / kDirThreads, by_matrix = dir_matrix_cap(R, cap) / f->n_tiles;
   if (chunks > by_matrix) chunks = by_matrix;
   if (chunks < 1) return p;
+  p.most_chunks = (int)std::min<int64_t>(chunks, (n + 63) / 64);
   p.groups = (int)groups;
   p.ordered = chunks < groups;
   if (!p.ordered) {   // few records: equal shares of whole 64s, as many as fill the chunks
@@ -929,7 +949,8 @@ struct DirWs {
   size_t bytes;
 };
 
-// Workspace: the zeroed words first, then the buffers. n_tiles and views of the frame.
+// Workspace: the zeroed words first, then the buffers. n_tiles and views of the frame. Its size
+// does not fall with more records or a larger capacity (chunks of whole 64s make their number do so).
 inline DirWs dir_layout(void *base, int64_t R, int64_t cap, int64_t views, int64_t n_tiles, const DirPlan &plan) {
   DirWs w{};
   char *p = static_cast<char *>(base);
@@ -953,8 +974,8 @@ inline DirWs dir_layout(void *base, int64_t R, int64_t cap, int64_t views, int64
   w.a.v1 = (uint32_t *)take(4 * (size_t)R);
   w.a.ordered = plan.ordered ? reinterpret_cast<uint2 *>(w.a.k0) : nullptr;
   w.a.weights = (uint32_t *)take(4 * (size_t)views * plan.groups);
-  w.a.starts = (uint32_t *)take(4 * (size_t)views * (plan.chunks + 1));
-  w.a.matrix = (uint32_t *)take(4 * (size_t)plan.chunks * n_tiles);
+  w.a.starts = (uint32_t *)take(4 * (size_t)views * (plan.most_chunks + 1));
+  w.a.matrix = (uint32_t *)take(4 * (size_t)plan.most_chunks * n_tiles);
   w.a.totals = (uint32_t *)take(4 * (size_t)n_tiles);
   w.bytes = off;
   return w;
@@ -964,15 +985,16 @@ inline size_t dir_ws_size(const gs_frame_t *f, int64_t R, int64_t cap, const Dir
   return dir_layout(nullptr, R, cap, f->n_views, f->n_tiles, p).bytes;
 }
 
-// The most any frame on this path needs for R records: kDirMaxViews views' words, a
-// partition and a group more per view than the records fill, and the matrix at its bound.
+// The most any frame on this path needs for R records: as many views as there may be, a
+// partition, a group and two chunks more per view than the records fill, the matrix at its bound, and the
+// tiles at theirs.
 inline size_t dir_ws_bound(int64_t R, int64_t cap) {
   DirPlan p{};
-  p.chunks = 1;
+  const int64_t views = std::min<int64_t>(kDirMaxViews, std::max<int64_t>(R, 1));
   p.unit_grid = kUnitBlocks * num_sms();
-  const DirWs w = dir_layout(nullptr, R, cap, kDirMaxViews, kDirMatrix, p);
-  return w.bytes + 4 * (size_t)kDirPasses * 256 * ((size_t)R / kDirTile + kDirMaxViews + 1) +
-         4 * ((size_t)R / kDirThreads + 16 * (size_t)num_sms() + 4 * kDirMaxViews) + 1024;
+  const DirWs w = dir_layout(nullptr, R, cap, views, std::max<int64_t>(kDirTilesFew, R / kDirTileRecords), p);
+  return w.bytes + 4 * (size_t)dir_matrix_cap(R, cap) + 4 * (size_t)kDirPasses * 256 * ((size_t)R / kDirTile + views + 1) +
+         4 * ((size_t)R / kDirThreads + 16 * (size_t)num_sms() + 4 * views) + 1024;
 }
 
 inline gs_status_t dir_bin_sort(const gs_proj_t *proj, const gs_frame_t *f, gs_bins_t *bins, void *ws, size_t ws_bytes,
@@ -990,6 +1012,7 @@ inline gs_status_t dir_bin_sort(const gs_proj_t *proj, const gs_frame_t *f, gs_b
   a.inv_tw = 1.f / (float)f->tile_w;
   a.cap = (uint64_t)bins->capacity;
   a.unit_cap = dir_unit_cap(R, bins->capacity, plan.unit_grid);
+  a.stretch = dir_stretch(R);
   a.groups = plan.groups;
   a.share = plan.share;
   a.parts = plan.parts;

@@ -929,10 +929,21 @@ extern "C" size_t gs_bin_sort_workspace_size(int64_t n_records, int64_t dup_capa
   if (n_records < 0 || dup_capacity < 0) return 0;
   int tile_bits = 32, fbits = kMaxFusedBits;
   if (frame && !frame_sort_plan(frame, tile_bits, fbits)) return 0;
-  const size_t pairs = bin_ws_layout(nullptr, n_records, dup_capacity, fbits).bytes;
-  if (!frame) return std::max(pairs, dir_ws_bound(n_records, dup_capacity));
-  const DirPlan plan = dir_plan(frame, n_records, dup_capacity);
-  return plan.ok ? dir_ws_size(frame, n_records, dup_capacity, plan) : pairs;
+  const auto pairs = [&](int64_t n) { return bin_ws_layout(nullptr, n, dup_capacity, fbits).bytes; };
+  if (!frame) return std::max(pairs(n_records), dir_ws_bound(n_records, dup_capacity));
+  // what this many records need, and no less than fewer do on the other path: at the lines between the two
+  const auto need = [&](int64_t n) {
+    const DirPlan plan = dir_plan(frame, n, dup_capacity);
+    return plan.ok ? dir_ws_size(frame, n, dup_capacity, plan) : pairs(n);
+  };
+  size_t bytes = need(n_records);
+  if (frame->n_views > 0)
+    for (const int64_t line : {kDirTileRecords * frame->n_tiles - 1, kDirUnequalRecords * frame->n_views - 1,
+                               kDirMostRecords * frame->n_views}) {
+      const int64_t n = line - line % frame->n_views;
+      if (n > 0 && n < n_records) bytes = std::max(bytes, need(n));
+    }
+  return bytes;
 }
 
 extern "C" gs_status_t gs_bin_sort(const gs_proj_t *proj, const gs_frame_t *frame, gs_bins_t *bins, void *ws,
@@ -947,6 +958,11 @@ extern "C" gs_status_t gs_bin_sort(const gs_proj_t *proj, const gs_frame_t *fram
   int tile_bits, fbits;
   if (!frame_sort_plan(frame, tile_bits, fbits)) return GS_ERR_INVALID_ARG;
   cudaStream_t s = as_stream(stream);
+  if (R == 0) {   // no lists, and no workspace needed: one sized for more records need not hold the general path's
+    GS_CUDA_TRY(cudaMemsetAsync(bins->ranges, 0, 8 * (size_t)frame->n_tiles, s));
+    GS_CUDA_TRY(cudaMemsetAsync(bins->d_count, 0, sizeof(int64_t), s));
+    return GS_OK;
+  }
   const DirPlan plan = dir_plan(frame, R, bins->capacity);
   if (plan.ok) return dir_bin_sort(proj, frame, bins, ws, ws_bytes, plan, d_error, s);
   const BinWs w = bin_ws_layout(ws, R, bins->capacity, fbits);

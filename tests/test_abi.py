@@ -215,3 +215,43 @@ assert all(s > 4 * 1000 for s in sizes), sizes
     r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True,
                        cwd=os.path.dirname(os.path.dirname(HEADER)))
     assert r.returncode == 0, (r.returncode, r.stderr)
+
+
+def _frame(lib, sizes, tile):
+    cams = (_abi.GsCamera * len(sizes))()
+    for c, (w, h) in zip(cams, sizes):
+        c.fx = c.fy = 100.0
+        c.width, c.height, c.near_plane = w, h, 0.2
+    fr = _abi.GsFrame()
+    assert lib.gs_frame_init(cams, len(sizes), tile, tile, C.byref(fr)) == 0
+    return fr
+
+
+@pytest.mark.parametrize("sizes,tile", [
+    ([(64, 64)], 16), ([(1246, 826)], 16), ([(1246, 826)], 8), ([(1700, 1300)], 8),
+    ([(1246, 826), (623, 413), (312, 207)], 16), ([(1246, 826), (623, 413), (312, 207)], 8),   # the latter: two paths
+    ([(700, 640)] * 10, 8), ([(40, 30)] * 1030, 8)])                                            # again two, and one
+def test_bin_sort_workspace_grows_with_records_and_capacity(lib, sizes, tile):
+    """A workspace sized for more records, or a larger capacity, on the same frame holds fewer: over the
+    edges of chunks, partitions and batches and the lines between the paths."""
+    fr, v = _frame(lib, sizes, tile), len(sizes)
+    edges = [1, 31, 63, 64, 65, 127, 128, 129, 255, 2047, 2048, 2049, 4095, 4096, 9999, 10000, 75_776, 75_777, 77_824,
+             77_825, 151_552, 151_553, 155_649, 311_296, 311_297, (1 << 20) // v, (1 << 20) // v + 1, 3_000_000,
+             12 * fr.n_tiles // v, 12 * fr.n_tiles // v + 1, (1 << 30) - 1, 1 << 30]
+    counts = sorted(n * v for n in set(edges) if n * v < 1 << 31)
+    for cap in (0, 1000, 1_000_000, 100_000_000):
+        got = [lib.gs_bin_sort_workspace_size(n, cap, C.byref(fr)) for n in counts]
+        assert all(0 < a <= b for a, b in zip(got, got[1:])), (cap, list(zip(counts, got)))
+    for n in counts:
+        got = [lib.gs_bin_sort_workspace_size(n, cap, C.byref(fr)) for cap in (0, 1, 999, 65_536, 800_000, 1 << 24, 1 << 30)]
+        assert all(0 < a <= b for a, b in zip(got, got[1:])), (n, got)
+
+
+@pytest.mark.parametrize("n,size,most_mb", [(2000, (64, 64), 2.0), (37_777, (417, 305), 6.0), (100_000, (312, 207), 13.0),
+                                            (300_000, (623, 413), 38.1), (600_000, (979, 653), 72.0)])
+def test_bin_sort_workspace_of_small_frames(lib, n, size, most_mb):
+    """At the binding's first capacity, against 12 bytes of each entry and 20 of each record, which the
+    general path's buffers hold (and a little of both paths' tables)."""
+    cap = max(1 << 16, 8 * n)
+    assert lib.gs_bin_sort_workspace_size(n, cap, C.byref(_frame(lib, [size], 16))) <= most_mb * 1e6
+    assert lib.gs_bin_sort_workspace_size(2000, 1 << 16, None) < 16e6

@@ -316,3 +316,26 @@ def test_bin_sort_on_both_sides_of_the_plans_lines(n, sizes):
     cams = [synth.Camera(np.eye(3, dtype=np.float32), np.zeros(3, np.float32), 100., 100., w / 2, h / 2, w, h)
             for w, h in sizes]
     _check(_synthetic_records(50, n, cams, (8, 8)), cams, (8, 8))
+
+
+@pytest.mark.parametrize("sizes,tile,counts", [
+    ([(1246, 826)], (16, 16), [75_777, 75_776, 40_000, 1, 0]),
+    ([(1000, 700), (500, 350)], (8, 8), [10_001, 10_000, 9_999, 300, 0]),   # pairs, then counted
+    ([(1700, 1300)], (8, 8), [3000, 1, 0])])
+def test_bins_sized_for_more_records_hold_fewer(sizes, tile, counts):
+    cams = [synth.Camera(np.eye(3, dtype=np.float32), np.zeros(3, np.float32), 100., 100., w / 2, h / 2, w, h)
+            for w, h in sizes]
+    frame = R.Frame(cams, tile=tile)
+    bins = R.alloc_bins(frame, counts[0] * len(cams), capacity=1_500_000)
+    for n in counts:
+        recs = _synthetic_records(60, n, cams, tile)
+        proj = records_to_gpu(recs)
+        R.bin_sort_into(proj, frame, bins)
+        assert int(bins.error.item()) == 0
+        M, ranges = int(bins.count.item()), bins.ranges.cpu().numpy().view(np.uint32)
+        if n == 0:
+            assert M == 0 and not ranges.any()
+            continue
+        _, vals, want = _oracle_bins(recs, frame)
+        assert M == len(vals) and np.array_equal(ranges, want)
+        assert np.array_equal(bins.vals[:M].cpu().numpy().view(np.uint32), vals)
