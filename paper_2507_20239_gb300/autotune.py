@@ -2,7 +2,8 @@
 
 For a given scene size and set of view resolutions it times the whole step
 (TrainStep, graph-replayed) for every candidate StepConfig -- tile shape, the
-low tile-id bits the binning sorts while emitting, the backward's staging
+low tile-id bits the binning sorts while emitting (where they change its work: else the
+candidate is another one over again and is left out), the backward's staging
 depth, the per-pixel or per-splat backward, and the forward as one CTA per tile or
 as a persistent grid claiming (tile, block) units -- and keeps the fastest. None of the knobs changes the rendered images
 (every candidate's images are compared with the first one's); the gradients agree
@@ -11,8 +12,9 @@ sizes, candidates) for the life of the process.
 """
 from __future__ import annotations
 
+import ctypes as C
 import itertools
-from dataclasses import dataclass, field
+from dataclasses import dataclass, field, replace
 from typing import Callable, Optional, Sequence
 
 import torch
@@ -80,6 +82,28 @@ def _fits(cfg: StepConfig, cameras) -> bool:
     return cfg.sort_fused_bits == 0 or cfg.sort_fused_bits <= bits
 
 
+def _same_binning(cfg: StepConfig, cameras, n: int) -> bool:
+    """Whether cfg's fused bits leave the binning as the library's own choice has it: frames whose lists
+    are counted have no use for them, and on the others they may be that choice. The workspace tells:
+    its size depends on them where the work does."""
+    arr = (_abi.GsCamera * len(cameras))()
+    for c, cam in zip(arr, cameras):
+        c.width, c.height, c.fx, c.fy, c.near_plane = int(cam.width), int(cam.height), 1.0, 1.0, 0.2
+    frame, sizes = _abi.GsFrame(), []
+    _abi.check(lib().gs_frame_init(arr, len(cameras), int(cfg.tile[0]), int(cfg.tile[1]), C.byref(frame)),
+               "gs_frame_init")
+    for bits in (0, cfg.sort_fused_bits):
+        frame.sort_fused_bits = bits
+        sizes.append(lib().gs_bin_sort_workspace_size(n * len(cameras), 0, C.byref(frame)))
+    return sizes[0] == sizes[1]
+
+
+def _repeats(cfg: StepConfig, candidates: Sequence[StepConfig], cameras, n: int) -> bool:
+    """Whether cfg is another candidate, the same but for the fused bits, over again."""
+    plain = replace(cfg, sort_fused_bits=0)
+    return cfg != plain and plain in candidates and _same_binning(cfg, cameras, n)
+
+
 _cache: dict = {}
 
 
@@ -112,7 +136,7 @@ def autotune(params: dict, sh_degree: int, cameras, target_images, candidates: S
     identical = [True]
 
     def measure(cfg: StepConfig):
-        if not _fits(cfg, cameras):
+        if not _fits(cfg, cameras) or _repeats(cfg, candidates, cameras, int(params["means"].shape[0])):
             return None
         step = TrainStep(params, sh_degree, cameras, target_images, cfg, device=device)
         ms = time_step(step, reps=reps)

@@ -60,3 +60,22 @@ def test_step_config_backward_is_validated():
     assert StepConfig((16, 16), 0, 0, "splat", True).label() == "16x16/f0/splat/queue"
     with pytest.raises(ValueError):
         StepConfig(backward="tile")
+
+
+class _View:
+    def __init__(self, width, height):
+        self.width, self.height = width, height
+
+
+@pytest.mark.parametrize("size,tile,bits,same", [
+    ((64, 48), (16, 16), 4, True), ((1246, 826), (16, 16), 8, True), ((1246, 826), (8, 8), 8, True),   # counted
+    ((1700, 1300), (8, 8), 8, True),         # sorted by tile id: 16 bits, of which 8 are the library's choice
+    ((1700, 1300), (8, 8), 3, False), ((2600, 2600), (8, 8), 8, False)])
+def test_fused_bits_that_change_nothing_are_not_timed_again(size, tile, bits, same):
+    views, cfg = [_View(*size)], StepConfig(tile, bits)
+    assert at._same_binning(cfg, views, 100_000) == same
+    both = [StepConfig(tile), cfg]
+    assert at._repeats(cfg, both, views, 100_000) == same
+    assert not at._repeats(cfg, [cfg], views, 100_000)           # nothing else stands for it
+    assert not at._repeats(both[0], both, views, 100_000)
+    assert not at._repeats(cfg, [StepConfig(tile, 0, 1), cfg], views, 100_000)
