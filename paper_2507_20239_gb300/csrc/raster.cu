@@ -834,7 +834,8 @@ __device__ __forceinline__ void splat_walk(const SplatEntries &e, int nl, float4
       // without an entry) where sigma reaches the floor; elsewhere sigma 0 leaves T,
       // R and every sum as they are
       const uint32_t stop = __float_as_uint(g.w);
-      const bool oka = e.ja < stop && raw.x >= kAlphaMin, okb = e.jb < stop && raw.y >= kAlphaMin;
+      // (the forward's test on min(0.99, sigma), in which a sigma that is no number counts as 0.99)
+      const bool oka = e.ja < stop && !(raw.x < kAlphaMin), okb = e.jb < stop && !(raw.y < kAlphaMin);
       // -<c, g>, in scalar form: the pixel's three words as broadcast operands of packed products
       // took register moves (534 against 558 us on a 1.5M-Gaussian 1246 x 826 view)
       const float2 ncd = f2(fmaf(e.NCZ.x, g.z, fmaf(e.NCY.x, g.y, e.NCX.x * g.x)),

@@ -231,3 +231,40 @@ def test_tile_backward_matches_per_pixel_backward(n, size, tile, zoom, depth, us
             print(f"lists of {lens.min()} to {lens.max()} entries, {(lens <= 32).mean():.2f} of them up to 32")
     for k, b in got["pixel"].items():
         assert np.linalg.norm(b) > 0 and rel_l2(got["tile"][k], b) < 1e-4, k
+
+
+@pytest.mark.parametrize("bad", [np.nan, np.inf])
+@pytest.mark.parametrize("backward", ["tile", "tile, cut-off recomputed", "splat"])
+def test_backwards_agree_on_records_that_are_no_numbers(backward, bad):
+    """An opacity that is NaN or infinite counts as 0.99 in the forward (min(0.99, sigma)), and so for the
+    transmittance of what lies behind it (here a record over every block of the view, in the middle of
+    the scene): the other records' gradients against raster_bwd_kernel's (a large second view beside the
+    small one), tolerance as above."""
+    n, w, h = 2500, 120, 90
+    sc = synth.small_scene(3, n=n, width=w, height=h)
+    cam = sc.cameras[0]
+    big = synth.Camera(cam.R, cam.t, 1000., 1000., 640., 480., 1280, 960)
+    P = R.to_device_params(sc.params())
+    rest = torch.arange(n, device="cuda") != 5
+    got = {}
+    for name, cams in ((backward, [cam]), ("pixel", [cam, big])):
+        frame = R.Frame(cams)
+        proj = R.project(P, 0, frame)
+        proj.mean2d[5] = torch.tensor([60.0, 45.0])
+        proj.conic_opacity[5] = torch.tensor([1e-5, 0.0, 1e-5, float(bad)])
+        proj.rgb[5] = torch.tensor([0.2, 0.9, 0.5, 9.0])
+        proj.depth[5], proj.radius[5] = 4.0, 900
+        proj.rect[5] = torch.tensor([0, 0, 8, 6], dtype=torch.int16)
+        bins = R.bin_sort(proj, frame)
+        ckpt = R.alloc_ckpt(frame, bins)
+        img, _, stop = R.raster_fwd_ckpt(proj, bins, frame, ckpt)
+        d_image = torch.zeros_like(img)
+        d_image[:3 * w * h] = torch.randn(3 * w * h, generator=torch.Generator("cuda").manual_seed(1), device="cuda")
+        if name == "splat":
+            rg = R.raster_bwd_splat(proj, bins, frame, img, d_image, stop, ckpt)
+        else:
+            rg = R.raster_bwd(proj, bins, frame, img, d_image, stop=None if "recomputed" in name else stop)
+        got[name] = {k: getattr(rg, k)[:n][rest].cpu().numpy() for k in ("d_mean2d", "d_conic_opacity", "d_rgb")}
+        assert torch.isfinite(img).all()
+    for k, b in got["pixel"].items():
+        assert np.linalg.norm(b) > 0 and rel_l2(got[backward][k], b) < 1e-4, k
