@@ -74,8 +74,9 @@ typedef struct {
   int32_t sort_fused_bits; /* gs_bin_sort: low tile-id bits sorted while emitting
                             * (1..8, at most the tile-id width); 0 = automatic.
                             * A tuning knob: the order produced is the same. It
-                            * has an effect only on views of more than 20000
-                            * tiles, whose entries are sorted by tile id.     */
+                            * has an effect only on frames whose entries are
+                            * sorted by tile id: views of more than 20000 tiles,
+                            * many tiles for few records, some unequal views.  */
 } gs_frame_t;
 
 /* Gaussian parameters, device SoA (Eq. 1: position, scale, rotation, opacity, SH):
@@ -181,8 +182,8 @@ gs_status_t gs_frame_init(gs_camera_t *cams_host, int32_t n_views, int32_t tile_
                           int32_t tile_h, gs_frame_t *frame);
 
 /* Bytes of scratch gs_bin_sort needs for n_records records and dup_capacity
- * duplicates on this frame (NULL frame: the most any frame needs); 0 for an
- * invalid size or sort_fused_bits. */
+ * duplicates on this frame, and for any fewer of either (NULL frame: the most any
+ * frame needs); 0 for an invalid size or sort_fused_bits. */
 size_t gs_bin_sort_workspace_size(int64_t n_records, int64_t dup_capacity, const gs_frame_t *frame);
 
 /* ---------------------------------------------------------------------- hot path */
@@ -241,8 +242,8 @@ gs_status_t gs_l1_loss_grad(const gs_frame_t *frame, const float *image, const f
  * with NULL the stop position is recomputed from the transmittance cut-off. Uses
  * dL/dsigma_i = T_i <c_i, g> - (<out, g> - sum_{j<=i} <c_j, g> sigma_j T_j) / (1 - sigma_i),
  * out being the forward's image; zero through the 0.99 clamp. Per-pixel terms are
- * summed per Gaussian in registers, across the warp and the CTA (on frames of few
- * tiles by the walk of gs_raster_bwd_splat, from states kept in shared memory), then
+ * summed per Gaussian in registers, across the warp and the CTA (on smaller frames the
+ * longer lists by the walk of gs_raster_bwd_splat, from states kept in shared memory), then
  * added once per (tile or part of a tile, record) into grads (see gs_rec_grads_t). */
 gs_status_t gs_raster_bwd(const gs_proj_t *proj, const gs_bins_t *bins, const gs_frame_t *frame,
                           const gs_raster_cfg_t *cfg, const float *image, const float *d_image,

@@ -12,8 +12,8 @@
 //   direct_scan_kernel   per tile: exclusive scan over the chunks; ranges, M, capacity check
 //   direct_emit_kernel   each chunk's record ids to the lists
 //
-// Compared with emitting (tile, record) pairs into partial order and sorting them (the path
-// for views of more tiles than shared memory has counters for), a hit moves 4 bytes once
+// Compared with emitting (tile, record) pairs into partial order and sorting them (the general
+// path, for the frames that dir_plan refuses), a hit moves 4 bytes once
 // instead of 8 bytes out, 8 in and 8 out again, the gathers in depth order touch one place per
 // record (its header and runs) instead of four, no two warps claim work from one
 // counter, and a frame takes 9 or 10 launches instead of 21. gs_bin_sort, that path -> this one,
@@ -97,7 +97,7 @@ __device__ __forceinline__ bool dir_stopped(const DirArgs &a) {
 // and five barriers per 256 records the kernel took 67 us at 1.5M records and 589 us at 20M, now 70
 // and 560: issue (69% of the slots, the exact roundings' square roots and divisions) is what is left.
 // With fewer records a batch draws what it needs: the stretches' rests would be most of the workspace (100k
-// records of 312 x 207 37.9 MB -> 12.2, 600k of 979 x 653 129 -> 65), for 0 to 3 us of the whole binning at 600k.
+// records of 312 x 207 37.9 MB -> 10.2, 600k of 979 x 653 129 -> 66), for 0 to 3 us of the whole binning at 600k.
 constexpr uint32_t kDirStretch = 1024;
 constexpr int64_t kStretchRecords = 1 << 20;   // more of them: stretches
 constexpr int kUnitBlocks = 5;            // per SM

@@ -8,9 +8,9 @@
 // per tile row, the ellipse's x-extent over the row's pixel centres keeps a
 // contiguous run of columns (the exact ellipse-box test, band_span_rn).
 //
-// Two paths give that order. Views whose tiles fit the shared-memory tables of
-// bin_direct.cuh (up to 20000, all but very large views or small tiles) have their entries
-// counted and written straight to their places. The others go the way of this file:
+// Two paths give that order. Frames whose views fit the shared-memory tables of
+// bin_direct.cuh (up to 20000 tiles) and have records enough for their tiles (dir_plan) have their
+// entries counted and written straight to their places. The others go the way of this file:
 //
 // Instead of one wide radix sort on (tile << 32 | depth) keys over all duplicates,
 // the order is built in two stable stages that give the same permutation:

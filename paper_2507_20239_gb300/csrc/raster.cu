@@ -716,7 +716,7 @@ __global__ void __launch_bounds__(TW *TH / PX) raster_bwd_kernel(
 
 // Per-splat backward (the per-splat parallel back-propagation of the Taming-3DGS
 // lineage that the paper's base trainer uses): the same gradient as
-// raster_bwd_tile_kernel, parallel over list entries instead of pixels. The warps of a
+// raster_bwd_kernel, parallel over list entries instead of pixels. The warps of a
 // tile's CTAs claim its 64-entry buckets (up to the tile's largest stop index) one
 // at a time, two consecutive entries per lane. A bucket's live pixels (stop index
 // beyond its first position) start from the forward's checkpoint (T and the colour
