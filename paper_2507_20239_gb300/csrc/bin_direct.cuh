@@ -95,7 +95,8 @@ __device__ __forceinline__ bool dir_stopped(const DirArgs &a) {
 // million records units come from a stretch of 1024 that the warp draws from the frame's counter when
 // its last one is used up, so that neither a barrier nor the counter is on a batch's path: with one draw
 // and five barriers per 256 records the kernel took 67 us at 1.5M records and 589 us at 20M, now 70
-// and 560: issue (69% of the slots, the exact roundings' square roots and divisions) is what is left.
+// and 560: issue (58% of the slots at 600k records, the exact roundings' square roots and divisions) is
+// what is left.
 // With fewer records a batch draws what it needs: the stretches' rests would be most of the workspace (100k
 // records of 312 x 207 37.9 MB -> 10.2, 600k of 979 x 653 129 -> 66), for 0 to 3 us of the whole binning at 600k.
 constexpr uint32_t kDirStretch = 1024;
@@ -696,8 +697,8 @@ __global__ void __launch_bounds__(kDirScanThreads) direct_scan_kernel(const DirA
 // the records of the set bits in order: the threads set the bits of their units (a record's run
 // of tiles in one tile row) and note the tiles that had none yet; then each noted tile's
 // thread writes its records after the tile's cursor and clears the mask. Two barriers a group.
-// Bound by the latency of a group's shared-memory steps (37% of issue slots, stalls on barriers
-// and shared memory). At 1.5M records / 20M in 4 views: this form 203 / 1690 us; every hit ranked by
+// Bound by the latency of a group's shared-memory steps (34% of issue slots at 600k records, stalls on
+// barriers and shared memory). At 1.5M records / 20M in 4 views: this form 203 / 1690 us; every hit ranked by
 // a population count of the bits below it, with a third barrier for the cursors, 210 / 1967,
 // and with the hits spread evenly over the lanes first, 242 / 1849; groups of 32, 64 or 128
 // records, 256 or 512 threads 203 to 216 / 1650 to 2130; a warp writing a tile's entries together
